@@ -378,6 +378,7 @@ kmpar_status kmpar_weight(kmpar_ctx *ctx, int64_t *m_out, const int32_t **cand_i
     kmpar_status ts = check_timeout(c);
     if (ts != KMPAR_OK) return ts;
     c.weighted = true;
+    c.m_host = st.m;
     if (m_out) *m_out = st.m;
     if (cand_idx_dev) *cand_idx_dev = c.cand;
     if (w_dev) *w_dev = reinterpret_cast<const int64_t *>(c.w);
@@ -389,11 +390,29 @@ kmpar_status kmpar_recluster(kmpar_ctx *ctx, float *centers_dev) {
     kmp::Ctx &c = ctx->c;
     if (!centers_dev) return fail(&c, KMPAR_ERR_ARG, "centers_dev is NULL");
     if (!c.weighted) return fail(&c, KMPAR_ERR_STATE, "recluster before weight");
-    if (!c.rCT) {
-        // the grid form and the batched form read the candidates transposed
-        const size_t nf = c.rs_batch > 0 ? (size_t)((c.cap_total + 31) / 32) * 32 * (c.d + 2)
-                                         : kmp::recluster_grid_floats(c);
-        if (nf) KMP_CUDA(&c, alloc(c, &c.rCT, nf), "alloc transposed candidates");
+    // the form of the draws: in batches (kmpar_set_recluster), else one at a time in a
+    // thread-block cluster, or in a cooperative grid (KMPAR_RECLUSTER_GRID=1 selects
+    // the latter for every size)
+    kmp::ReclusterPlan plan;
+    if (c.rs_batch == 0) {
+        const char *grid = getenv("KMPAR_RECLUSTER_GRID");
+        int max_cs = 0;
+        KMP_CUDA(&c, kmp::recluster_max_cluster(c.dev, &max_cs), "cluster size");
+        if (!(grid && grid[0] == '1')) plan = kmp::recluster_plan(c.m_host, c.d, max_cs);
+    }
+    // their transposed copy of the candidates: the grid and batched forms need it, the
+    // cluster form reads row-major candidates where it cannot be had
+    const int d4 = (c.d + 3) / 4;
+    const size_t nf = plan.cs > 0 ? (plan.qs4 < d4 ? (size_t)plan.slots * d4 * 4 : 0)
+                                  : (size_t)((c.cap_total + 31) / 32) * 32 * (c.d + 2);
+    if (nf > c.rCT_floats) {
+        if (c.rCT) cudaFreeAsync(c.rCT, c.stream);
+        c.alloc_bytes -= (sizeof(float) * c.rCT_floats + 255) & ~(size_t)255;
+        c.rCT_floats = 0;
+        const cudaError_t e = alloc(c, &c.rCT, nf);
+        if (e == cudaSuccess) c.rCT_floats = nf;
+        else if (plan.cs == 0) return cuda_fail(&c, e, "alloc transposed candidates");
+        else cudaGetLastError();
     }
     if (c.rs_batch > 0 && !c.rs_buf) {
         unsigned char *b = nullptr;
@@ -404,8 +423,11 @@ kmpar_status kmpar_recluster(kmpar_ctx *ctx, float *centers_dev) {
     KMP_CUDA(&c, cudaMemsetAsync(c.rc_err, 0, sizeof(int), c.stream), "memset recluster error");
     if (c.rs_batch > 0)
         KMP_CUDA(&c, kmp::launch_recluster_batch(c, centers_dev), "batched recluster");
+    else if (plan.cs > 0)
+        KMP_CUDA(&c, kmp::launch_recluster_draws(c, centers_dev, plan, c.rCT_floats >= nf ? c.rCT : nullptr),
+                 "recluster kernel");
     else
-        KMP_CUDA(&c, kmp::launch_recluster(c, centers_dev), "recluster kernel");
+        KMP_CUDA(&c, kmp::launch_recluster_grid(c, centers_dev), "recluster kernel");
     int32_t warn = 0, rerr = 0;
     KMP_CUDA(&c, cudaMemcpyAsync(&warn, &c.st->warn, sizeof(warn), cudaMemcpyDeviceToHost, c.stream), "read warn");
     KMP_CUDA(&c, cudaMemcpyAsync(&rerr, c.rc_err, sizeof(rerr), cudaMemcpyDeviceToHost, c.stream), "read error");

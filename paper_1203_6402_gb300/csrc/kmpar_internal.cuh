@@ -68,7 +68,9 @@ struct Ctx {
     long long *w = nullptr;       // cap_total
     float *rD2 = nullptr;         // recluster D^2, 2 x cap_total rounded up to 32
     double *rc_cmass = nullptr;   // recluster chunk masses, 2 x ceil(cap_total / 32), then 2048 doubles of CTA slots
-    float *rCT = nullptr;         // recluster grid form: candidates transposed (d x cap_total padded to 32)
+    float *rCT = nullptr;         // reclustering: transposed candidates (each form its own layout)
+    size_t rCT_floats = 0;
+    int m_host = 0;               // candidates, as kmpar_weight read them
     int32_t *wl_lab[2] = {nullptr, nullptr};   // weighted Lloyd: candidate labels (cap_total each)
     int rs_batch = 0;             // reclustering: 0 = one draw at a time, B = up to B draws per D^2 snapshot
     void *rs_buf = nullptr;       // batched reclustering: control word, proposals, their pair distances
@@ -244,7 +246,15 @@ cudaError_t launch_round(Ctx &c, int round);
 cudaError_t launch_round_distance(Ctx &c, int round);
 cudaError_t launch_phi_finalize(Ctx &c, int nparts, double *out, double *hist_slot);
 cudaError_t launch_weights(Ctx &c);
-cudaError_t launch_recluster(Ctx &c, float *centers);
+// step 8 one draw at a time: the cluster form (recluster_cluster.cu) by a plan of
+// its own, cs = 0 when it does not apply, and the cooperative grid form
+struct ReclusterPlan {
+    int cs = 0, cpw = 0, qs4 = 0, slots = 0;
+};
+ReclusterPlan recluster_plan(int m, int d, int max_cs);
+cudaError_t recluster_max_cluster(int dev, int *max_cs);
+cudaError_t launch_recluster_draws(Ctx &c, float *centers, const ReclusterPlan &p, float *CT4);
+cudaError_t launch_recluster_grid(Ctx &c, float *centers);
 // batched reclustering (recluster_batch.cu): up to kRsMaxBatch draws per D^2 snapshot
 constexpr int kRsMaxBatch = 64;
 constexpr int kRsMaxProposals = 2 * kRsMaxBatch;
@@ -252,7 +262,6 @@ size_t recluster_batch_bytes();
 cudaError_t launch_recluster_batch(Ctx &c, float *centers);
 cudaError_t launch_transpose_cand(Ctx &c);   // candidates -> c.rCT (d x cap_total padded to 32)
 size_t recluster_sync_bytes();
-size_t recluster_grid_floats(const Ctx &c);   // floats of the transposed copy the grid form needs (0: none)
 cudaError_t launch_weighted_centroids(const Ctx &c, int m, const int32_t *lab, float *centers);
 cudaError_t launch_assign(const float *X, int64_t n, int d, const float *C, int k, int32_t *labels,
                           const int32_t *prev, int *changed, double *partials, int nparts,
