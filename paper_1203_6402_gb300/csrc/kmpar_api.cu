@@ -128,7 +128,8 @@ void free_ctx(kmp::Ctx &c) {
                     c.tc_anchor, c.tc_anchor_part, c.lloyd_rec, c.ex_keys, c.ex_ws, c.ex_ties,
                     c.tc_ncol, c.tc_tscale, c.tc_xscale, c.tc_ub, c.tc_cimg, c.tc_cscale, c.tc_thr,
                     c.tc_lst, c.tc_lcnt, c.fix_rows2, c.fix_cnt2, c.rCT, c.wl_lab[0], c.wl_lab[1], c.rs_buf,
-                    c.ll_ub, c.ll_lb, c.ll_rows, c.ll_cnt, c.ll_cold, c.ll_drift, c.ll_other};
+                    c.ll_ub, c.ll_lb, c.ll_rows, c.ll_cnt, c.ll_cold, c.ll_drift, c.ll_other, c.rf_rad2, c.rf_num, c.rf_lst, c.rf_head,
+                    c.rf_lcnt, c.rf_rows, c.rf_cnt};
     // stream-ordered: the memory returns to the pool once the context's work is done
     for (void *b : bufs)
         if (b) cudaFreeAsync(b, c.stream);
@@ -297,6 +298,15 @@ kmpar_status kmpar_init(kmpar_ctx **out, const float *X, int64_t n, int32_t d, i
             KMP_INIT_CUDA(alloc(c, &c.tc_lcnt, (size_t)n * 4), "alloc list counts");
             KMP_INIT_CUDA(alloc(c, &c.fix_rows2, n), "alloc exact-scan rows");
             KMP_INIT_CUDA(alloc(c, &c.fix_cnt2, 1), "alloc exact-scan count");
+            if (kmp::round_filter_sizes(c)) {
+                KMP_INIT_CUDA(alloc(c, &c.rf_rad2, 2 * (size_t)c.cap_total), "alloc candidate radii");
+                KMP_INIT_CUDA(alloc(c, &c.rf_num, 2 * (size_t)c.cap_total), "alloc candidate numbers");
+                KMP_INIT_CUDA(alloc(c, &c.rf_lst, (size_t)c.cap_total * 4 * tc::kListSlots), "alloc candidate lists");
+                KMP_INIT_CUDA(alloc(c, &c.rf_head, c.cap_total), "alloc candidate list heads");
+                KMP_INIT_CUDA(alloc(c, &c.rf_lcnt, tc::kListLevels), "alloc candidate list counts");
+                KMP_INIT_CUDA(alloc(c, &c.rf_rows, n), "alloc open rows");
+                KMP_INIT_CUDA(alloc(c, &c.rf_cnt, 1), "alloc open row count");
+            }
         }
         KMP_INIT_CUDA(alloc(c, &c.tc_anchor, d), "alloc anchor");
         KMP_INIT_CUDA(alloc(c, &c.tc_anchor_part, tc::tc_anchor_scratch_doubles(d)), "alloc anchor sums");

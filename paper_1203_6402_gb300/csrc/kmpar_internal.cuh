@@ -39,6 +39,8 @@ struct DevState {
     unsigned long long screen_exact;                   // rows that needed the exact scan
     unsigned long long screen_listed;                  // undecided round rows refined from the pass's own lists
     unsigned long long recluster_snapshots;            // batched reclustering: D^2 snapshots taken
+    int32_t part_begin, part_total, part_next;         // the round's batch while its parts are passed over
+    int32_t part_open;                                 // rows the filter left open in the last pass (-1: none yet)
     unsigned long long lloyd_settled;                  // Lloyd rows whose assignment the bounds settled
 };
 
@@ -127,6 +129,15 @@ struct Ctx {
     int32_t *tc_lcnt = nullptr;   // list pass: entries per row and column group
     int32_t *fix_rows2 = nullptr; // rows left to the exact scan after the list pass
     int *fix_cnt2 = nullptr;
+    // round filter: per candidate the bits of the largest D^2 among its rows and a list of
+    // new candidates around it; the rows it leaves open, and their number
+    unsigned int *rf_rad2 = nullptr;
+    int32_t *rf_num = nullptr, *rf_lst = nullptr;
+    int2 *rf_head = nullptr;
+    int *rf_lcnt = nullptr;
+    int32_t *rf_rows = nullptr;
+    int *rf_cnt = nullptr;
+    int round_part = 0;           // part of the round's batch that the pass covers
     // exactly-l rounds (Sec. 5.3): 0 = independent draws, 1 = floor(l) per round
     int sampling = 0;
     uint32_t *ex_keys = nullptr;  // per point: FP32 clock bits
@@ -275,6 +286,9 @@ cudaError_t count_fixups(Ctx &c, const int *exact_cnt);   // adds the pass's cou
 cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_t *labels, const int32_t *prev,
                            int *changed, float *dmin, int timing_cls, const int32_t *rows = nullptr,
                            const int *rows_cnt = nullptr);
+// whether the round passes of a tensor context (its format known) filter rows by their
+// candidate, by its sizes
+bool round_filter_sizes(const Ctx &c);
 // Lloyd's bounds (round_simt.cu): whether this context can use them with centers C,
 // and one assignment after a centroid update that uses them
 bool lloyd_bounds_usable(const Ctx &c, const float *C);

@@ -395,7 +395,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restr
                                                           const float *__restrict__ ub, const float *__restrict__ xnorm,
                                                           const unsigned int *cmax_bits, float ep, float en, float ec,
                                                           uint8_t *__restrict__ cimg, float *__restrict__ cscale,
-                                                          float *__restrict__ thr) {
+                                                          float *__restrict__ thr,
+                                                          const unsigned int *__restrict__ rad2) {
     const int64_t nf = *cnt;
     const int per_row = KA * 8;
     const float W = fp32_tie_window(d);
@@ -410,7 +411,61 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restr
         *reinterpret_cast<uint4 *>(dst) = __ldg(reinterpret_cast<const uint4 *>(src));
         if (a == 0 && ch == 0) {
             cscale[i] = xscale ? xscale[R] : 1.f;
-            thr[i] = list_threshold(ub[R], xnorm[R], cmax, ep, en, ec, W);
+            const float u = rad2 ? 4.f * (1.f + 16.f * W) * __uint_as_float(rad2[i]) : ub[R];
+            thr[i] = list_threshold(u, xnorm[R], cmax, ep, en, ec, W);
+        }
+    }
+}
+
+// After a list pass over candidates (position i of the pass = candidate cin[i], or i):
+// a candidate whose lists hold gets head {entries, squared radius} and its entries in
+// one run; one that overflowed goes to the next pass (its image row, scale, candidate
+// number, radius and threshold to the next position there) with half the radius, or,
+// when there is none (cout null), gets a negative radius: no row of it is covered.
+// One warp per candidate.
+__global__ void __launch_bounds__(256) list_level_kernel(
+    const int *cnt, const int32_t *__restrict__ cin, const unsigned int *__restrict__ rin,
+    const int32_t *__restrict__ lst, const int32_t *__restrict__ lcnt, const uint8_t *__restrict__ img,
+    const float *__restrict__ scale, int KA, int d, const int32_t *__restrict__ cand,
+    const float *__restrict__ xnorm, const unsigned int *cmax_bits, float ep, float en, float ec, int32_t *glst,
+    int2 *ghead, int *cnt_out, int32_t *cout, unsigned int *rout, uint8_t *img_out, float *scale_out, float *thr_out) {
+    const int lane = threadIdx.x & 31;
+    const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+    const int total = *cnt;
+    const float W = fp32_tie_window(d);
+    const float cmax = __uint_as_float(*cmax_bits);
+    for (int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); i < total; i += nw) {
+        const int a = cin ? cin[i] : i;
+        const float r2 = __uint_as_float(rin[i]);
+        const int4 c = __ldg(reinterpret_cast<const int4 *>(lcnt) + i);
+        if (max(max(c.x, c.y), max(c.z, c.w)) <= kListSlots) {
+            // lane l: entry l % 8 of column group l / 8
+            const int g = lane >> 3, e = lane & 7;
+            const int n = g == 0 ? c.x : g == 1 ? c.y : g == 2 ? c.z : c.w;
+            const int before = (g > 0 ? c.x : 0) + (g > 1 ? c.y : 0) + (g > 2 ? c.z : 0);
+            if (e < n) glst[(size_t)a * 4 * kListSlots + before + e] = lst[(size_t)i * 4 * kListSlots + lane];
+            if (lane == 0) ghead[a] = make_int2(c.x + c.y + c.z + c.w, __float_as_int(r2));
+            continue;
+        }
+        if (!cout) {
+            if (lane == 0) ghead[a] = make_int2(0, __float_as_int(-1.f));
+            continue;
+        }
+        int o = 0;
+        if (lane == 0) o = atomicAdd(cnt_out, 1);
+        o = __shfl_sync(0xffffffffu, o, 0);
+        for (int f = lane; f < KA * 8; f += 32) {
+            const int k = f >> 3, ch = f & 7;
+            const uint8_t *src = img + (size_t)(i / BM) * KA * BM * 128 + (size_t)k * BM * 128 + sw128_off(i % BM, ch);
+            uint8_t *dst = img_out + (size_t)(o / BM) * KA * BM * 128 + (size_t)k * BM * 128 + sw128_off(o % BM, ch);
+            *reinterpret_cast<uint4 *>(dst) = __ldg(reinterpret_cast<const uint4 *>(src));
+        }
+        if (lane == 0) {
+            const float h = 0.25f * r2;
+            cout[o] = a;
+            rout[o] = __float_as_uint(h);
+            scale_out[o] = scale[i];
+            thr_out[o] = list_threshold(4.f * (1.f + 16.f * W) * h, xnorm[cand[a]], cmax, ep, en, ec, W);
         }
     }
 }
@@ -541,11 +596,46 @@ void tc_bound(int d, int fmt, float *ep, float *en, float *ec) {
 cudaError_t launch_gather_rows(const uint8_t *img, const float *xscale, int d, int fmt, const int32_t *rows,
                                const int *cnt, const float *ub, const float *xnorm, const unsigned int *cmax_bits,
                                float ep, float en, float ec, uint8_t *cimg, float *cscale, float *thr, int grid,
-                               cudaStream_t s) {
+                               cudaStream_t s, const unsigned int *rad2) {
     gather_rows_kernel<<<grid, 256, 0, s>>>(img, fmt == FMT_FP8 ? xscale : nullptr, d, tc_katoms(d, fmt), rows, cnt,
-                                            ub, xnorm, cmax_bits, ep, en, ec, cimg, cscale, thr);
+                                            ub, xnorm, cmax_bits, ep, en, ec, cimg, cscale, thr, rad2);
     count_launches(1);
     return cudaGetLastError();
+}
+
+// Lists of the new candidates (p: the pass's center side) around every old one: levels
+// of halved radius for the old candidates whose lists overflow.
+cudaError_t launch_candidate_lists(TcParams p, const ListBufs &b, const int32_t *cand, const int *old_cnt,
+                                   float ep, float en, float ec, int num_sms, cudaStream_t s) {
+    const int KA = tc_katoms(p.d, p.fmt);
+    const size_t second = (size_t)((b.cap + BM - 1) / BM) * KA * BM * 128;   // image of the odd levels
+    uint8_t *img[2] = {b.cimg, b.cimg + second};
+    float *scale[2] = {b.cscale, b.cscale + b.cap}, *thr[2] = {b.thr, b.thr + b.cap};
+    unsigned int *rad[2] = {b.rad2, b.rad2 + b.cap};
+    int32_t *num[2] = {b.num, b.num + b.cap};
+    cudaError_t e = cudaMemsetAsync(b.cnt, 0, sizeof(int) * kListLevels, s);
+    if (e != cudaSuccess) return e;
+    // level 0: the old candidates are rows of X
+    if ((e = launch_gather_rows(p.ximg, p.xscale, p.d, p.fmt, cand, old_cnt, nullptr, p.xnorm, p.cmax_bits, ep, en, ec,
+                                img[0], scale[0], thr[0], num_sms * 8, s, rad[0])) != cudaSuccess)
+        return e;
+    const float *xnorm = p.xnorm;
+    for (int l = 0; l < kListLevels; ++l) {
+        const int h = l & 1;
+        const bool last = l == kListLevels - 1;
+        p.ximg = img[h];
+        p.xscale = scale[h];
+        p.thr = thr[h];
+        p.nrows_dev = l == 0 ? old_cnt : b.cnt + l;
+        if ((e = launch_nearest_tc(p, 1, EPI_LIST, num_sms, s)) != cudaSuccess) return e;
+        list_level_kernel<<<num_sms * 4, 256, 0, s>>>(
+            p.nrows_dev, l == 0 ? nullptr : num[h], rad[h], p.lst, p.lcnt, img[h], scale[h], KA, p.d, cand, xnorm,
+            p.cmax_bits, ep, en, ec, b.glst, b.ghead, last ? nullptr : b.cnt + l + 1, last ? nullptr : num[h ^ 1],
+            rad[h ^ 1], img[h ^ 1], scale[h ^ 1], thr[h ^ 1]);
+        count_launches(1);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_row_thresholds(const float *ub, int64_t n, int d, const float *xnorm,

@@ -22,6 +22,14 @@ namespace kmp {
 
 constexpr int kNearThreads = 128;
 
+// How the resident refine covers a pass of cap_rows centers: `parts` launches of
+// `rows` centers each (`hold` rows of shared memory, `warps` warps per CTA).
+// parts = 0: the per-row kernel (refine_kernel) is used instead.
+struct ResidentPlan {
+    int parts, rows, hold, warps;
+};
+ResidentPlan resident_plan(int cap_rows, int d);
+
 enum { MODE_FIRST = 0, MODE_ROUND = 1, MODE_ASSIGN = 2 };
 
 struct NearestParams {
@@ -230,6 +238,7 @@ __global__ void pick_first_kernel(const float *X, int64_t n, int d, uint64_t see
         st->i0 = (int32_t)i0;
         cand[0] = (int32_t)i0;
         st->m = 1;
+        st->part_open = -1;
         st->batch_begin = 0;
         st->batch_cnt = 1;
         st->drawn = 0;
@@ -387,12 +396,73 @@ cudaError_t launch_round(Ctx &c, int round) {
 cudaError_t launch_sum_rows(const float *v, int64_t n, double *partials, int max_parts, double *out, double *copy,
                             cudaStream_t s);
 
+// Whether the round passes filter rows by their candidate (see the round filter): the
+// lists take a screening pass over the old candidates, at most cap_total of them, so
+// they have to be few against the rows.
+bool round_filter_sizes(const Ctx &c) {
+    return c.rounds > 0 && tc::tc_norms_in_epilogue(c.tc_fmt) && c.d % 4 == 0 &&
+           resident_plan(c.cap_round, c.d).parts == 0 && (int64_t)c.cap_total <= c.n / 8;
+}
+static bool round_filter_usable(const Ctx &c) {
+    return c.rf_rows != nullptr && ((reinterpret_cast<uintptr_t>(c.X) | reinterpret_cast<uintptr_t>(c.C)) & 15u) == 0;
+}
+
+// The part of the round's batch that the next distance pass covers: part s of S equal
+// ones, or all that is left when the filter left most rows open in the pass before (the
+// data does not separate, and every part would go over all rows again) or hardly any
+// (nothing is left to save); s = S: the whole batch again.
+__global__ void round_part_kernel(DevState *st, int s, int S, const int *open_cnt, int64_t n) {
+    if (s > 0 && open_cnt && st->batch_cnt > 0) st->part_open = *open_cnt;   // of the pass before
+    if (s == 0) {
+        st->part_begin = st->batch_begin;
+        st->part_total = st->batch_cnt;
+        st->part_next = 0;
+    }
+    const int total = st->part_total, from = st->part_next;
+    if (s == S) {
+        st->batch_begin = st->part_begin;
+        st->batch_cnt = total;
+        return;
+    }
+    const int64_t open = st->part_open;
+    const bool rest = s == S - 1 || (open >= 0 && (open * 4 > 3 * n || open * 50 < n));
+    const int to = rest ? total : max(from, (int)((int64_t)total * (s + 1) / S));
+    st->batch_begin = st->part_begin + from;
+    st->batch_cnt = to - from;
+    st->part_next = to;
+}
+
+// Parts of a round's batch.  A part's candidates filter the parts after it, so the dense
+// pass of a later part covers fewer rows; a part costs about 9 ns a row beyond its
+// screening (2 ps a row and candidate at d = 128), which parts of about 5,000
+// candidates outweigh.
+static int round_parts(const Ctx &c) {
+    if (!round_filter_usable(c)) return 1;
+    return std::max(1, std::min(4, c.cap_round / 5000));
+}
+
 // Alg. 2 step 5: D^2/idx against the batch just appended, then phi
 cudaError_t launch_round_distance(Ctx &c, int round) {
     cudaError_t e;
     if (c.precision != KMPAR_FP32) {
-        if ((e = launch_tc_pass(c, 1, c.C, 0, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr)) != cudaSuccess)
-            return e;
+        const int S = round_parts(c);
+        for (int s = 0; s < S; ++s) {
+            c.round_part = s;
+            if (S > 1) {
+                // (the first pass of the first round has no filter)
+                round_part_kernel<<<1, 1, 0, c.stream>>>(c.st, s, S, s + c.rounds_done > 1 ? c.rf_cnt : nullptr, c.n);
+                count_launches(1);
+            }
+            if ((e = launch_tc_pass(c, 1, c.C, 0, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr)) !=
+                cudaSuccess)
+                return e;
+        }
+        c.round_part = 0;
+        if (S > 1) {
+            round_part_kernel<<<1, 1, 0, c.stream>>>(c.st, S, S, c.rf_cnt, c.n);
+            count_launches(1);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
         return launch_sum_rows(c.D2, c.n, c.partials, c.num_partials, &c.st->phi, &c.st->phi_hist[round], c.stream);
     }
     cudaEvent_t ev = nullptr;
@@ -561,24 +631,25 @@ __device__ __forceinline__ int decide_top2(const float *__restrict__ X, int d, c
 // screening statistics of a pass: rows screened, rows the pair screening left
 // undecided, and (after the list pass) rows that needed the exact scan
 __global__ void count_fixups_kernel(const int *fix_cnt, const int *exact_cnt, int64_t n, const int *rows_cnt,
-                                    DevState *st) {
+                                    DevState *st, int count_rows) {
     st->screen_fallback += (unsigned long long)*fix_cnt;
-    st->screen_rows += (unsigned long long)(rows_cnt ? (int64_t)*rows_cnt : n);
+    if (count_rows) st->screen_rows += (unsigned long long)(rows_cnt ? (int64_t)*rows_cnt : n);
     st->screen_exact += (unsigned long long)(exact_cnt ? *exact_cnt : *fix_cnt);
 }
 
 cudaError_t count_fixups(Ctx &c, const int *exact_cnt, const int *rows_cnt = nullptr) {
-    count_fixups_kernel<<<1, 1, 0, c.stream>>>(c.fix_cnt, exact_cnt, c.n, rows_cnt, c.st);
+    count_fixups_kernel<<<1, 1, 0, c.stream>>>(c.fix_cnt, exact_cnt, c.n, rows_cnt, c.st, c.round_part == 0);
     count_launches(1);
     return cudaGetLastError();
 }
 
 // the two halves of count_fixups when the undecided rows pass through several stages
-__global__ void count_stage_kernel(const int *fallback_cnt, const int *exact_cnt, int64_t n, DevState *st) {
+__global__ void count_stage_kernel(const int *fallback_cnt, const int *exact_cnt, int64_t n, const int *rows_cnt,
+                                   DevState *st, int count_rows) {
     if (fallback_cnt) {   // the rows the pair screening left, all refined from their own lists
         st->screen_fallback += (unsigned long long)*fallback_cnt;
         st->screen_listed += (unsigned long long)*fallback_cnt;
-        st->screen_rows += (unsigned long long)n;
+        if (count_rows) st->screen_rows += (unsigned long long)(rows_cnt ? (int64_t)*rows_cnt : n);
     }
     if (exact_cnt) st->screen_exact += (unsigned long long)*exact_cnt;
 }
@@ -852,6 +923,8 @@ __global__ void __launch_bounds__(256) refine_direct_kernel(const float *__restr
                                                            int *changed, float *dmin, unsigned long long *fp64_cnt,
                                                            unsigned long long *wide_cnt, const int32_t *order,
                                                            const int *nrows_dev, float *ubd, float *lbd) {
+    // (the rows a compact round pass leaves undecided are listed by position, as its
+    // lists are)
     // rows in the order given (a permutation of 0..n-1, e.g. the rows sorted by
     // their previous label: neighbouring threads then mostly read the same center
     // rows, which L1 serves), or in storage order.  nrows_dev: a compact pass over
@@ -917,7 +990,7 @@ __global__ void __launch_bounds__(256) refine_direct_kernel(const float *__restr
     } else if (fix) {
         sb.ub[R] = deciding<MODE>(D2, R, FLT_MAX);
     }
-    append_fixups(sb, fix, R);
+    append_fixups(sb, fix, MODE == MODE_ROUND ? Ri : R);
     if (MODE == MODE_ASSIGN && changed) {
         const int c = warp_sum_i32(chg);
         if (lane == 0 && c) atomicAdd(changed, c);
@@ -1066,13 +1139,6 @@ int resident_warps(int cap_rows, int d) {
 size_t resident_smem_bytes(int cap_rows, int d, int warps) {
     return sizeof(float) * ((size_t)resident_center_floats(cap_rows, d) + (size_t)warps * 2 * resident_block_floats(d));
 }
-
-// How the resident refine covers a pass of cap_rows centers: `parts` launches of
-// `rows` centers each (`hold` rows of shared memory, `warps` warps per CTA).
-// parts = 0: the per-row kernel (refine_kernel) is used instead.
-struct ResidentPlan {
-    int parts, rows, hold, warps;
-};
 
 ResidentPlan resident_plan(int cap_rows, int d) {
     const int w1 = resident_warps(cap_rows, d);
@@ -1425,7 +1491,7 @@ __device__ __forceinline__ float dist2_fp32_v4(const float *__restrict__ x, cons
 template <int MODE, bool BYROW>
 __global__ void __launch_bounds__(256) refine_list_kernel(
     const float *__restrict__ X, int d, const float *__restrict__ C, int c_cnt, const int32_t *__restrict__ rows,
-    const int *rows_cnt, const int32_t *__restrict__ lst, const int32_t *__restrict__ lcnt,
+    const int *rows_cnt, const int32_t *__restrict__ order, const int32_t *__restrict__ lst, const int32_t *__restrict__ lcnt,
     const float *__restrict__ thr, ScreenBound sb, int32_t *rows2, int *cnt2, float *D2, int32_t *idx,
     int32_t *labels, const int32_t *prev, int *changed, float *dmin, unsigned long long *fp64_cnt,
     unsigned long long *wide_cnt) {
@@ -1444,8 +1510,11 @@ __global__ void __launch_bounds__(256) refine_list_kernel(
     for (int64_t i0 = gw * 4; i0 < nrows; i0 += W * 4) {   // uniform per warp
         const int64_t i = i0 + sub;
         const bool valid = i < nrows;
-        const int64_t R = valid ? rows[i] : 0;
-        const int64_t li = BYROW ? R : i;   // the row's lists and threshold: by row, or by list position
+        // the row's lists and threshold are by list position, or (BYROW) by the listed
+        // number: the row, or its position in `order`
+        const int64_t r0 = valid ? rows[i] : 0;
+        const int64_t li = BYROW ? r0 : i;
+        const int64_t R = BYROW && order && valid ? (int64_t)order[r0] : r0;
         const int cg = valid && sl < 4 ? lcnt[li * 4 + sl] : 0;
         const bool over = (__ballot_sync(0xffffffffu, cg > S) & gmask) != 0;
         const int c0 = __shfl_sync(0xffffffffu, cg, 8 * sub), c1 = __shfl_sync(0xffffffffu, cg, 8 * sub + 1);
@@ -1496,9 +1565,231 @@ __global__ void __launch_bounds__(256) refine_list_kernel(
     }
 }
 
-// A distance pass on the tensor cores.  rows / rows_cnt (Lloyd, direct refine
-// only): the pass covers just the rows rows[0 .. *rows_cnt), gathered into a compact
-// image; the others keep what the caller wrote for them.
+// ---------------------------------------------------------------- the round filter
+// A new candidate c can only become nearest to a row x of candidate a (D(x) = d(x, a))
+// when d(a, c) < 2 D(x): otherwise d(x, c) >= d(a, c) - d(x, a) >= D(x).  So the new
+// candidates within twice the largest D of a's rows are listed once per candidate a (a
+// screening pass over the few old candidates instead of all rows), and a row examines
+// its candidate's list in exact FP32.  Margins (16 W on the squared radius, the
+// screening bound in the threshold) keep every center left off the list beyond the
+// tie window, so the decisions are those of the dense pass.  A candidate that serves a
+// far cluster too has a radius that lists everything: its list is taken again at half
+// the radius, down to an eighth, and only its rows within that are settled.
+// 1e7 x 128, l = 20,000 (a mixture of 10,000): rounds 79 + 63 + 52 + 52 + 52 ms dense ->
+// 56 + 11 + 5.2 + 5.3 + 5.4 ms; where the data do not separate, the lists cost a pass over
+// the old candidates (at most an eighth of the rows) and the rows are gathered.
+
+// per candidate, the bits of the largest D^2 among its rows (a read first: most rows
+// are below the maximum already stored)
+__global__ void __launch_bounds__(256) candidate_radius_kernel(const float *__restrict__ D2,
+                                                              const int32_t *__restrict__ idx, int64_t n,
+                                                              unsigned int *rad2) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned int v = __float_as_uint(D2[i]);
+        unsigned int *r = rad2 + idx[i];
+        if (v > *reinterpret_cast<volatile unsigned int *>(r)) atomicMax(r, v);
+    }
+}
+
+// The rows' lists examined exactly: a warp takes 32 rows (a lane holds a row's list head;
+// the next block's are loaded meanwhile) and deals their (row, entry) pairs to its lanes,
+// 32 at a time, so lanes stay busy however the lists' lengths vary (2 entries on average,
+// 5 at most of 32 rows in a late round of a mixture).  A lane computes its pair's exact
+// FP32 distance (the chain of dist2_fp32); the row's lane takes the top two of its pairs
+// and the decision of the dense pass.  Rows beyond the radius that the list covers go to
+// open_rows.  Rows and candidates are staged in shared memory by whole warps (row stride
+// an odd number of 16-byte units: a lane-per-row 16-byte read is conflict-free; straight
+// from global memory 16 bytes of 32 different rows touch 32 lines an instruction).
+// 1e7 x 128 against lists of 1.9 entries (5.1 GB of rows from HBM, 9.7 GB of candidates
+// from L2): 2.8 ms; 4.5 ms as one thread per row, 5.0 ms with the copies in loops, 5.0 ms
+// with a bulk copy a row.
+__host__ __device__ __forceinline__ int stage_stride4(int d) { return (d >> 2) | 1; }   // in 16-byte units
+constexpr int kStageExtra = 512;   // bytes per warp: 64 open rows, 32 pairs' values
+
+// RP: rows a warp copies with one instruction, each by 32 / RP lanes of 16 bytes, in NQ
+// steps (the copies are a fixed unrolled sequence of a shuffle and a predicated copy a
+// row; as a loop over rows and pieces they were two thirds of the kernel's instructions)
+template <int RP, int NQ>
+__global__ void __launch_bounds__(256) refine_group_kernel(const float *__restrict__ X, int64_t n, int d,
+                                                          const float *__restrict__ C,
+                                                          const int32_t *__restrict__ glst,
+                                                          const int2 *__restrict__ ghead, float *D2, int32_t *idx,
+                                                          int32_t *open_rows, int *open_cnt, DevState *st,
+                                                          int count_rows) {
+    extern __shared__ __align__(16) float4 gst[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int d4 = d >> 2, ss = stage_stride4(d);
+    float4 *xs = gst + (size_t)wid * (64 * ss + kStageExtra / 16), *cs = xs + 32 * ss;
+    int32_t *ob = reinterpret_cast<int32_t *>(cs + 32 * ss);    // open rows not written yet
+    float *pv = reinterpret_cast<float *>(ob + 64);              // the pairs' values
+    int32_t *pj = reinterpret_cast<int32_t *>(pv + 32);          // and candidates
+    constexpr int LW = 32 / RP;   // lanes per copied row
+    const int gq = lane / LW, lq = lane % LW;
+    const float4 *C4 = reinterpret_cast<const float4 *>(C) + lq;
+    const int64_t W = (int64_t)gridDim.x * nwarps;
+    const int begin = st->batch_begin;
+    const bool any = st->batch_cnt > 0;   // (an empty batch has no lists and changes nothing)
+    const int64_t nb = (n + 31) / 32;
+    unsigned int settled = 0, listed = 0;
+    int no = 0;
+    int64_t b = (int64_t)blockIdx.x * nwarps + wid;
+    int a = 0;
+    int2 hd = make_int2(0, 0);
+    float dd = 0.f;
+    if (any && b < nb && b * 32 + lane < n) {
+        a = idx[b * 32 + lane];
+        dd = D2[b * 32 + lane];
+        hd = __ldg(ghead + a);
+    }
+    for (; b < nb; b += W) {   // uniform per warp
+        const int64_t R = b * 32 + lane, Rn = R + 32 * W;
+        const bool valid = any && R < n, next = any && Rn < n;
+        int an = 0;
+        float ddn = 0.f;
+        if (next) {
+            an = idx[Rn];
+            ddn = D2[Rn];
+        }
+        const bool open = valid && !(dd <= __int_as_float(hd.y));
+        const int total = valid && !open ? hd.x : 0;
+        int incl = total;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        const int excl = incl - total, P = __shfl_sync(0xffffffffu, incl, 31);
+        float b1 = FLT_MAX, b2 = FLT_MAX;
+        int i1 = INT_MAX, i2 = INT_MAX;
+        const unsigned xm = __ballot_sync(0xffffffffu, total > 0);
+        const float4 *xblk = reinterpret_cast<const float4 *>(X + b * 32 * d);
+        for (int p0 = 0; p0 < P; p0 += 32) {
+            const int pi = p0 + lane;
+            // the pair's row: the first whose inclusive count exceeds pi
+            int r = 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(0xffffffffu, incl, r + o - 1) <= pi) r += o;
+            const int ar = __shfl_sync(0xffffffffu, a, r), er = pi - __shfl_sync(0xffffffffu, excl, r);
+            int j = -1;
+            if (pi < P) j = begin + __ldg(glst + (size_t)ar * 4 * tc::kListSlots + er);
+            if (p0 == 0) {
+#pragma unroll 8
+                for (int r0 = 0; r0 < 32; r0 += RP) {
+                    const int rr = r0 + gq;
+                    const bool on = (xm >> rr) & 1u;
+#pragma unroll
+                    for (int u = 0; u < NQ; ++u)
+                        if (on && lq + u * LW < d4)
+                            cp_async16(xs + rr * ss + lq + u * LW, xblk + rr * d4 + lq + u * LW);
+                }
+            }
+            const int off = j >= 0 ? j * d4 : -1;
+#pragma unroll 8
+            for (int r0 = 0; r0 < 32; r0 += RP) {
+                const int rr = r0 + gq;
+                const int o = __shfl_sync(0xffffffffu, off, rr);
+#pragma unroll
+                for (int u = 0; u < NQ; ++u)
+                    if (o >= 0 && lq + u * LW < d4) cp_async16(cs + rr * ss + lq + u * LW, C4 + o + u * LW);
+            }
+            cp_async_commit();
+            cp_async_wait<0>();
+            __syncwarp();
+            if (j >= 0) {
+                float v = 0.f;
+                const float4 *x = xs + r * ss, *c = cs + lane * ss;
+#pragma unroll 8
+                for (int p = 0; p < d4; ++p) {
+                    const float4 u = x[p], w = c[p];
+                    float t;
+                    t = __fsub_rn(u.x, w.x); v = __fmaf_rn(t, t, v);
+                    t = __fsub_rn(u.y, w.y); v = __fmaf_rn(t, t, v);
+                    t = __fsub_rn(u.z, w.z); v = __fmaf_rn(t, t, v);
+                    t = __fsub_rn(u.w, w.w); v = __fmaf_rn(t, t, v);
+                }
+                pv[lane] = v;
+                pj[lane] = j;
+            }
+            __syncwarp();   // the values are there; the staged rows are read
+            for (int q = max(excl, p0); q < min(incl, p0 + 32); ++q) {
+                const float v = pv[q - p0];
+                const int jq = pj[q - p0];
+                if (lex_lt(v, jq, b2, i2)) {
+                    if (lex_lt(v, jq, b1, i1)) { b2 = b1; i2 = i1; b1 = v; i1 = jq; }
+                    else { b2 = v; i2 = jq; }
+                }
+            }
+            __syncwarp();
+        }
+        const int2 hdn = next ? __ldg(ghead + an) : make_int2(0, 0);
+        if (i1 != INT_MAX) {
+            if (i2 == INT_MAX) { i2 = -1; b2 = FLT_MAX; }
+            decide_top2<MODE_ROUND>(X, d, C, R, b1, i1, b2, i2, D2, idx, nullptr, nullptr, nullptr, &st->argmin_fp64,
+                                    &st->argmin_wide);
+        }
+        // open rows are collected and written 32 or more at a time: one atomic on the one
+        // counter for every block of rows would queue
+        const unsigned m = __ballot_sync(0xffffffffu, open);
+        if (open) ob[no + __popc(m & ((1u << lane) - 1u))] = (int32_t)R;
+        no += __popc(m);
+        if (no > 0 && (no >= 32 || b + W >= nb)) {
+            __syncwarp();
+            int base = 0;
+            if (lane == 0) base = atomicAdd(open_cnt, no);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            for (int i = lane; i < no; i += 32) open_rows[base + i] = ob[i];
+            no = 0;
+            __syncwarp();
+        }
+        if (lane == 0) settled += (unsigned int)min((int64_t)32, n - b * 32) - __popc(m);
+        listed += (unsigned int)(total > 0);
+        a = an;
+        dd = ddn;
+        hd = hdn;
+    }
+    listed = __reduce_add_sync(0xffffffffu, listed);
+    if (lane == 0) {   // the rows settled here (the dense pass counts the open ones)
+        if (settled && count_rows) atomicAdd(&st->screen_rows, (unsigned long long)settled);
+        if (listed) {
+            atomicAdd(&st->screen_fallback, (unsigned long long)listed);
+            atomicAdd(&st->screen_listed, (unsigned long long)listed);
+        }
+    }
+}
+
+// warps per CTA: about 100 KB of staged rows a CTA, two CTAs on an SM
+int stage_warps(int d) {
+    const int w = (int)((108u * 1024u) / (64u * 16u * (unsigned)stage_stride4(d) + kStageExtra));
+    return w < 1 ? 1 : (w > 8 ? 8 : w);
+}
+size_t stage_smem_bytes(int d) { return (size_t)stage_warps(d) * (64 * 16 * stage_stride4(d) + kStageExtra); }
+
+template <int RP, int NQ>
+static cudaError_t launch_refine_group_as(Ctx &c, const float *C) {
+    const size_t smem = stage_smem_bytes(c.d);
+    cudaError_t e = cudaFuncSetAttribute(refine_group_kernel<RP, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    const int sw = stage_warps(c.d);
+    const int grid = (int)std::min<int64_t>((c.n + 32 * sw - 1) / (32 * sw), 2 * (int64_t)c.num_sms);
+    refine_group_kernel<RP, NQ><<<grid, 32 * sw, smem, c.stream>>>(c.X, c.n, c.d, C, c.rf_lst, c.rf_head, c.D2, c.idx,
+                                                                   c.rf_rows, c.rf_cnt, c.st, c.round_part == 0);
+    count_launches(1);
+    return cudaGetLastError();
+}
+static cudaError_t launch_refine_group(Ctx &c, const float *C) {
+    const int d4 = c.d >> 2;
+    if (d4 > 32) return launch_refine_group_as<1, 2>(c, C);   // (d <= 188)
+    if (d4 > 16) return launch_refine_group_as<1, 1>(c, C);
+    if (d4 > 8) return launch_refine_group_as<2, 1>(c, C);
+    if (d4 > 4) return launch_refine_group_as<4, 1>(c, C);
+    return launch_refine_group_as<8, 1>(c, C);
+}
+
+// A distance pass on the tensor cores.  rows / rows_cnt (direct refine only): the pass
+// covers just the rows rows[0 .. *rows_cnt), gathered into a compact image; the others
+// keep what the caller wrote for them.
 cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_t *labels, const int32_t *prev,
                            int *changed, float *dmin, int timing_cls, const int32_t *rows, const int *rows_cnt) {
     cudaError_t e;
@@ -1533,26 +1824,54 @@ cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_
     // the rows the groups leave undecided then need no second screening
     // (Not in the first round: its rows' D^2 is the distance to the first center alone,
     // far above the spread of any cluster, so their lists would only overflow.)
-    const bool plist = mode_round && p.group == 4 && c.tc_list && c.rounds_done >= 1;
+    const bool plist = mode_round && p.group == 4 && c.tc_list && (c.rounds_done >= 1 || c.round_part > 0);
+    // the round filter settles the rows near an old candidate; the dense pass then covers
+    // only the rows it leaves open
+    const int64_t old = 1 + (int64_t)(c.rounds_done + 1) * c.cap_round;
+    if (plist && !rows && round_filter_usable(c)) {
+        if ((e = cudaMemsetAsync(c.rf_rad2, 0, sizeof(unsigned int) * (size_t)old, c.stream)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(c.rf_cnt, 0, sizeof(int), c.stream)) != cudaSuccess) return e;
+        candidate_radius_kernel<<<c.num_sms * 8, 256, 0, c.stream>>>(c.D2, c.idx, c.n, c.rf_rad2);
+        count_launches(1);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        tc::TcParams pf = p;
+        pf.lst = c.tc_lst; pf.lcnt = c.tc_lcnt;
+        const tc::ListBufs lb{c.cap_total, c.tc_cimg, c.tc_cscale, c.tc_thr, c.rf_rad2, c.rf_num, c.rf_lst, c.rf_head,
+                              c.rf_lcnt};
+        if ((e = tc::launch_candidate_lists(pf, lb, c.cand, &c.st->batch_begin, sb.ep, sb.en, sb.ec, c.num_sms,
+                                            c.stream)) != cudaSuccess)
+            return e;
+        if ((e = launch_refine_group(c, C)) != cudaSuccess) return e;
+        rows = c.rf_rows;
+        rows_cnt = c.rf_cnt;
+    }
     if (plist) {
-        if ((e = tc::launch_row_thresholds(c.D2, c.n, c.d, c.tc_xnorm, c.tc_cmax, sb.ep, sb.en, sb.ec, c.tc_thr,
+        if (!rows && (e = tc::launch_row_thresholds(c.D2, c.n, c.d, c.tc_xnorm, c.tc_cmax, sb.ep, sb.en, sb.ec, c.tc_thr,
                                            c.stream)) != cudaSuccess)
             return e;
         p.thr = c.tc_thr; p.lst = c.tc_lst; p.lcnt = c.tc_lcnt;
     }
     if (rows) {
-        // the compact image of the listed rows (their scales too; the thresholds the
-        // gather also writes are not used by the pair epilogue)
-        if (mode_round || !direct || p.group != 4 || !c.tc_cimg) return cudaErrorInvalidValue;
-        if ((e = tc::launch_gather_rows(c.tc_ximg, c.tc_xscale, c.d, fmt, rows, rows_cnt, c.tc_ub, c.tc_xnorm,
-                                        c.tc_cmax, sb.ep, sb.en, sb.ec, c.tc_cimg, c.tc_cscale, c.tc_thr,
-                                        c.num_sms * 8, c.stream)) != cudaSuccess)
+        // the compact image of the listed rows, with their scales and, for a listing
+        // pass, their thresholds (by D^2)
+        if (!direct || p.group != 4 || !c.tc_cimg) return cudaErrorInvalidValue;
+        if ((e = tc::launch_gather_rows(c.tc_ximg, c.tc_xscale, c.d, fmt, rows, rows_cnt,
+                                        mode_round ? c.D2 : c.tc_ub, c.tc_xnorm, c.tc_cmax, sb.ep, sb.en, sb.ec,
+                                        c.tc_cimg, c.tc_cscale, c.tc_thr, c.num_sms * 8, c.stream)) != cudaSuccess)
             return e;
         p.ximg = c.tc_cimg; p.xscale = c.tc_cscale; p.nrows_dev = rows_cnt;
-        if ((e = tc::launch_nearest_tc(p, 0, tc::EPI_PAIR, c.num_sms, c.stream)) != cudaSuccess) return e;
-        refine_direct_kernel<MODE_ASSIGN, 4><<<(int)((c.n + 255) / 256), 256, 0, c.stream>>>(
-            c.X, c.n, c.d, C, k, c.cand1, c.tc_v2, sb, nullptr, nullptr, labels, prev, changed, dmin,
-            &c.st->argmin_fp64, &c.st->argmin_wide, rows, rows_cnt, c.ll_ub, c.ll_lb);
+        if ((e = tc::launch_nearest_tc(p, mode_round, plist ? tc::EPI_PAIRLIST : tc::EPI_PAIR, c.num_sms, c.stream)) !=
+            cudaSuccess)
+            return e;
+        const int grid = (int)((c.n + 255) / 256);
+        if (mode_round)
+            refine_direct_kernel<MODE_ROUND, 4><<<grid, 256, 0, c.stream>>>(
+                c.X, c.n, c.d, C, 0, c.cand1, c.tc_v2, sb, c.D2, c.idx, nullptr, nullptr, nullptr, nullptr,
+                &c.st->argmin_fp64, &c.st->argmin_wide, rows, rows_cnt, nullptr, nullptr);
+        else
+            refine_direct_kernel<MODE_ASSIGN, 4><<<grid, 256, 0, c.stream>>>(
+                c.X, c.n, c.d, C, k, c.cand1, c.tc_v2, sb, nullptr, nullptr, labels, prev, changed, dmin,
+                &c.st->argmin_fp64, &c.st->argmin_wide, rows, rows_cnt, c.ll_ub, c.ll_lb);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     } else {
@@ -1639,11 +1958,11 @@ cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_
         if ((e2 = tc::launch_nearest_tc(pl, mode_round, tc::EPI_LIST, c.num_sms, c.stream)) != cudaSuccess) return e2;
         if (mode_round)
             refine_list_kernel<MODE_ROUND, false><<<lgrid, 256, 0, c.stream>>>(
-                c.X, c.d, C, 0, rows_in, cnt_in, c.tc_lst, c.tc_lcnt, c.tc_thr, sb, rows_out, cnt_out, c.D2, c.idx,
+                c.X, c.d, C, 0, rows_in, cnt_in, nullptr, c.tc_lst, c.tc_lcnt, c.tc_thr, sb, rows_out, cnt_out, c.D2, c.idx,
                 nullptr, nullptr, nullptr, nullptr, &c.st->argmin_fp64, &c.st->argmin_wide);
         else
             refine_list_kernel<MODE_ASSIGN, false><<<lgrid, 256, 0, c.stream>>>(
-                c.X, c.d, C, k, rows_in, cnt_in, c.tc_lst, c.tc_lcnt, c.tc_thr, sb, rows_out, cnt_out, nullptr,
+                c.X, c.d, C, k, rows_in, cnt_in, nullptr, c.tc_lst, c.tc_lcnt, c.tc_thr, sb, rows_out, cnt_out, nullptr,
                 nullptr, labels, prev, changed, dmin, &c.st->argmin_fp64, &c.st->argmin_wide);
         count_launches(1);
         return cudaGetLastError();
@@ -1658,14 +1977,14 @@ cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_
     // rows that one leaves, the exact scan
     if ((e = cudaMemsetAsync(c.fix_cnt2, 0, sizeof(int), c.stream)) != cudaSuccess) return e;
     refine_list_kernel<MODE_ROUND, true><<<lgrid, 256, 0, c.stream>>>(
-        c.X, c.d, C, 0, c.fix_rows, c.fix_cnt, c.tc_lst, c.tc_lcnt, c.tc_thr, sb, c.fix_rows2, c.fix_cnt2, c.D2, c.idx,
+        c.X, c.d, C, 0, c.fix_rows, c.fix_cnt, rows, c.tc_lst, c.tc_lcnt, c.tc_thr, sb, c.fix_rows2, c.fix_cnt2, c.D2, c.idx,
         nullptr, nullptr, nullptr, nullptr, &c.st->argmin_fp64, &c.st->argmin_wide);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    count_stage_kernel<<<1, 1, 0, c.stream>>>(c.fix_cnt, nullptr, c.n, c.st);
+    count_stage_kernel<<<1, 1, 0, c.stream>>>(c.fix_cnt, nullptr, c.n, rows_cnt, c.st, c.round_part == 0);
     count_launches(1);
     if ((e = list_pass(c.fix_rows2, c.fix_cnt2, c.fix_rows, c.fix_cnt)) != cudaSuccess) return e;
-    count_stage_kernel<<<1, 1, 0, c.stream>>>(nullptr, c.fix_cnt, c.n, c.st);
+    count_stage_kernel<<<1, 1, 0, c.stream>>>(nullptr, c.fix_cnt, c.n, nullptr, c.st, 0);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return launch_fixup(c, mode_round, C, k, labels, prev, changed, dmin, c.fix_rows, c.fix_cnt);
