@@ -129,7 +129,8 @@ void free_ctx(kmp::Ctx &c) {
                     c.tc_ncol, c.tc_tscale, c.tc_xscale, c.tc_ub, c.tc_cimg, c.tc_cscale, c.tc_thr,
                     c.tc_lst, c.tc_lcnt, c.fix_rows2, c.fix_cnt2, c.rCT, c.wl_lab[0], c.wl_lab[1], c.rs_buf,
                     c.ll_ub, c.ll_lb, c.ll_rows, c.ll_cnt, c.ll_cold, c.ll_drift, c.ll_other, c.rf_rad2, c.rf_num, c.rf_lst, c.rf_head,
-                    c.rf_lcnt, c.rf_rows, c.rf_cnt};
+                    c.rf_lcnt, c.rf_rows, c.rf_cnt, c.ll_rad2, c.ll_num, c.ll_lst, c.ll_head, c.ll_lcnt, c.ll_tau2,
+                    c.ll_img, c.ll_xnorm, c.ll_xscale, c.ll_pend, c.ll_flag, c.ll_pick};
     // stream-ordered: the memory returns to the pool once the context's work is done
     for (void *b : bufs)
         if (b) cudaFreeAsync(b, c.stream);
@@ -501,10 +502,26 @@ static kmpar_status ensure_lloyd_buffers(kmp::Ctx &c) {
         KMP_ENSURE(c.ll_ub, (size_t)c.n, "alloc Lloyd bounds");
         KMP_ENSURE(c.ll_lb, (size_t)c.n, "alloc Lloyd bounds");
         KMP_ENSURE(c.ll_rows, (size_t)c.n, "alloc Lloyd rows");
-        KMP_ENSURE(c.ll_cnt, 1, "alloc Lloyd row count");
+        KMP_ENSURE(c.ll_cnt, 2, "alloc Lloyd row counts");
         KMP_ENSURE(c.ll_cold, (size_t)c.k * c.d, "alloc previous centers");
         KMP_ENSURE(c.ll_drift, (size_t)c.k, "alloc center drifts");
         KMP_ENSURE(c.ll_other, (size_t)c.k, "alloc center drifts");
+        if (kmp::lloyd_lists_usable(c)) {
+            namespace tc = kmp::tc;
+            const size_t cap = (size_t)std::max(c.cap_total, c.k), k128 = (size_t)((c.k + 127) / 128) * 128;
+            KMP_ENSURE(c.ll_rad2, 2 * cap, "alloc Lloyd list radii");
+            KMP_ENSURE(c.ll_num, 2 * cap, "alloc Lloyd list numbers");
+            KMP_ENSURE(c.ll_lst, cap * 4 * tc::kListSlots, "alloc Lloyd lists");
+            KMP_ENSURE(c.ll_head, cap, "alloc Lloyd list heads");
+            KMP_ENSURE(c.ll_lcnt, tc::kListLevels + 2, "alloc Lloyd list counts");
+            KMP_ENSURE(c.ll_tau2, cap, "alloc Lloyd list distances");
+            KMP_ENSURE(c.ll_img, tc::tc_points_image_bytes(c.d, c.tc_fmt, c.k), "alloc center image");
+            KMP_ENSURE(c.ll_xnorm, k128, "alloc center norms");
+            KMP_ENSURE(c.ll_xscale, k128, "alloc center scales");
+            KMP_ENSURE(c.ll_pend, (size_t)c.n, "alloc pending rows");
+            KMP_ENSURE(c.ll_flag, (size_t)c.k, "alloc cluster flags");
+            KMP_ENSURE(c.ll_pick, (size_t)kmp::pick_counts(c.n) + 1, "alloc changed row counts");
+        }
     }
 #undef KMP_ENSURE
     c.lloyd_ready = true;
@@ -542,6 +559,7 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
     // after the first assignment, rows whose bounds prove their center unchanged are
     // settled without the tensor pass (the results are the same)
     const bool bounded = kmp::lloyd_bounds_usable(c, centers_dev);
+    const bool listed = bounded && kmp::lloyd_lists_usable(c);
     auto keep_centers = [&]() -> cudaError_t {
         return bounded ? cudaMemcpyAsync(c.ll_cold, centers_dev, sizeof(float) * (size_t)c.k * c.d,
                                          cudaMemcpyDeviceToDevice, c.stream)
@@ -553,7 +571,9 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
         for (int tt = t; tt <= t_end; ++tt) {
             if (tt > t) {
                 KMP_CUDA(&c, keep_centers(), "keep centers");
-                KMP_CUDA(&c, kmp::launch_centroids(c, c.labels[cur], centers_dev), "centroid kernels");
+                KMP_CUDA(&c, kmp::launch_centroids(c, c.labels[cur], listed && tt > 1 ? c.labels[cur ^ 1] : nullptr,
+                                                   centers_dev),
+                         "centroid kernels");
                 cur ^= 1;
             }
             KMP_CUDA(&c, cudaMemsetAsync(changed, 0, sizeof(int), c.stream), "memset changed");
@@ -567,9 +587,10 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
                 KMP_CUDA(&c, kmp::timing_end(c, ev, 1), "timing");
                 KMP_CUDA(&c, kmp::launch_sum_f64(c.partials, c.num_partials, c.cost_dev, nullptr, c.stream),
                          "cost sum");
-            } else if (bounded && tt > 0) {
-                KMP_CUDA(&c, kmp::launch_lloyd_bounded_pass(c, centers_dev, c.labels[cur], c.labels[cur ^ 1],
-                                                             changed, c.dmin),
+            } else if (bounded && (tt > 0 || listed)) {
+                KMP_CUDA(&c, tt > 0 ? kmp::launch_lloyd_bounded_pass(c, centers_dev, c.labels[cur], c.labels[cur ^ 1],
+                                                                     changed, c.dmin)
+                                    : kmp::launch_lloyd_first_pass(c, centers_dev, c.labels[cur], changed, c.dmin),
                          "bounded assign pass");
                 KMP_CUDA(&c, kmp::launch_sum_rows(c.dmin, c.n, c.partials, c.num_partials, c.cost_dev, nullptr,
                                                   c.stream),
@@ -604,7 +625,9 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
         if (done < 0) {
             // the last iteration of the batch still needs its centroid update
             KMP_CUDA(&c, keep_centers(), "keep centers");
-            KMP_CUDA(&c, kmp::launch_centroids(c, c.labels[cur], centers_dev), "centroid kernels");
+            KMP_CUDA(&c, kmp::launch_centroids(c, c.labels[cur], listed && t_end > 0 ? c.labels[cur ^ 1] : nullptr,
+                                               centers_dev),
+                     "centroid kernels");
             cur ^= 1;
             t = t_end + 1;
         }

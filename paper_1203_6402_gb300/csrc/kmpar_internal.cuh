@@ -93,6 +93,20 @@ struct Ctx {
     float *ll_cold = nullptr, *ll_drift = nullptr, *ll_other = nullptr;
     int32_t *ll_rows = nullptr;
     int *ll_cnt = nullptr;
+    // Lloyd's lists: references (candidates in the first assignment, centers after) with
+    // their radii, lists and distances to some center; the centers' own point image; rows
+    // whose bounds fail; per cluster, whether its members changed
+    unsigned int *ll_rad2 = nullptr;
+    int32_t *ll_num = nullptr, *ll_lst = nullptr;
+    int2 *ll_head = nullptr;
+    int *ll_lcnt = nullptr;       // kListLevels counts, then k, then the pending rows
+    float *ll_tau2 = nullptr;
+    uint8_t *ll_img = nullptr;
+    float *ll_xnorm = nullptr, *ll_xscale = nullptr;
+    int32_t *ll_pend = nullptr;
+    int *ll_flag = nullptr;
+    int *ll_pick = nullptr;       // rows of changed clusters per warp's share, then their number
+    bool tc_prepared = false;     // the pass's center tiles are encoded already
     int32_t *hist = nullptr;      // nsb x k
     int32_t *base = nullptr;      // k + 1
     int32_t *piece = nullptr;     // k + 1: first piece of each cluster
@@ -278,10 +292,13 @@ cudaError_t launch_assign(const float *X, int64_t n, int d, const float *C, int 
                           const int32_t *prev, int *changed, double *partials, int nparts,
                           unsigned long long *fp64_cnt, cudaStream_t s);
 int assign_num_partials(int64_t n, int d);
-cudaError_t launch_centroids(Ctx &c, const int32_t *labels, float *centers);
+// before: the labels the centers are the centroids of, so that clusters whose members
+// are the same keep their center (null: all are summed; needs Lloyd's lists)
+cudaError_t launch_centroids(Ctx &c, const int32_t *labels, const int32_t *before, float *centers);
 int sort_block_size(int64_t n, int k);
 int64_t max_pieces(int64_t n, int k);
 int64_t scan_chunks(int nsb);
+int pick_counts(int64_t n);
 cudaError_t count_fixups(Ctx &c, const int *exact_cnt);   // adds the pass's counts to the screening stats
 cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_t *labels, const int32_t *prev,
                            int *changed, float *dmin, int timing_cls, const int32_t *rows = nullptr,
@@ -294,6 +311,9 @@ bool round_filter_sizes(const Ctx &c);
 bool lloyd_bounds_usable(const Ctx &c, const float *C);
 cudaError_t launch_lloyd_bounded_pass(Ctx &c, const float *C, int32_t *labels, const int32_t *prev, int *changed,
                                       float *dmin);
+// the first assignment of a context that can use the bounds, by the candidates' lists
+bool lloyd_lists_usable(const Ctx &c);
+cudaError_t launch_lloyd_first_pass(Ctx &c, const float *C, int32_t *labels, int *changed, float *dmin);
 cudaError_t launch_sum_rows(const float *v, int64_t n, double *partials, int max_parts, double *out, double *copy,
                             cudaStream_t s);
 cudaError_t launch_uniforms(int64_t count, uint32_t round, uint32_t tag, uint64_t seed, double *out,

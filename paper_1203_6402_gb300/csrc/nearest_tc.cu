@@ -379,6 +379,13 @@ __device__ __forceinline__ float list_threshold(float u, float xnorm, float cmax
     return t;
 }
 
+// squared reach of a reference's list that covers its rows up to the squared radius r2,
+// tau2 the squared distance from the reference to some center: (2 r + tau)^2, widened
+__device__ __forceinline__ float list_reach2(float r2, float tau2, float W) {
+    const float r = 2.f * sqrtf(r2) + sqrtf(tau2);
+    return r * r * (1.f + 20.f * W);
+}
+
 __global__ void __launch_bounds__(256) row_thresholds_kernel(const float *__restrict__ ub, int64_t n, int d,
                                                              const float *__restrict__ xnorm,
                                                              const unsigned int *cmax_bits, float ep, float en,
@@ -396,7 +403,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restr
                                                           const unsigned int *cmax_bits, float ep, float en, float ec,
                                                           uint8_t *__restrict__ cimg, float *__restrict__ cscale,
                                                           float *__restrict__ thr,
-                                                          const unsigned int *__restrict__ rad2) {
+                                                          const unsigned int *__restrict__ rad2,
+                                                          const float *__restrict__ tau2) {
     const int64_t nf = *cnt;
     const int per_row = KA * 8;
     const float W = fp32_tie_window(d);
@@ -405,30 +413,30 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restr
          f += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = f / per_row;
         const int a = (int)((f % per_row) >> 3), ch = (int)(f & 7);
-        const int64_t R = rows[i];
+        const int64_t R = rows ? (int64_t)rows[i] : i;
         const uint8_t *src = img + (size_t)(R / BM) * KA * BM * 128 + (size_t)a * BM * 128 + sw128_off((int)(R % BM), ch);
         uint8_t *dst = cimg + (size_t)(i / BM) * KA * BM * 128 + (size_t)a * BM * 128 + sw128_off((int)(i % BM), ch);
         *reinterpret_cast<uint4 *>(dst) = __ldg(reinterpret_cast<const uint4 *>(src));
         if (a == 0 && ch == 0) {
             cscale[i] = xscale ? xscale[R] : 1.f;
-            const float u = rad2 ? 4.f * (1.f + 16.f * W) * __uint_as_float(rad2[i]) : ub[R];
+            const float u = rad2 ? list_reach2(__uint_as_float(rad2[i]), tau2 ? tau2[i] : 0.f, W) : ub[R];
             thr[i] = list_threshold(u, xnorm[R], cmax, ep, en, ec, W);
         }
     }
 }
 
-// After a list pass over candidates (position i of the pass = candidate cin[i], or i):
-// a candidate whose lists hold gets head {entries, squared radius} and its entries in
-// one run; one that overflowed goes to the next pass (its image row, scale, candidate
-// number, radius and threshold to the next position there) with half the radius, or,
-// when there is none (cout null), gets a negative radius: no row of it is covered.
-// One warp per candidate.
+// After a list pass over references (position i of the pass = reference rin_num[i], or i):
+// a reference whose lists hold gets head {entries, squared radius} and its entries in
+// one run; one that overflowed goes to the next pass (its image row, scale, number,
+// radius and threshold to the next position there) with half the radius, or, when there
+// is none (cout null), gets a negative radius: no row of it is covered.  One warp per
+// reference.
 __global__ void __launch_bounds__(256) list_level_kernel(
     const int *cnt, const int32_t *__restrict__ cin, const unsigned int *__restrict__ rin,
     const int32_t *__restrict__ lst, const int32_t *__restrict__ lcnt, const uint8_t *__restrict__ img,
     const float *__restrict__ scale, int KA, int d, const int32_t *__restrict__ cand,
-    const float *__restrict__ xnorm, const unsigned int *cmax_bits, float ep, float en, float ec, int32_t *glst,
-    int2 *ghead, int *cnt_out, int32_t *cout, unsigned int *rout, uint8_t *img_out, float *scale_out, float *thr_out) {
+    const float *__restrict__ xnorm, const float *__restrict__ tau2, const unsigned int *cmax_bits, float ep, float en,
+    float ec, int32_t *glst, int2 *ghead, int *cnt_out, int32_t *cout, unsigned int *rout, uint8_t *img_out, float *scale_out, float *thr_out) {
     const int lane = threadIdx.x & 31;
     const int nw = (int)((gridDim.x * blockDim.x) >> 5);
     const int total = *cnt;
@@ -439,12 +447,15 @@ __global__ void __launch_bounds__(256) list_level_kernel(
         const float r2 = __uint_as_float(rin[i]);
         const int4 c = __ldg(reinterpret_cast<const int4 *>(lcnt) + i);
         if (max(max(c.x, c.y), max(c.z, c.w)) <= kListSlots) {
-            // lane l: entry l % 8 of column group l / 8
+            // lane l: entry l % 8 of column group l / 8; references that are the centers
+            // themselves (cand null) are left off their own lists
             const int g = lane >> 3, e = lane & 7;
             const int n = g == 0 ? c.x : g == 1 ? c.y : g == 2 ? c.z : c.w;
-            const int before = (g > 0 ? c.x : 0) + (g > 1 ? c.y : 0) + (g > 2 ? c.z : 0);
-            if (e < n) glst[(size_t)a * 4 * kListSlots + before + e] = lst[(size_t)i * 4 * kListSlots + lane];
-            if (lane == 0) ghead[a] = make_int2(c.x + c.y + c.z + c.w, __float_as_int(r2));
+            const int v = e < n ? lst[(size_t)i * 4 * kListSlots + lane] : -1;
+            const bool keep = v >= 0 && (cand || v != a);
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (keep) glst[(size_t)a * 4 * kListSlots + __popc(m & ((1u << lane) - 1u))] = v;
+            if (lane == 0) ghead[a] = make_int2(__popc(m), __float_as_int(r2));
             continue;
         }
         if (!cout) {
@@ -465,7 +476,8 @@ __global__ void __launch_bounds__(256) list_level_kernel(
             cout[o] = a;
             rout[o] = __float_as_uint(h);
             scale_out[o] = scale[i];
-            thr_out[o] = list_threshold(4.f * (1.f + 16.f * W) * h, xnorm[cand[a]], cmax, ep, en, ec, W);
+            thr_out[o] = list_threshold(list_reach2(h, tau2 ? tau2[a] : 0.f, W), xnorm[cand ? cand[a] : a], cmax, ep, en,
+                                        ec, W);
         }
     }
 }
@@ -596,17 +608,17 @@ void tc_bound(int d, int fmt, float *ep, float *en, float *ec) {
 cudaError_t launch_gather_rows(const uint8_t *img, const float *xscale, int d, int fmt, const int32_t *rows,
                                const int *cnt, const float *ub, const float *xnorm, const unsigned int *cmax_bits,
                                float ep, float en, float ec, uint8_t *cimg, float *cscale, float *thr, int grid,
-                               cudaStream_t s, const unsigned int *rad2) {
+                               cudaStream_t s, const unsigned int *rad2, const float *tau2) {
     gather_rows_kernel<<<grid, 256, 0, s>>>(img, fmt == FMT_FP8 ? xscale : nullptr, d, tc_katoms(d, fmt), rows, cnt,
-                                            ub, xnorm, cmax_bits, ep, en, ec, cimg, cscale, thr, rad2);
+                                            ub, xnorm, cmax_bits, ep, en, ec, cimg, cscale, thr, rad2, tau2);
     count_launches(1);
     return cudaGetLastError();
 }
 
-// Lists of the new candidates (p: the pass's center side) around every old one: levels
-// of halved radius for the old candidates whose lists overflow.
-cudaError_t launch_candidate_lists(TcParams p, const ListBufs &b, const int32_t *cand, const int *old_cnt,
-                                   float ep, float en, float ec, int num_sms, cudaStream_t s) {
+// Lists of centers (p: the pass's center side) around references: levels of halved
+// radius for the references whose lists overflow.
+cudaError_t launch_reference_lists(TcParams p, int mode_round, const ListBufs &b, const int32_t *cand, const int *cnt,
+                                   const float *tau2, float ep, float en, float ec, int num_sms, cudaStream_t s) {
     const int KA = tc_katoms(p.d, p.fmt);
     const size_t second = (size_t)((b.cap + BM - 1) / BM) * KA * BM * 128;   // image of the odd levels
     uint8_t *img[2] = {b.cimg, b.cimg + second};
@@ -615,9 +627,9 @@ cudaError_t launch_candidate_lists(TcParams p, const ListBufs &b, const int32_t 
     int32_t *num[2] = {b.num, b.num + b.cap};
     cudaError_t e = cudaMemsetAsync(b.cnt, 0, sizeof(int) * kListLevels, s);
     if (e != cudaSuccess) return e;
-    // level 0: the old candidates are rows of X
-    if ((e = launch_gather_rows(p.ximg, p.xscale, p.d, p.fmt, cand, old_cnt, nullptr, p.xnorm, p.cmax_bits, ep, en, ec,
-                                img[0], scale[0], thr[0], num_sms * 8, s, rad[0])) != cudaSuccess)
+    // level 0: the references' image rows (rows cand[i] of the image, or row i)
+    if ((e = launch_gather_rows(p.ximg, p.xscale, p.d, p.fmt, cand, cnt, nullptr, p.xnorm, p.cmax_bits, ep, en, ec,
+                                img[0], scale[0], thr[0], num_sms * 8, s, rad[0], tau2)) != cudaSuccess)
         return e;
     const float *xnorm = p.xnorm;
     for (int l = 0; l < kListLevels; ++l) {
@@ -626,10 +638,10 @@ cudaError_t launch_candidate_lists(TcParams p, const ListBufs &b, const int32_t 
         p.ximg = img[h];
         p.xscale = scale[h];
         p.thr = thr[h];
-        p.nrows_dev = l == 0 ? old_cnt : b.cnt + l;
-        if ((e = launch_nearest_tc(p, 1, EPI_LIST, num_sms, s)) != cudaSuccess) return e;
+        p.nrows_dev = l == 0 ? cnt : b.cnt + l;
+        if ((e = launch_nearest_tc(p, mode_round, EPI_LIST, num_sms, s)) != cudaSuccess) return e;
         list_level_kernel<<<num_sms * 4, 256, 0, s>>>(
-            p.nrows_dev, l == 0 ? nullptr : num[h], rad[h], p.lst, p.lcnt, img[h], scale[h], KA, p.d, cand, xnorm,
+            p.nrows_dev, l == 0 ? nullptr : num[h], rad[h], p.lst, p.lcnt, img[h], scale[h], KA, p.d, cand, xnorm, tau2,
             p.cmax_bits, ep, en, ec, b.glst, b.ghead, last ? nullptr : b.cnt + l + 1, last ? nullptr : num[h ^ 1],
             rad[h ^ 1], img[h ^ 1], scale[h ^ 1], thr[h ^ 1]);
         count_launches(1);

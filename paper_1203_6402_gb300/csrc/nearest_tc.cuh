@@ -84,13 +84,15 @@ cudaError_t launch_nearest_tc(TcParams p, int mode_round, int epi, int num_sms, 
 cudaError_t launch_gather_rows(const uint8_t *img, const float *xscale, int d, int fmt, const int32_t *rows,
                                const int *cnt, const float *ub, const float *xnorm, const unsigned int *cmax_bits,
                                float ep, float en, float ec, uint8_t *cimg, float *cscale, float *thr, int grid,
-                               cudaStream_t s, const unsigned int *rad2 = nullptr);
-// (rad2: instead of ub, the bound of listed row i is 4 (1 + 16 W) rad2[i], rad2 the bits
-// of a squared radius: the list then holds every center within twice that radius)
-// Work space of the candidate lists, for at most `cap` old candidates: cimg, cscale and
-// thr hold two passes' worth; rad2 (2 cap) starts with every candidate's squared
-// radius; the result is ghead (entries, squared radius covered; negative: none) and
-// glst (4 kListSlots pass-local center numbers per candidate).
+                               cudaStream_t s, const unsigned int *rad2 = nullptr, const float *tau2 = nullptr);
+// (rows null: row i.  rad2: instead of by ub, row i is a reference whose list holds every
+// center within 2 r + tau of it, r^2 given by its bits rad2[i], tau^2 = tau2[i] or 0)
+// Lists of the centers around references (points that rows are known to be near): a row
+// within r of its reference, the reference within tau of some center, has its nearest
+// center within 2 r + tau of the reference.  Work space for at most `cap` references:
+// cimg, cscale and thr hold two passes' worth; rad2 (2 cap) starts with every
+// reference's squared radius; the result is ghead (entries, squared radius covered;
+// negative: none) and glst (4 kListSlots pass-local center numbers per reference).
 constexpr int kListLevels = 4;   // radii R, R/2, R/4, R/8
 struct ListBufs {
     int cap;
@@ -101,8 +103,8 @@ struct ListBufs {
     int2 *ghead;
     int *cnt;
 };
-cudaError_t launch_candidate_lists(TcParams p, const ListBufs &b, const int32_t *cand, const int *old_cnt,
-                                   float ep, float en, float ec, int num_sms, cudaStream_t s);
+cudaError_t launch_reference_lists(TcParams p, int mode_round, const ListBufs &b, const int32_t *cand, const int *cnt,
+                                   const float *tau2, float ep, float en, float ec, int num_sms, cudaStream_t s);
 // screening error bound E(x, c) = ep ||x'|| ||c'|| + en (||x'||^2 + ||c'||^2) + ec ||x'|| max ||c'||
 void tc_bound(int d, int fmt, float *ep, float *en, float *ec);
 // per row R < n, the list threshold of a row whose nearest distance is at most ub[R]

@@ -733,8 +733,14 @@ cudaError_t launch_weighted_centroids(const Ctx &c, int m, const int32_t *lab, f
 constexpr int kPiece = 256;
 
 // per sort block b (sb points): hist[b][j] = #points with label j
-__global__ void label_hist_kernel(const int32_t *__restrict__ labels, int64_t n, int k, int sb, int32_t *hist) {
+// (the sort kernels take n rows, or *n_dev of them when given)
+__global__ void label_hist_kernel(const int32_t *__restrict__ labels, int64_t n, const int *n_dev, int k, int sb,
+                                  int32_t *hist) {
     extern __shared__ int32_t h[];
+    if (n_dev) {
+        n = *n_dev;
+        if ((int64_t)blockIdx.x * sb >= n) return;   // uniform per block
+    }
     for (int j = threadIdx.x; j < k; j += blockDim.x) h[j] = 0;
     __syncthreads();
     const int64_t b0 = (int64_t)blockIdx.x * sb;
@@ -749,11 +755,15 @@ __global__ void label_hist_kernel(const int32_t *__restrict__ labels, int64_t n,
 // row by row: hist[b][j] <- sum_{b' < b} hist[b'][j]; tot[j] = column total.
 constexpr int kScanRows = 64;
 
-__global__ void __launch_bounds__(256) column_chunk_kernel(const int32_t *__restrict__ hist, int nsb, int k,
-                                                           int32_t *chunk) {
+__global__ void __launch_bounds__(256) column_chunk_kernel(const int32_t *__restrict__ hist, int nsb, const int *n_dev,
+                                                           int sb, int k, int32_t *chunk) {
     __shared__ int part[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int j = blockIdx.x * 32 + lane, rc = blockIdx.y;
+    if (n_dev) {
+        nsb = (*n_dev + sb - 1) / sb;
+        if (rc * kScanRows >= nsb) return;   // uniform per block
+    }
     const int b0 = rc * kScanRows + w * (kScanRows / 8);
     const int b1 = min(nsb, b0 + kScanRows / 8);
     int s = 0;
@@ -768,11 +778,17 @@ __global__ void __launch_bounds__(256) column_chunk_kernel(const int32_t *__rest
     }
 }
 
-__global__ void __launch_bounds__(256) column_offset_kernel(int32_t *hist, int nsb, int k,
+__global__ void __launch_bounds__(256) column_offset_kernel(int32_t *hist, int nsb, const int *n_dev, int sb, int k,
                                                             const int32_t *__restrict__ chunk, int nrc, int32_t *tot) {
     __shared__ int part[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int j = blockIdx.x * 32 + lane, rc = blockIdx.y;
+    if (n_dev) {
+        nsb = (*n_dev + sb - 1) / sb;
+        nrc = (nsb + kScanRows - 1) / kScanRows;
+        if (nrc == 0 && rc == 0 && w == 0 && j < k) tot[j] = 0;
+        if (rc >= nrc) return;   // uniform per block
+    }
     // offset of this chunk (earlier chunks, split over the 8 warps, fixed order)
     int s = 0;
     if (j < k)
@@ -842,11 +858,17 @@ __global__ void __launch_bounds__(1024) base_scan_kernel(int32_t *tot_base, int 
 }
 
 // one warp per sort block: stable scatter of point numbers into label order
-__global__ void __launch_bounds__(32) scatter_kernel(const int32_t *__restrict__ labels, int64_t n, int k, int sb,
-                                                     const int32_t *__restrict__ hist,
+// (the rows are 0 .. n - 1, or `rows`)
+__global__ void __launch_bounds__(32) scatter_kernel(const int32_t *__restrict__ labels,
+                                                     const int32_t *__restrict__ rows, int64_t n, const int *n_dev,
+                                                     int k, int sb, const int32_t *__restrict__ hist,
                                                      const int32_t *__restrict__ base, int32_t *perm) {
     extern __shared__ int32_t cur[];
     const int lane = threadIdx.x;
+    if (n_dev) {
+        n = *n_dev;
+        if ((int64_t)blockIdx.x * sb >= n) return;   // uniform per block
+    }
     for (int j = lane; j < k; j += 32) cur[j] = base[j] + hist[(int64_t)blockIdx.x * k + j];
     __syncwarp();
     const int64_t b0 = (int64_t)blockIdx.x * sb;
@@ -857,7 +879,7 @@ __global__ void __launch_bounds__(32) scatter_kernel(const int32_t *__restrict__
         const int l = valid ? labels[i] : -1;
         const unsigned mask = __match_any_sync(0xffffffffu, l);
         const int rank = __popc(mask & ((1u << lane) - 1u));
-        if (valid) perm[cur[l] + rank] = (int32_t)i;
+        if (valid) perm[cur[l] + rank] = rows ? rows[i] : (int32_t)i;
         __syncwarp();
         if (valid && lane == __ffs(mask) - 1) cur[l] += __popc(mask);
         __syncwarp();
@@ -1008,19 +1030,116 @@ int64_t max_pieces(int64_t n, int k) { return (n + kPiece - 1) / kPiece + k; }
 
 int64_t scan_chunks(int nsb) { return (nsb + kScanRows - 1) / kScanRows; }
 
-cudaError_t launch_centroids(Ctx &c, const int32_t *labels, float *centers) {
+// Clusters that a row left or joined since the labels `before`.  A cluster with the
+// same members has the same sorted member list, pieces and sums, so its centroid is
+// the one it has, bit for bit: only the rows of the other clusters are sorted and summed,
+// and a cluster without any of them keeps its center as an empty one does.
+__global__ void __launch_bounds__(256) label_flags_kernel(const int32_t *__restrict__ labels,
+                                                         const int32_t *__restrict__ before, int64_t n, int *flag) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int a = labels[i], b = before[i];
+        if (a != b) {
+            flag[a] = 1;
+            flag[b] = 1;
+        }
+    }
+}
+
+// Rows of flagged clusters in ascending order, with their labels: counts per block of
+// kPickRows rows, their prefix, then the rows (a warp per kPickRows / 8 of them).
+constexpr int kPickRows = 8192;
+
+__global__ void __launch_bounds__(256) pick_count_kernel(const int32_t *__restrict__ labels, int64_t n,
+                                                        const int *__restrict__ flag, int *__restrict__ wcnt) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * kPickRows + w * (kPickRows / 8), r1 = min(n, r0 + kPickRows / 8);
+    int t = 0;
+    for (int64_t i = r0 + lane; i < r1; i += 32) t += flag[labels[i]] != 0;
+    t = __reduce_add_sync(0xffffffffu, t);
+    if (lane == 0) wcnt[blockIdx.x * 8 + w] = t;
+}
+
+__global__ void __launch_bounds__(1024) pick_scan_kernel(int *wcnt, int m, int *total) {
+    __shared__ int sh[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int run = 0;
+    for (int b = 0; b < m; b += 1024) {
+        const int i = b + threadIdx.x;
+        const int v = i < m ? wcnt[i] : 0;
+        int incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (lane == 31) sh[wid] = incl;
+        __syncthreads();
+        int before = run, all = 0;
+        for (int q = 0; q < 32; ++q) {
+            if (q < wid) before += sh[q];
+            all += sh[q];
+        }
+        if (i < m) wcnt[i] = before + incl - v;
+        run += all;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *total = run;
+}
+
+__global__ void __launch_bounds__(256) pick_rows_kernel(const int32_t *__restrict__ labels, int64_t n,
+                                                       const int *__restrict__ flag, const int *__restrict__ woff,
+                                                       int32_t *__restrict__ rows, int32_t *__restrict__ lab) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * kPickRows + w * (kPickRows / 8), r1 = min(n, r0 + kPickRows / 8);
+    int o = woff[blockIdx.x * 8 + w];
+    for (int64_t i0 = r0; i0 < r1; i0 += 32) {
+        const int64_t i = i0 + lane;
+        const int l = i < r1 ? labels[i] : -1;
+        const bool take = l >= 0 && flag[l] != 0;
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        if (take) {
+            const int at = o + __popc(m & ((1u << lane) - 1u));
+            rows[at] = (int32_t)i;
+            lab[at] = l;
+        }
+        o += __popc(m);
+    }
+}
+
+int pick_counts(int64_t n) { return (int)((n + kPickRows - 1) / kPickRows) * 8; }
+
+cudaError_t launch_centroids(Ctx &c, const int32_t *labels, const int32_t *before, float *centers) {
     cudaError_t e;
     const int k = c.k, sb = c.sort_block;
-    label_hist_kernel<<<c.nsb, 256, sizeof(int32_t) * k, c.stream>>>(labels, c.n, k, sb, c.hist);
+    const int32_t *rows = nullptr, *lab = labels;
+    int *n_dev = nullptr;
+    if (before) {
+        const int pb = pick_counts(c.n) / 8;
+        n_dev = c.ll_pick + (size_t)pb * 8;
+        if ((e = cudaMemsetAsync(c.ll_flag, 0, sizeof(int) * (size_t)k, c.stream)) != cudaSuccess) return e;
+        label_flags_kernel<<<(int)std::min<int64_t>((c.n + 255) / 256, (int64_t)c.num_sms * 8), 256, 0, c.stream>>>(
+            labels, before, c.n, c.ll_flag);
+        pick_count_kernel<<<pb, 256, 0, c.stream>>>(labels, c.n, c.ll_flag, c.ll_pick);
+        pick_scan_kernel<<<1, 1024, 0, c.stream>>>(c.ll_pick, pb * 8, n_dev);
+        // (the lists of rows pending and open in an assignment are free between them)
+        pick_rows_kernel<<<pb, 256, 0, c.stream>>>(labels, c.n, c.ll_flag, c.ll_pick, c.ll_pend, c.ll_rows);
+        count_launches(4);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        rows = c.ll_pend;
+        lab = c.ll_rows;
+    }
+    label_hist_kernel<<<c.nsb, 256, sizeof(int32_t) * k, c.stream>>>(lab, c.n, n_dev, k, sb, c.hist);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int nrc = (c.nsb + kScanRows - 1) / kScanRows;
-    column_chunk_kernel<<<dim3((k + 31) / 32, nrc), 256, 0, c.stream>>>(c.hist, c.nsb, k, c.chunk);
+    column_chunk_kernel<<<dim3((k + 31) / 32, nrc), 256, 0, c.stream>>>(c.hist, c.nsb, n_dev, sb, k, c.chunk);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    column_offset_kernel<<<dim3((k + 31) / 32, nrc), 256, 0, c.stream>>>(c.hist, c.nsb, k, c.chunk, nrc, c.base);
+    column_offset_kernel<<<dim3((k + 31) / 32, nrc), 256, 0, c.stream>>>(c.hist, c.nsb, n_dev, sb, k, c.chunk, nrc,
+                                                                             c.base);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     base_scan_kernel<<<1, 1024, 0, c.stream>>>(c.base, k, c.piece);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    scatter_kernel<<<c.nsb, 32, sizeof(int32_t) * k, c.stream>>>(labels, c.n, k, sb, c.hist, c.base, c.perm);
+    scatter_kernel<<<c.nsb, 32, sizeof(int32_t) * k, c.stream>>>(lab, rows, c.n, n_dev, k, sb, c.hist, c.base,
+                                                                  c.perm);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // coordinate pairs need 8-byte aligned rows: d even and X 8-byte aligned
     const int pairs = (c.d % 2 == 0) && (reinterpret_cast<uintptr_t>(c.X) % 8 == 0);

@@ -398,10 +398,13 @@ cudaError_t launch_sum_rows(const float *v, int64_t n, double *partials, int max
 
 // Whether the round passes filter rows by their candidate (see the round filter): the
 // lists take a screening pass over the old candidates, at most cap_total of them, so
-// they have to be few against the rows.
+// they have to be few against the rows, and its 25 launches cost some 60 us a round, which
+// a dense pass of under 4e7 rows x candidates does not (seeding of 30,000 x 64, l = 100:
+// 1.55 ms without, 1.67 with; 100,000 x 64, l = 200: 2.21, 2.13).
 bool round_filter_sizes(const Ctx &c) {
     return c.rounds > 0 && tc::tc_norms_in_epilogue(c.tc_fmt) && c.d % 4 == 0 &&
-           resident_plan(c.cap_round, c.d).parts == 0 && (int64_t)c.cap_total <= c.n / 8;
+           resident_plan(c.cap_round, c.d).parts == 0 && (int64_t)c.cap_total <= c.n / 8 &&
+           (double)c.n * c.cap_round >= 4e7;
 }
 static bool round_filter_usable(const Ctx &c) {
     return c.rf_rows != nullptr && ((reinterpret_cast<uintptr_t>(c.X) | reinterpret_cast<uintptr_t>(c.C)) & 15u) == 0;
@@ -1610,48 +1613,123 @@ constexpr int kStageExtra = 512;   // bytes per warp: 64 open rows, 32 pairs' va
 // steps (the copies are a fixed unrolled sequence of a shuffle and a predicated copy a
 // row; as a loop over rows and pieces they were two thirds of the kernel's instructions)
 template <int RP, int NQ>
-__global__ void __launch_bounds__(256) refine_group_kernel(const float *__restrict__ X, int64_t n, int d,
-                                                          const float *__restrict__ C,
-                                                          const int32_t *__restrict__ glst,
-                                                          const int2 *__restrict__ ghead, float *D2, int32_t *idx,
-                                                          int32_t *open_rows, int *open_cnt, DevState *st,
-                                                          int count_rows) {
-    extern __shared__ __align__(16) float4 gst[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int d4 = d >> 2, ss = stage_stride4(d);
-    float4 *xs = gst + (size_t)wid * (64 * ss + kStageExtra / 16), *cs = xs + 32 * ss;
-    int32_t *ob = reinterpret_cast<int32_t *>(cs + 32 * ss);    // open rows not written yet
-    float *pv = reinterpret_cast<float *>(ob + 64);              // the pairs' values
-    int32_t *pj = reinterpret_cast<int32_t *>(pv + 32);          // and candidates
+__device__ __forceinline__ void stage_rows(float4 *dst, int ss, const float *base, int d4, int row, int lane) {
+    // row: this lane's row of base (negative: none), staged as row `lane` of dst
     constexpr int LW = 32 / RP;   // lanes per copied row
     const int gq = lane / LW, lq = lane % LW;
-    const float4 *C4 = reinterpret_cast<const float4 *>(C) + lq;
-    const int64_t W = (int64_t)gridDim.x * nwarps;
-    const int begin = st->batch_begin;
-    const bool any = st->batch_cnt > 0;   // (an empty batch has no lists and changes nothing)
-    const int64_t nb = (n + 31) / 32;
-    unsigned int settled = 0, listed = 0;
-    int no = 0;
+    const float4 *b4 = reinterpret_cast<const float4 *>(base) + lq;
+    float4 *to = dst + gq * ss + lq;
+#pragma unroll 8
+    for (int r0 = 0; r0 < 32; r0 += RP) {
+        const int o = __shfl_sync(0xffffffffu, row, r0 + gq);
+#pragma unroll
+        for (int u = 0; u < NQ; ++u)
+            if (o >= 0 && lq + u * LW < d4) cp_async16(to + r0 * ss + u * LW, b4 + (int64_t)o * d4 + u * LW);
+    }
+}
+
+// the exact FP32 chain of dist2_fp32 over two staged rows
+__device__ __forceinline__ float stage_dist2(const float4 *x, const float4 *c, int d4) {
+    float v = 0.f;
+#pragma unroll 8
+    for (int p = 0; p < d4; ++p) {
+        const float4 u = x[p], w = c[p];
+        float t;
+        t = __fsub_rn(u.x, w.x); v = __fmaf_rn(t, t, v);
+        t = __fsub_rn(u.y, w.y); v = __fmaf_rn(t, t, v);
+        t = __fsub_rn(u.z, w.z); v = __fmaf_rn(t, t, v);
+        t = __fsub_rn(u.w, w.w); v = __fmaf_rn(t, t, v);
+    }
+    return v;
+}
+
+// Rows of a warp collected for a list in memory and written 32 or more at a time: one
+// atomic on the list's one counter for every block of rows would queue.
+struct RowSink {
+    int32_t *buf;   // 64 entries of the warp's shared memory
+    int n = 0;
+    __device__ __forceinline__ void put(bool take, int32_t row, int lane) {
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        if (take) buf[n + __popc(m & ((1u << lane) - 1u))] = row;
+        n += __popc(m);
+    }
+    __device__ __forceinline__ void flush(int32_t *rows, int *cnt, int lane, bool last) {
+        if (n == 0 || (n < 32 && !last)) return;
+        __syncwarp();
+        int base = 0;
+        if (lane == 0) base = atomicAdd(cnt, n);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        for (int i = lane; i < n; i += 32) rows[base + i] = buf[i];
+        n = 0;
+        __syncwarp();
+    }
+};
+
+struct GroupArgs {
+    const float *X;
+    int64_t n;                  // rows, or null counts below: rows[0 .. *rows_cnt)
+    const int32_t *rows;
+    const int *rows_cnt;
+    int d;
+    const float *C;
+    const int32_t *glst;
+    const int2 *ghead;
+    const int32_t *ref;         // per row, its reference
+    const float *refd2;         // and the exact squared distance to it
+    const float *tau2;          // per reference, squared distance to some center (null: 0)
+    int32_t *open_rows;
+    int *open_cnt;
+    DevState *st;
+    // round
+    float *D2;
+    int32_t *idx;
+    int count_rows;
+    // Lloyd; `own`: the reference is the row's previous center and refd2 its exact distance
+    int own;
+    int32_t *labels;
+    const int32_t *prev;
+    float *dmin, *ub, *lb;
+    int *changed;
+};
+
+template <int MODE, int RP, int NQ>
+__global__ void __launch_bounds__(256) refine_group_kernel(GroupArgs g) {
+    extern __shared__ __align__(16) float4 gst[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int d = g.d, d4 = d >> 2, ss = stage_stride4(d);
+    float4 *xs = gst + (size_t)wid * (64 * ss + kStageExtra / 16), *cs = xs + 32 * ss;
+    RowSink open_sink{reinterpret_cast<int32_t *>(cs + 32 * ss)};
+    float *pv = reinterpret_cast<float *>(open_sink.buf + 64);   // the pairs' values
+    int32_t *pj = reinterpret_cast<int32_t *>(pv + 32);          // and centers
+    const float W = fp32_tie_window(d);
+    const int64_t stride = (int64_t)gridDim.x * nwarps;
+    const int begin = MODE == MODE_ROUND ? g.st->batch_begin : 0;
+    const bool any = MODE != MODE_ROUND || g.st->batch_cnt > 0;   // (an empty batch has no lists, changes nothing)
+    const int64_t n = g.rows ? (int64_t)*g.rows_cnt : g.n, nb = (n + 31) / 32;
+    unsigned int settled = 0, listed = 0, chg = 0;
     int64_t b = (int64_t)blockIdx.x * nwarps + wid;
-    int a = 0;
+    // this lane's row of block b: its number, reference, distance and list head
+    int R = -1, a = 0;
     int2 hd = make_int2(0, 0);
     float dd = 0.f;
     if (any && b < nb && b * 32 + lane < n) {
-        a = idx[b * 32 + lane];
-        dd = D2[b * 32 + lane];
-        hd = __ldg(ghead + a);
+        R = g.rows ? g.rows[b * 32 + lane] : (int)(b * 32 + lane);
+        a = g.ref[R];
+        dd = g.refd2[R];
+        hd = __ldg(g.ghead + a);
     }
-    for (; b < nb; b += W) {   // uniform per warp
-        const int64_t R = b * 32 + lane, Rn = R + 32 * W;
-        const bool valid = any && R < n, next = any && Rn < n;
-        int an = 0;
+    for (; b < nb; b += stride) {   // uniform per warp
+        const int64_t tn = (b + stride) * 32 + lane;
+        int Rn = -1, an = 0;
         float ddn = 0.f;
-        if (next) {
-            an = idx[Rn];
-            ddn = D2[Rn];
+        if (any && tn < n) {
+            Rn = g.rows ? g.rows[tn] : (int)tn;
+            an = g.ref[Rn];
+            ddn = g.refd2[Rn];
         }
-        const bool open = valid && !(dd <= __int_as_float(hd.y));
-        const int total = valid && !open ? hd.x : 0;
+        // (in the first assignment a list holds a center, or it covers nothing)
+        const bool open = R >= 0 && (!(dd <= __int_as_float(hd.y)) || (MODE == MODE_ASSIGN && !g.own && hd.x == 0));
+        const int total = R >= 0 && !open ? hd.x : 0;
         int incl = total;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1661,8 +1739,7 @@ __global__ void __launch_bounds__(256) refine_group_kernel(const float *__restri
         const int excl = incl - total, P = __shfl_sync(0xffffffffu, incl, 31);
         float b1 = FLT_MAX, b2 = FLT_MAX;
         int i1 = INT_MAX, i2 = INT_MAX;
-        const unsigned xm = __ballot_sync(0xffffffffu, total > 0);
-        const float4 *xblk = reinterpret_cast<const float4 *>(X + b * 32 * d);
+        if (MODE == MODE_ASSIGN && g.own && R >= 0 && !open) { b1 = dd; i1 = a; }
         for (int p0 = 0; p0 < P; p0 += 32) {
             const int pi = p0 + lane;
             // the pair's row: the first whose inclusive count exceeds pi
@@ -1672,45 +1749,14 @@ __global__ void __launch_bounds__(256) refine_group_kernel(const float *__restri
                 if (__shfl_sync(0xffffffffu, incl, r + o - 1) <= pi) r += o;
             const int ar = __shfl_sync(0xffffffffu, a, r), er = pi - __shfl_sync(0xffffffffu, excl, r);
             int j = -1;
-            if (pi < P) j = begin + __ldg(glst + (size_t)ar * 4 * tc::kListSlots + er);
-            if (p0 == 0) {
-#pragma unroll 8
-                for (int r0 = 0; r0 < 32; r0 += RP) {
-                    const int rr = r0 + gq;
-                    const bool on = (xm >> rr) & 1u;
-#pragma unroll
-                    for (int u = 0; u < NQ; ++u)
-                        if (on && lq + u * LW < d4)
-                            cp_async16(xs + rr * ss + lq + u * LW, xblk + rr * d4 + lq + u * LW);
-                }
-            }
-            const int off = j >= 0 ? j * d4 : -1;
-#pragma unroll 8
-            for (int r0 = 0; r0 < 32; r0 += RP) {
-                const int rr = r0 + gq;
-                const int o = __shfl_sync(0xffffffffu, off, rr);
-#pragma unroll
-                for (int u = 0; u < NQ; ++u)
-                    if (o >= 0 && lq + u * LW < d4) cp_async16(cs + rr * ss + lq + u * LW, C4 + o + u * LW);
-            }
+            if (pi < P) j = begin + __ldg(g.glst + (size_t)ar * 4 * tc::kListSlots + er);
+            if (p0 == 0) stage_rows<RP, NQ>(xs, ss, g.X, d4, total > 0 ? R : -1, lane);
+            stage_rows<RP, NQ>(cs, ss, g.C, d4, j, lane);
             cp_async_commit();
             cp_async_wait<0>();
             __syncwarp();
-            if (j >= 0) {
-                float v = 0.f;
-                const float4 *x = xs + r * ss, *c = cs + lane * ss;
-#pragma unroll 8
-                for (int p = 0; p < d4; ++p) {
-                    const float4 u = x[p], w = c[p];
-                    float t;
-                    t = __fsub_rn(u.x, w.x); v = __fmaf_rn(t, t, v);
-                    t = __fsub_rn(u.y, w.y); v = __fmaf_rn(t, t, v);
-                    t = __fsub_rn(u.z, w.z); v = __fmaf_rn(t, t, v);
-                    t = __fsub_rn(u.w, w.w); v = __fmaf_rn(t, t, v);
-                }
-                pv[lane] = v;
-                pj[lane] = j;
-            }
+            pj[lane] = j;
+            if (j >= 0) pv[lane] = stage_dist2(xs + r * ss, cs + lane * ss, d4);
             __syncwarp();   // the values are there; the staged rows are read
             for (int q = max(excl, p0); q < min(incl, p0 + 32); ++q) {
                 const float v = pv[q - p0];
@@ -1722,38 +1768,51 @@ __global__ void __launch_bounds__(256) refine_group_kernel(const float *__restri
             }
             __syncwarp();
         }
-        const int2 hdn = next ? __ldg(ghead + an) : make_int2(0, 0);
+        const int2 hdn = Rn >= 0 ? __ldg(g.ghead + an) : make_int2(0, 0);
         if (i1 != INT_MAX) {
             if (i2 == INT_MAX) { i2 = -1; b2 = FLT_MAX; }
-            decide_top2<MODE_ROUND>(X, d, C, R, b1, i1, b2, i2, D2, idx, nullptr, nullptr, nullptr, &st->argmin_fp64,
-                                    &st->argmin_wide);
+            if (MODE == MODE_ROUND) {
+                decide_top2<MODE_ROUND>(g.X, d, g.C, R, b1, i1, b2, i2, g.D2, g.idx, nullptr, nullptr, nullptr,
+                                        &g.st->argmin_fp64, &g.st->argmin_wide);
+            } else {
+                chg += decide_top2<MODE_ASSIGN>(g.X, d, g.C, R, b1, i1, b2, i2, nullptr, nullptr, g.labels, g.prev,
+                                                g.dmin, &g.st->argmin_fp64, &g.st->argmin_wide);
+                if (g.lb) {
+                    // the exact runner-up, and for a center off the list its distance to the
+                    // reference less the row's (real distances: FP32 ones within W of them)
+                    const bool fst = g.labels[R] == i1;
+                    g.ub[R] = bound_upper(fst ? b1 : b2, W);
+                    const float reach = 2.f * sqrtf(__int_as_float(hd.y)) + (g.tau2 ? sqrtf(g.tau2[a]) : 0.f);
+                    const float off = reach * (1.f - 1e-6f) - bound_upper(dd, W);
+                    const float run = fst ? b2 : b1;
+                    const float l2 = run < FLT_MAX ? sqrtf(run * (1.f - 2.f * W)) * (1.f - 1e-6f) : FLT_MAX;
+                    g.lb[R] = fmaxf(0.f, fminf(l2, off));
+                }
+            }
         }
-        // open rows are collected and written 32 or more at a time: one atomic on the one
-        // counter for every block of rows would queue
-        const unsigned m = __ballot_sync(0xffffffffu, open);
-        if (open) ob[no + __popc(m & ((1u << lane) - 1u))] = (int32_t)R;
-        no += __popc(m);
-        if (no > 0 && (no >= 32 || b + W >= nb)) {
-            __syncwarp();
-            int base = 0;
-            if (lane == 0) base = atomicAdd(open_cnt, no);
-            base = __shfl_sync(0xffffffffu, base, 0);
-            for (int i = lane; i < no; i += 32) open_rows[base + i] = ob[i];
-            no = 0;
-            __syncwarp();
-        }
-        if (lane == 0) settled += (unsigned int)min((int64_t)32, n - b * 32) - __popc(m);
+        open_sink.put(open, R, lane);
+        open_sink.flush(g.open_rows, g.open_cnt, lane, b + stride >= nb);
+        settled += (unsigned int)(R >= 0 && !open) + (unsigned int)(!any && b * 32 + lane < n);
         listed += (unsigned int)(total > 0);
+        R = Rn;
         a = an;
         dd = ddn;
         hd = hdn;
     }
+    settled = __reduce_add_sync(0xffffffffu, settled);
     listed = __reduce_add_sync(0xffffffffu, listed);
+    if (MODE == MODE_ASSIGN) chg = __reduce_add_sync(0xffffffffu, chg);
     if (lane == 0) {   // the rows settled here (the dense pass counts the open ones)
-        if (settled && count_rows) atomicAdd(&st->screen_rows, (unsigned long long)settled);
-        if (listed) {
-            atomicAdd(&st->screen_fallback, (unsigned long long)listed);
-            atomicAdd(&st->screen_listed, (unsigned long long)listed);
+        if (MODE == MODE_ROUND) {
+            if (settled && g.count_rows) atomicAdd(&g.st->screen_rows, (unsigned long long)settled);
+            if (listed) {
+                atomicAdd(&g.st->screen_fallback, (unsigned long long)listed);
+                atomicAdd(&g.st->screen_listed, (unsigned long long)listed);
+            }
+        } else {
+            if (settled && g.own) atomicAdd(&g.st->lloyd_settled, (unsigned long long)settled);
+            if (settled && !g.own) atomicAdd(&g.st->screen_rows, (unsigned long long)settled);
+            if (chg && g.changed) atomicAdd(g.changed, (int)chg);
         }
     }
 }
@@ -1765,26 +1824,26 @@ int stage_warps(int d) {
 }
 size_t stage_smem_bytes(int d) { return (size_t)stage_warps(d) * (64 * 16 * stage_stride4(d) + kStageExtra); }
 
-template <int RP, int NQ>
-static cudaError_t launch_refine_group_as(Ctx &c, const float *C) {
+// a kernel of the staged kind over n rows: persistent, two CTAs an SM
+template <typename K, typename A>
+static cudaError_t launch_staged(K kern, const Ctx &c, int64_t n, const A &args) {
     const size_t smem = stage_smem_bytes(c.d);
-    cudaError_t e = cudaFuncSetAttribute(refine_group_kernel<RP, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int sw = stage_warps(c.d);
-    const int grid = (int)std::min<int64_t>((c.n + 32 * sw - 1) / (32 * sw), 2 * (int64_t)c.num_sms);
-    refine_group_kernel<RP, NQ><<<grid, 32 * sw, smem, c.stream>>>(c.X, c.n, c.d, C, c.rf_lst, c.rf_head, c.D2, c.idx,
-                                                                   c.rf_rows, c.rf_cnt, c.st, c.round_part == 0);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n + 32 * sw - 1) / (32 * sw), 2 * (int64_t)c.num_sms));
+    kern<<<grid, 32 * sw, smem, c.stream>>>(args);
     count_launches(1);
     return cudaGetLastError();
 }
-static cudaError_t launch_refine_group(Ctx &c, const float *C) {
+template <int MODE>
+static cudaError_t launch_refine_group(const Ctx &c, const GroupArgs &g) {
     const int d4 = c.d >> 2;
-    if (d4 > 32) return launch_refine_group_as<1, 2>(c, C);   // (d <= 188)
-    if (d4 > 16) return launch_refine_group_as<1, 1>(c, C);
-    if (d4 > 8) return launch_refine_group_as<2, 1>(c, C);
-    if (d4 > 4) return launch_refine_group_as<4, 1>(c, C);
-    return launch_refine_group_as<8, 1>(c, C);
+    if (d4 > 32) return launch_staged(refine_group_kernel<MODE, 1, 2>, c, c.n, g);   // (d <= 188)
+    if (d4 > 16) return launch_staged(refine_group_kernel<MODE, 1, 1>, c, c.n, g);
+    if (d4 > 8) return launch_staged(refine_group_kernel<MODE, 2, 1>, c, c.n, g);
+    if (d4 > 4) return launch_staged(refine_group_kernel<MODE, 4, 1>, c, c.n, g);
+    return launch_staged(refine_group_kernel<MODE, 8, 1>, c, c.n, g);
 }
 
 // A distance pass on the tensor cores.  rows / rows_cnt (direct refine only): the pass
@@ -1794,7 +1853,8 @@ cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_
                            int *changed, float *dmin, int timing_cls, const int32_t *rows, const int *rows_cnt) {
     cudaError_t e;
     const int fmt = c.tc_fmt;
-    if ((e = tc::launch_prep_centers(C, c.d, fmt, c.st, k, mode_round, mode_round ? c.cap_round : k, c.tc_anchor,
+    if (!c.tc_prepared &&
+        (e = tc::launch_prep_centers(C, c.d, fmt, c.st, k, mode_round, mode_round ? c.cap_round : k, c.tc_anchor,
                                      c.tc_img, c.tc_ncol, c.tc_tscale, c.tc_cmax, c.stream)) != cudaSuccess)
         return e;
     if ((e = cudaMemsetAsync(c.fix_cnt, 0, sizeof(int), c.stream)) != cudaSuccess) return e;
@@ -1838,10 +1898,14 @@ cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_
         pf.lst = c.tc_lst; pf.lcnt = c.tc_lcnt;
         const tc::ListBufs lb{c.cap_total, c.tc_cimg, c.tc_cscale, c.tc_thr, c.rf_rad2, c.rf_num, c.rf_lst, c.rf_head,
                               c.rf_lcnt};
-        if ((e = tc::launch_candidate_lists(pf, lb, c.cand, &c.st->batch_begin, sb.ep, sb.en, sb.ec, c.num_sms,
+        if ((e = tc::launch_reference_lists(pf, 1, lb, c.cand, &c.st->batch_begin, nullptr, sb.ep, sb.en, sb.ec, c.num_sms,
                                             c.stream)) != cudaSuccess)
             return e;
-        if ((e = launch_refine_group(c, C)) != cudaSuccess) return e;
+        GroupArgs ga{};
+        ga.X = c.X; ga.n = c.n; ga.d = c.d; ga.C = C; ga.glst = c.rf_lst; ga.ghead = c.rf_head; ga.ref = c.idx;
+        ga.refd2 = c.D2; ga.open_rows = c.rf_rows; ga.open_cnt = c.rf_cnt; ga.st = c.st; ga.D2 = c.D2; ga.idx = c.idx;
+        ga.count_rows = c.round_part == 0;
+        if ((e = launch_refine_group<MODE_ROUND>(c, ga)) != cudaSuccess) return e;
         rows = c.rf_rows;
         rows_cnt = c.rf_cnt;
     }
@@ -2056,59 +2120,134 @@ __global__ void __launch_bounds__(1024) lloyd_drift_other_kernel(const float *__
     for (int c = threadIdx.x; c < k; c += blockDim.x) other[c] = c == i1 ? m2 : m1;
 }
 
-// The bounds test for every row (in the order given: rows sorted by their previous
-// label, so neighbouring threads read the same center row).  A row it settles gets
-// its label, the exact FP32 d^2 to the moved center (bit-identical to the refine's
-// chains) and fresh bounds; the others are listed for the compact pass (with l = 0
-// until that pass certifies them again).
-__global__ void __launch_bounds__(256) lloyd_bounds_kernel(const float *__restrict__ X, int64_t n, int d,
-                                                           const float *__restrict__ C,
-                                                           const int32_t *__restrict__ prev,
-                                                           const int32_t *__restrict__ order, int32_t *labels,
-                                                           float *dmin, float *ubd, float *lbd,
-                                                           const float *__restrict__ drift,
-                                                           const float *__restrict__ other, int32_t *rows, int *cnt,
-                                                           unsigned long long *settled) {
-    const int64_t T = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = T < n;
-    const int64_t R = order && valid ? (int64_t)order[T] : T;
-    const int lane = threadIdx.x & 31;
-    bool keep = false;
-    if (valid) {
-        const int a = prev[R];
-        const float u = ubd[R] + drift[a];
-        const float l = lbd[R] - other[a];
-        keep = l > 0.f && u < l;
-        if (keep) {
-            const float4 *x4 = reinterpret_cast<const float4 *>(X + R * d);
-            const float4 *c4 = reinterpret_cast<const float4 *>(C + (int64_t)a * d);
-            float v = 0.f;
-#pragma unroll 4
-            for (int p = 0; p < (d >> 2); ++p) {
-                const float4 x = __ldg(x4 + p), c = __ldg(c4 + p);
-                float t;
-                t = __fsub_rn(x.x, c.x); v = __fmaf_rn(t, t, v);
-                t = __fsub_rn(x.y, c.y); v = __fmaf_rn(t, t, v);
-                t = __fsub_rn(x.z, c.z); v = __fmaf_rn(t, t, v);
-                t = __fsub_rn(x.w, c.w); v = __fmaf_rn(t, t, v);
+// The bounds test, in two kernels.  A row whose center did not move keeps its exact d^2
+// and its upper bound: lloyd_still_kernel settles it, or lists it as pending, without a
+// look at X (16 bytes of state read a row), and lists the rows of moved centers.  Those get
+// the exact FP32 d^2 to the moved center (the chain of the refine, rows and centers staged
+// by whole warps) and with it a tight upper bound for the test (lloyd_moved_kernel).
+// Settled rows get their label, distance and bounds; a pending one has l = 0 until a pass
+// certifies it again, and its distance goes into its center's radius for the lists.
+// 1e7 x 128, k = 10,000, 4% of the centers moving: 1.9 ms an assignment as one kernel with
+// a row a thread, 0.8 staged over all rows, 0.13 + 0.1 so.
+struct BoundsArgs {
+    const float *X;
+    int64_t n;
+    int d;
+    const float *C;
+    const int32_t *prev;
+    int32_t *labels;
+    float *dmin, *ub, *lb;
+    const float *drift, *other;
+    unsigned int *rad2;   // per center (null: not wanted)
+    int32_t *moved;       // rows of moved centers
+    int *moved_cnt;
+    int32_t *rows;        // pending rows
+    int *cnt;
+    unsigned long long *settled;
+
+    __device__ __forceinline__ void radius(int a, float v) const {
+        if (!rad2) return;
+        unsigned int *r = rad2 + a;
+        const unsigned int bits = __float_as_uint(v);
+        if (bits > *reinterpret_cast<volatile unsigned int *>(r)) atomicMax(r, bits);
+    }
+};
+
+__global__ void __launch_bounds__(256) lloyd_still_kernel(BoundsArgs g) {
+    __shared__ int32_t buf[16][64];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    RowSink moved{buf[wid]}, pend{buf[8 + wid]};
+    const int64_t nb = (g.n + 31) / 32, stride = (int64_t)gridDim.x * 8;
+    unsigned int settled = 0;
+    for (int64_t b = (int64_t)blockIdx.x * 8 + wid; b < nb; b += stride) {   // uniform per warp
+        const int64_t R = b * 32 + lane;
+        bool mv = false, pd = false;
+        if (R < g.n) {
+            const int a = g.prev[R];
+            mv = g.drift[a] != 0.f;
+            g.labels[R] = a;
+            if (!mv) {
+                const float lo = g.lb[R] - g.other[a];
+                pd = !(lo > 0.f && g.ub[R] < lo);
+                g.lb[R] = pd ? 0.f : lo;
+                if (pd) g.radius(a, g.dmin[R]);
+                settled += (unsigned int)!pd;
             }
-            labels[R] = a;
-            dmin[R] = v;
-            ubd[R] = bound_upper(v, fp32_tie_window(d));
-            lbd[R] = l;
-        } else {
-            lbd[R] = 0.f;
         }
+        moved.put(mv, (int32_t)R, lane);
+        pend.put(pd, (int32_t)R, lane);
+        const bool last = b + stride >= nb;
+        moved.flush(g.moved, g.moved_cnt, lane, last);
+        pend.flush(g.rows, g.cnt, lane, last);
     }
-    const unsigned m = __ballot_sync(0xffffffffu, valid && !keep);
-    if (m) {
-        int base = 0;
-        if (lane == 0) base = atomicAdd(cnt, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (valid && !keep) rows[base + __popc(m & ((1u << lane) - 1u))] = (int32_t)R;
+    settled = __reduce_add_sync(0xffffffffu, settled);
+    if (lane == 0 && settled) atomicAdd(g.settled, (unsigned long long)settled);
+}
+
+template <int RP, int NQ>
+__global__ void __launch_bounds__(256) lloyd_moved_kernel(BoundsArgs g) {
+    extern __shared__ __align__(16) float4 gst[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int d = g.d, d4 = d >> 2, ss = stage_stride4(d);
+    float4 *xs = gst + (size_t)wid * (64 * ss + kStageExtra / 16), *cs = xs + 32 * ss;
+    RowSink sink{reinterpret_cast<int32_t *>(cs + 32 * ss)};
+    const float W = fp32_tie_window(d);
+    const int n = *g.moved_cnt, nb = (n + 31) / 32, stride = gridDim.x * nwarps;
+    unsigned int settled = 0;
+    int b = blockIdx.x * nwarps + wid;
+    // this lane's row of block b
+    int R = -1, a = -1;
+    if (b < nb && b * 32 + lane < n) {
+        R = g.moved[b * 32 + lane];
+        a = g.prev[R];
     }
-    const unsigned kp = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0 && kp) atomicAdd(settled, (unsigned long long)__popc(kp));
+    for (; b < nb; b += stride) {   // uniform per warp
+        stage_rows<RP, NQ>(xs, ss, g.X, d4, R, lane);
+        stage_rows<RP, NQ>(cs, ss, g.C, d4, a, lane);
+        cp_async_commit();
+        // while the copies are in flight: this row's bound, the next block's rows
+        const int cr = R, ca = a;
+        const float lo = cr >= 0 ? g.lb[cr] - g.other[ca] : 0.f;
+        const int tn = (b + stride) * 32 + lane;
+        R = a = -1;
+        if (b + stride < nb && tn < n) {
+            R = g.moved[tn];
+            a = g.prev[R];
+        }
+        cp_async_wait<0>();
+        __syncwarp();
+        bool keep = false;
+        if (cr >= 0) {
+            const float v = stage_dist2(xs + lane * ss, cs + lane * ss, d4);
+            const float u = bound_upper(v, W);
+            keep = lo > 0.f && u < lo;
+            g.dmin[cr] = v;
+            g.ub[cr] = u;
+            g.lb[cr] = keep ? lo : 0.f;
+            if (!keep) g.radius(ca, v);
+        }
+        __syncwarp();   // the staged rows are read
+        sink.put(cr >= 0 && !keep, cr, lane);
+        sink.flush(g.rows, g.cnt, lane, b + stride >= nb);
+        settled += (unsigned int)keep;
+    }
+    settled = __reduce_add_sync(0xffffffffu, settled);
+    if (lane == 0 && settled) atomicAdd(g.settled, (unsigned long long)settled);
+}
+
+// tau2: the squared FP32 distance from reference i (row i of A) to the nearest of the
+// screened group of four centers at cand1[i] (any center serves), +inf without one
+__global__ void __launch_bounds__(256) reference_tau_kernel(const float *__restrict__ A, const int *cnt, int d,
+                                                           const float *__restrict__ C, int k,
+                                                           const int32_t *__restrict__ cand1,
+                                                           float *__restrict__ tau2) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= *cnt) return;
+    const int j = cand1[i];
+    float best = __int_as_float(0x7f800000);
+    if (j >= 0)
+        for (int u = j; u < min(j + 4, k); ++u) best = fminf(best, dist2_fp32(A + (int64_t)i * d, C + (int64_t)u * d, d));
+    tau2[i] = best;
 }
 
 bool lloyd_bounds_usable(const Ctx &c, const float *C) {
@@ -2118,24 +2257,144 @@ bool lloyd_bounds_usable(const Ctx &c, const float *C) {
            ((reinterpret_cast<uintptr_t>(c.X) | reinterpret_cast<uintptr_t>(C)) & 15u) == 0;
 }
 
-// one Lloyd assignment after a centroid update, using the bounds: the rows they
-// settle, then a compact tensor pass over the rest
+// Whether the lists around references can take the place of the dense passes: the
+// references have to be few against the rows, and the rows x centers of a dense pass
+// have to outweigh the lists' 18 launches an assignment (10 updates: 300,000 x 128,
+// k = 1,000 4.3 ms without, 4.6 with; 1,000,000 x 96, k = 2,000 8.2 and 6.3).
+bool lloyd_lists_usable(const Ctx &c) {
+    return c.precision != KMPAR_FP32 && c.tc_cimg && tc::tc_norms_in_epilogue(c.tc_fmt) && c.d % 4 == 0 &&
+           resident_plan(c.k, c.d).parts == 0 && (int64_t)std::max(c.cap_total, c.k) <= c.n / 8 &&
+           (double)c.n * c.k >= 1e9;
+}
+
+__global__ void set_int_kernel(int *p, int v) { *p = v; }
+
+static cudaError_t launch_bounds(const Ctx &c, const BoundsArgs &g) {
+    const int grid = (int)std::min<int64_t>((c.n + 255) / 256, (int64_t)c.num_sms * 8);
+    lloyd_still_kernel<<<grid, 256, 0, c.stream>>>(g);
+    count_launches(1);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int d4 = c.d >> 2;
+    if (d4 > 32) return launch_staged(lloyd_moved_kernel<1, 2>, c, c.n, g);
+    if (d4 > 16) return launch_staged(lloyd_moved_kernel<1, 1>, c, c.n, g);
+    if (d4 > 8) return launch_staged(lloyd_moved_kernel<2, 1>, c, c.n, g);
+    if (d4 > 4) return launch_staged(lloyd_moved_kernel<4, 1>, c, c.n, g);
+    return launch_staged(lloyd_moved_kernel<8, 1>, c, c.n, g);
+}
+
+// center tiles of the assignment's centers, the pass parameters and bounds with them
+static cudaError_t lloyd_prepare(Ctx &c, const float *C, tc::TcParams &p, ScreenBound &sb) {
+    p = tc::TcParams{};
+    p.X = c.X; p.n = c.n; p.d = c.d; p.fmt = c.tc_fmt;
+    p.Cf = C; p.cnt = c.k; p.st = c.st; p.bimg = c.tc_img; p.ncol = c.tc_ncol; p.tscale = c.tc_tscale;
+    p.cmax_bits = c.tc_cmax; p.cand1 = c.cand1; p.v2 = c.tc_v2; p.err = c.tc_err; p.group = 4;
+    p.lst = c.tc_lst; p.lcnt = c.tc_lcnt;
+    sb = ScreenBound{};
+    tc::tc_bound(c.d, c.tc_fmt, &sb.ep, &sb.en, &sb.ec);
+    return tc::launch_prep_centers(C, c.d, c.tc_fmt, c.st, c.k, 0, c.k, c.tc_anchor, c.tc_img, c.tc_ncol, c.tc_tscale,
+                                   c.tc_cmax, c.stream);
+}
+
+static tc::ListBufs lloyd_list_bufs(const Ctx &c) {
+    return tc::ListBufs{std::max(c.cap_total, c.k), c.tc_cimg, c.tc_cscale, c.tc_thr, c.ll_rad2, c.ll_num, c.ll_lst,
+                        c.ll_head, c.ll_lcnt};
+}
+
+// the dense compact pass over the rows the lists leave open, with the centers prepared
+static cudaError_t lloyd_open_pass(Ctx &c, const float *C, int32_t *labels, const int32_t *prev, int *changed,
+                                   float *dmin) {
+    c.tc_prepared = true;
+    const cudaError_t e = launch_tc_pass(c, 0, C, c.k, labels, prev, changed, dmin, -1, c.ll_rows, c.ll_cnt);
+    c.tc_prepared = false;
+    return e;
+}
+
+// The first assignment.  Every row is within D(x) of its candidate, and a candidate
+// within tau of some center, so the row's nearest center is within 2 D(x) + tau of its
+// candidate: centers are listed around the candidates, rows examine their candidate's
+// list, and the dense pass covers the rows beyond the lists.  1e7 x 128, k = 10,000:
+// 24 ms dense, 3.5 ms.
+cudaError_t launch_lloyd_first_pass(Ctx &c, const float *C, int32_t *labels, int *changed, float *dmin) {
+    cudaError_t e;
+    tc::TcParams p;
+    ScreenBound sb;
+    if ((e = lloyd_prepare(c, C, p, sb)) != cudaSuccess) return e;
+    const tc::ListBufs lb = lloyd_list_bufs(c);
+    if ((e = cudaMemsetAsync(c.ll_rad2, 0, sizeof(unsigned int) * (size_t)lb.cap, c.stream)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(c.ll_cnt, 0, sizeof(int), c.stream)) != cudaSuccess) return e;
+    candidate_radius_kernel<<<c.num_sms * 8, 256, 0, c.stream>>>(c.D2, c.idx, c.n, c.ll_rad2);
+    count_launches(1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // tau: the candidates' best screened groups
+    const int *m = &c.st->m;
+    if ((e = tc::launch_gather_rows(c.tc_ximg, c.tc_xscale, c.d, c.tc_fmt, c.cand, m, c.D2, c.tc_xnorm, c.tc_cmax, sb.ep,
+                                    sb.en, sb.ec, c.tc_cimg, c.tc_cscale, c.tc_thr, c.num_sms * 8, c.stream)) !=
+        cudaSuccess)
+        return e;
+    tc::TcParams pt = p;
+    pt.ximg = c.tc_cimg; pt.xscale = c.tc_cscale; pt.nrows_dev = m;
+    if ((e = tc::launch_nearest_tc(pt, 0, tc::EPI_PAIR, c.num_sms, c.stream)) != cudaSuccess) return e;
+    reference_tau_kernel<<<(c.cap_total + 255) / 256, 256, 0, c.stream>>>(c.C, m, c.d, C, c.k, c.cand1, c.ll_tau2);
+    count_launches(1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    p.ximg = c.tc_ximg; p.xnorm = c.tc_xnorm; p.xscale = c.tc_xscale;
+    if ((e = tc::launch_reference_lists(p, 0, lb, c.cand, m, c.ll_tau2, sb.ep, sb.en, sb.ec, c.num_sms, c.stream)) !=
+        cudaSuccess)
+        return e;
+    GroupArgs g{};
+    g.X = c.X; g.n = c.n; g.d = c.d; g.C = C; g.glst = c.ll_lst; g.ghead = c.ll_head; g.ref = c.idx; g.refd2 = c.D2;
+    g.tau2 = c.ll_tau2; g.open_rows = c.ll_rows; g.open_cnt = c.ll_cnt; g.st = c.st; g.labels = labels; g.dmin = dmin;
+    g.ub = c.ll_ub; g.lb = c.ll_lb;
+    if ((e = launch_refine_group<MODE_ASSIGN>(c, g)) != cudaSuccess) return e;
+    return lloyd_open_pass(c, C, labels, nullptr, changed, dmin);
+}
+
+// One assignment after a centroid update: the rows the bounds settle; for the others the
+// exact distances to the centers listed within twice their distance of their own center
+// (an open row of a mixture has one or two), and a dense compact pass over the rows
+// beyond the lists.
 cudaError_t launch_lloyd_bounded_pass(Ctx &c, const float *C, int32_t *labels, const int32_t *prev, int *changed,
                                       float *dmin) {
     cudaError_t e;
     const int k = c.k;
+    const bool lists = lloyd_lists_usable(c);
     lloyd_drift_kernel<<<(k + 7) / 8, 256, 0, c.stream>>>(C, c.ll_cold, k, c.d, c.ll_drift);
     lloyd_drift_other_kernel<<<1, 1024, 0, c.stream>>>(c.ll_drift, k, c.ll_other);
     count_launches(2);
-    if ((e = cudaMemsetAsync(c.ll_cnt, 0, sizeof(int), c.stream)) != cudaSuccess) return e;
-    // rows in storage order: X streams from HBM, the settled rows' center rows (k x d,
-    // a few MB) come from L2
-    lloyd_bounds_kernel<<<(int)((c.n + 255) / 256), 256, 0, c.stream>>>(
-        c.X, c.n, c.d, C, prev, nullptr, labels, dmin, c.ll_ub, c.ll_lb, c.ll_drift, c.ll_other, c.ll_rows, c.ll_cnt,
-        &c.st->lloyd_settled);
+    // (ll_cnt: the open rows, then the rows of moved centers)
+    if ((e = cudaMemsetAsync(c.ll_cnt, 0, 2 * sizeof(int), c.stream)) != cudaSuccess) return e;
+    int *pend_cnt = lists ? c.ll_lcnt + tc::kListLevels + 1 : c.ll_cnt;
+    if (lists) {
+        if ((e = cudaMemsetAsync(c.ll_rad2, 0, sizeof(unsigned int) * (size_t)k, c.stream)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(pend_cnt, 0, sizeof(int), c.stream)) != cudaSuccess) return e;
+    }
+    BoundsArgs ba{};
+    ba.X = c.X; ba.n = c.n; ba.d = c.d; ba.C = C; ba.prev = prev; ba.labels = labels; ba.dmin = dmin; ba.ub = c.ll_ub;
+    ba.lb = c.ll_lb; ba.drift = c.ll_drift; ba.other = c.ll_other; ba.rad2 = lists ? c.ll_rad2 : nullptr;
+    ba.moved = c.perm; ba.moved_cnt = c.ll_cnt + 1;   // (the centroids are made: their sort is free)
+    ba.rows = lists ? c.ll_pend : c.ll_rows; ba.cnt = pend_cnt; ba.settled = &c.st->lloyd_settled;
+    if ((e = launch_bounds(c, ba)) != cudaSuccess) return e;
+    if (!lists) return launch_tc_pass(c, 0, C, k, labels, prev, changed, dmin, -1, c.ll_rows, c.ll_cnt);
+    tc::TcParams p;
+    ScreenBound sb;
+    if ((e = lloyd_prepare(c, C, p, sb)) != cudaSuccess) return e;
+    if ((e = tc::launch_prep_points(C, k, c.d, c.tc_fmt, c.tc_anchor, c.ll_img, c.ll_xnorm, c.ll_xscale, c.stream)) !=
+        cudaSuccess)
+        return e;
+    int *kdev = c.ll_lcnt + tc::kListLevels;
+    set_int_kernel<<<1, 1, 0, c.stream>>>(kdev, k);
     count_launches(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return launch_tc_pass(c, 0, C, k, labels, prev, changed, dmin, -1, c.ll_rows, c.ll_cnt);
+    p.ximg = c.ll_img; p.xnorm = c.ll_xnorm; p.xscale = c.ll_xscale;
+    if ((e = tc::launch_reference_lists(p, 0, lloyd_list_bufs(c), nullptr, kdev, nullptr, sb.ep, sb.en, sb.ec, c.num_sms,
+                                        c.stream)) != cudaSuccess)
+        return e;
+    GroupArgs g{};
+    g.X = c.X; g.n = c.n; g.rows = c.ll_pend; g.rows_cnt = pend_cnt; g.d = c.d; g.C = C; g.glst = c.ll_lst;
+    g.ghead = c.ll_head; g.ref = prev; g.refd2 = dmin; g.own = 1; g.open_rows = c.ll_rows; g.open_cnt = c.ll_cnt;
+    g.st = c.st; g.labels = labels; g.prev = prev; g.dmin = dmin; g.ub = c.ll_ub; g.lb = c.ll_lb; g.changed = changed;
+    if ((e = launch_refine_group<MODE_ASSIGN>(c, g)) != cudaSuccess) return e;
+    return lloyd_open_pass(c, C, labels, prev, changed, dmin);
 }
 
 }  // namespace kmp

@@ -20,16 +20,16 @@ def _far(n, d, seed):
 
 
 CASES = [
-    # name, rows, k, l, rounds, precision
-    ("d4", lambda: datagen.gauss_mixture(30011, 4, 40, 100.0, seed=1), 40, 80.0, 4, "fp8"),
-    ("d16_no_separation", lambda: datagen.uniform_box(20001, 16, seed=2), 30, 200.0, 4, "fp8"),
-    ("d20", lambda: datagen.gauss_mixture(25000, 20, 100, 4.0, seed=3), 100, 150.0, 5, "fp8"),
+    # name, rows, k, l, rounds, precision (rows x draws a round are enough for the filter)
+    ("d4", lambda: datagen.gauss_mixture(60011, 4, 40, 100.0, seed=1), 300, 600.0, 4, "fp8"),
+    ("d16_no_separation", lambda: datagen.uniform_box(60001, 16, seed=2), 300, 600.0, 4, "fp8"),
+    ("d20", lambda: datagen.gauss_mixture(80000, 20, 100, 4.0, seed=3), 100, 450.0, 5, "fp8"),
     ("d64_bf16", lambda: datagen.gauss_mixture(60000, 64, 300, 10.0, seed=4), 300, 700.0, 5, "bf16"),
-    ("d96_far_and_copies", lambda: _far(40000, 96, 5), 60, 300.0, 5, "fp8"),
-    ("d132", lambda: datagen.gauss_mixture(20033, 132, 50, 100.0, seed=6), 50, 100.0, 4, "fp8"),
-    ("d188", lambda: datagen.gauss_mixture(15000, 188, 30, 100.0, seed=7), 30, 60.0, 3, "fp8"),
+    ("d96_far_and_copies", lambda: _far(90000, 96, 5), 60, 300.0, 5, "fp8"),
+    ("d132", lambda: datagen.gauss_mixture(50033, 132, 50, 100.0, seed=6), 250, 600.0, 4, "fp8"),
+    ("d188", lambda: datagen.gauss_mixture(50000, 188, 30, 100.0, seed=7), 200, 600.0, 3, "fp8"),
     ("d128_parts", lambda: datagen.gauss_mixture(400_001, 128, 5000, 100.0, seed=8), 5000, 15000.0, 3, "bf16"),
-    ("d64_all_drawn", lambda: np.repeat(datagen.uniform_box(40, 64, seed=9), 500, 0), 20, 200.0, 4, "bf16"),
+    ("d64_all_drawn", lambda: np.repeat(datagen.uniform_box(40, 64, seed=9), 2000, 0), 20, 300.0, 4, "bf16"),
 ]
 
 
