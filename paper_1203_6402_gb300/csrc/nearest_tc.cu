@@ -242,56 +242,81 @@ __global__ void __launch_bounds__(256) prep_centers_ne_kernel(const float *__res
     }
 }
 
-// One CTA per 128-row tile of the A image [row tile][katom][128 rows][128 B]: the
-// tile's rows (contiguous in X) come into shared memory with coalesced loads; then
-// eight consecutive threads build the eight 16-byte chunks of one row segment of an
-// atom (position p of row r holds logical chunk p ^ (r & 7)), so the stores are
-// coalesced too; thread r sums ||x'||^2 of row r (FP32, ascending; x' = x - anchor)
-// and, for FP8, finds the row's largest |x'_q| and its power-of-two scale s_x.
-__global__ void __launch_bounds__(128) prep_points_kernel(const float *__restrict__ X, int64_t n, int64_t n_pad, int d,
-                                                          int fmt, int KA, const float *__restrict__ anchor,
-                                                          uint8_t *__restrict__ img, float *__restrict__ xnorm,
-                                                          float *__restrict__ xscale) {
-    extern __shared__ float xsm[];   // BM x d moved rows
-    __shared__ float inv_s[BM];
-    const int64_t ntile = n_pad / BM;
-    for (int64_t t = blockIdx.x; t < ntile; t += gridDim.x) {
-        const int64_t r0 = t * BM;
-        const int nr = (int)max((int64_t)0, min((int64_t)BM, n - r0));
-        __syncthreads();   // the previous tile's readers are done
-        for (int f = threadIdx.x; f < nr * d; f += BM) xsm[f] = __fsub_rn(__ldg(X + r0 * d + f), anchor[f % d]);
-        __syncthreads();
-        {
-            const int r = threadIdx.x;
-            float xn = 0.f, am = 0.f;
-            if (r < nr)
-                for (int q = 0; q < d; ++q) {
-                    const float v = xsm[r * d + q];
-                    xn = __fmaf_rn(v, v, xn);
-                    am = fmaxf(am, fabsf(v));
-                }
-            xnorm[r0 + r] = xn;
-            const float s = fmt == FMT_FP8 ? fp8_scale(am) : 1.f;
-            if (fmt == FMT_FP8) xscale[r0 + r] = s;
-            inv_s[r] = 1.f / s;
+// The A image [row tile][katom][128 rows][128 B], eight rows a warp: the rows (contiguous
+// in X) come into the warp's shared memory with coalesced loads, moved by the anchor, at
+// an odd row stride; four lanes a row sum ||x'||^2 (FP32, strided partial sums, then a
+// fixed shuffle tree) and, for FP8, find the largest |x'_q| and with it the row's
+// power-of-two scale s_x; then consecutive lanes build the consecutive 16-byte chunks of a
+// row's atom (position p of row r holds logical chunk p ^ (r & 7)), so loads, stores and
+// shared-memory reads all spread.  Bound by reading X and writing the image: preparing
+// 1e7 x 128 for BF16 (kmpar_init as a whole) takes 7.1 ms; 14.6 ms with a thread a row,
+// whose reads of one bank queued.
+constexpr int kPrepWarps = 8, kPrepRows = 8;
+
+template <int fmt>
+__global__ void __launch_bounds__(32 * kPrepWarps) prep_points_kernel(const float *__restrict__ X, int64_t n,
+                                                                      int64_t n_pad, int d, int KA,
+                                                                      const float *__restrict__ anchor,
+                                                                      uint8_t *__restrict__ img,
+                                                                      float *__restrict__ xnorm,
+                                                                      float *__restrict__ xscale) {
+    extern __shared__ float xsm[];   // per warp kPrepRows x ds moved rows
+    __shared__ float inv_s[kPrepWarps][kPrepRows];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ds = d | 1;
+    float *xw = xsm + (size_t)w * kPrepRows * ds;
+    const int64_t nblk = n_pad / kPrepRows, stride = (int64_t)gridDim.x * kPrepWarps;
+    const Enc em{d, fmt, nullptr};   // the staged rows are already moved
+    for (int64_t b = (int64_t)blockIdx.x * kPrepWarps + w; b < nblk; b += stride) {   // uniform per warp
+        const int64_t r0 = b * kPrepRows;
+        const int nr = (int)max((int64_t)0, min((int64_t)kPrepRows, n - r0));
+        __syncwarp();   // the previous rows' readers are done
+        for (int q = lane; q < d; q += 32) {
+            const float a = __ldg(anchor + q);
+            float v[kPrepRows];
+#pragma unroll
+            for (int r = 0; r < kPrepRows; ++r) v[r] = r < nr ? __ldg(X + (r0 + r) * d + q) : a;
+#pragma unroll
+            for (int r = 0; r < kPrepRows; ++r) xw[r * ds + q] = __fsub_rn(v[r], a);
         }
-        __syncthreads();
-        uint8_t *tile = img + (size_t)t * KA * BM * 128;
-        const int pos = threadIdx.x & 7;
-        const Enc em{d, fmt, nullptr};   // the staged rows are already moved
+        __syncwarp();
+        {
+            const int r = lane >> 2;
+            float xn = 0.f, am = 0.f;
+            for (int q = lane & 3; q < d; q += 4) {
+                const float v = xw[r * ds + q];
+                xn = __fmaf_rn(v, v, xn);
+                am = fmaxf(am, fabsf(v));
+            }
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                xn += __shfl_xor_sync(0xffffffffu, xn, o);
+                am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
+            }
+            if ((lane & 3) == 0) {
+                xnorm[r0 + r] = xn;
+                const float s = fmt == FMT_FP8 ? fp8_scale(am) : 1.f;
+                if (fmt == FMT_FP8) xscale[r0 + r] = s;
+                inv_s[w][r] = 1.f / s;
+            }
+        }
+        __syncwarp();
+        uint8_t *tile = img + (size_t)(r0 / BM) * KA * BM * 128;
+        const int rb = (int)(r0 % BM);
         for (int a = 0; a < KA; ++a)
-            for (int r = threadIdx.x >> 3; r < BM; r += BM / 8) {
-                const int ch = pos ^ (r & 7);
+#pragma unroll
+            for (int f = lane; f < kPrepRows * 8; f += 32) {
+                const int r = f >> 3, pos = f & 7, ch = pos ^ ((rb + r) & 7);
+                const float *x = xw + r * ds;
                 uint4 u;
                 if (fmt == FMT_FP8) {
-                    u = pack16_e4m3(xsm + r * d, d, a * 128 + ch * 16, inv_s[r], r >= nr);
+                    u = pack16_e4m3(x, d, a * 128 + ch * 16, inv_s[w][r], r >= nr);
                 } else {
                     __nv_bfloat16 v[8];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) v[q] = r < nr ? a_elem(em, xsm + r * d, a * 64 + ch * 8 + q) : bf(0.f);
+                    for (int q = 0; q < 8; ++q) v[q] = r < nr ? a_elem(em, x, a * 64 + ch * 8 + q) : bf(0.f);
                     u = pack8(v);
                 }
-                *reinterpret_cast<uint4 *>(tile + (size_t)a * BM * 128 + r * 128 + pos * 16) = u;
+                *reinterpret_cast<uint4 *>(tile + (size_t)a * BM * 128 + (rb + r) * 128 + pos * 16) = u;
             }
     }
 }
@@ -525,11 +550,23 @@ cudaError_t launch_anchor(const float *X, int64_t n, int d, double *scratch, flo
 cudaError_t launch_prep_points(const float *X, int64_t n, int d, int fmt, const float *anchor, uint8_t *img,
                                float *xnorm, float *xscale, cudaStream_t s) {
     const int64_t n_pad = ((n + BM - 1) / BM) * BM;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(n_pad / BM, 8192));
-    const size_t sm = sizeof(float) * BM * (size_t)d;
-    cudaError_t e = cudaFuncSetAttribute(prep_points_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const int64_t blocks = n_pad / (kPrepWarps * kPrepRows);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, 8192));
+    const size_t sm = sizeof(float) * kPrepWarps * kPrepRows * (size_t)(d | 1);
+    auto go = [&](auto kern) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+        kern<<<grid, 32 * kPrepWarps, sm, s>>>(X, n, n_pad, d, tc_katoms(d, fmt), anchor, img, xnorm, xscale);
+        return cudaGetLastError();
+    };
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (fmt) {
+        case FMT_BF16: e = go(prep_points_kernel<FMT_BF16>); break;
+        case FMT_BF16X3: e = go(prep_points_kernel<FMT_BF16X3>); break;
+        case FMT_BF16N: e = go(prep_points_kernel<FMT_BF16N>); break;
+        case FMT_FP8: e = go(prep_points_kernel<FMT_FP8>); break;
+    }
     if (e != cudaSuccess) return e;
-    prep_points_kernel<<<grid, BM, sm, s>>>(X, n, n_pad, d, fmt, tc_katoms(d, fmt), anchor, img, xnorm, xscale);
     count_launches(1);
     return cudaGetLastError();
 }
