@@ -240,7 +240,7 @@ kmpar_status kmpar_init(kmpar_ctx **out, const float *X, int64_t n, int32_t d, i
     c.cap_total = (int)cap_total64;
     c.sort_block = kmp::sort_block_size(n, k);
     c.nsb = (int)((n + c.sort_block - 1) / c.sort_block);
-    c.num_partials = kmp::assign_num_partials(n, d);
+    c.num_partials = (int)((n + 31) / 32) + 1;   // enough for a scan of up to n rows, and one slot more
 
     auto bail = [&](kmpar_status s) {
         std::string m = c.err;
@@ -461,7 +461,7 @@ kmpar_status kmpar_weighted_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t ma
     KMP_CUDA(&c, cudaStreamSynchronize(c.stream), "sync");
     int *changed = reinterpret_cast<int *>(c.partials + c.num_partials - 1);   // the last partial slot
     const int np = kmp::assign_num_partials(m, c.d);
-    if (np + 1 > c.num_partials) return fail(&c, KMPAR_ERR_UNSUPPORTED, "candidate set larger than the point set");
+    if ((m + 127) / 128 + 1 > (int)((c.n + 127) / 128)) return fail(&c, KMPAR_ERR_UNSUPPORTED, "candidate set larger than the point set");
     int cur = 0, t = 0;
     for (;; ++t) {
         KMP_CUDA(&c, cudaMemsetAsync(changed, 0, sizeof(int), c.stream), "memset changed");
@@ -585,7 +585,8 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
                                                 c.num_partials, &c.st->argmin_fp64, c.stream),
                          "assign kernel");
                 KMP_CUDA(&c, kmp::timing_end(c, ev, 1), "timing");
-                KMP_CUDA(&c, kmp::launch_sum_f64(c.partials, c.num_partials, c.cost_dev, nullptr, c.stream),
+                KMP_CUDA(&c, kmp::launch_sum_f64(c.partials, kmp::assign_num_partials(c.n, c.d), c.cost_dev, nullptr,
+                                                 c.stream),
                          "cost sum");
             } else if (bounded && (tt > 0 || listed)) {
                 KMP_CUDA(&c, tt > 0 ? kmp::launch_lloyd_bounded_pass(c, centers_dev, c.labels[cur], c.labels[cur ^ 1],

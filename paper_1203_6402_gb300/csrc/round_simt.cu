@@ -4,7 +4,8 @@
 //
 // Kernels:
 //   pick_first_kernel   Alg. 2 step 1: i0 = floor(u n), row gathered as candidate 0
-//   nearest_kernel      d^2(x, C') for the batch C' (or all k centers), top-2 per
+//   first_dist_kernel   Alg. 2 step 2: D^2 to the first center, per-block FP64 sums
+//   nearest_tile_kernel d^2(x, C') for the batch C' (or all k centers), top-2 per
 //                       row, FP64 re-decision of near ties, D^2/idx/labels update,
 //                       per-block FP64 partial of phi
 //   sample_kernel       Alg. 2 step 4: p = min(1, l D^2/phi), Philox draw,
@@ -20,8 +21,6 @@
 
 namespace kmp {
 
-constexpr int kNearThreads = 128;
-
 // How the resident refine covers a pass of cap_rows centers: `parts` launches of
 // `rows` centers each (`hold` rows of shared memory, `warps` warps per CTA).
 // parts = 0: the per-row kernel (refine_kernel) is used instead.
@@ -30,17 +29,17 @@ struct ResidentPlan {
 };
 ResidentPlan resident_plan(int cap_rows, int d);
 
-enum { MODE_FIRST = 0, MODE_ROUND = 1, MODE_ASSIGN = 2 };
+enum { MODE_ROUND = 1, MODE_ASSIGN = 2 };
 
 struct NearestParams {
     const float *X;
     int64_t n;
     int d;
     const float *C;        // center rows, stride d
-    int c_begin, c_cnt;    // ASSIGN: static range; FIRST/ROUND: taken from st
+    int c_begin, c_cnt;    // ASSIGN: static range; ROUND: taken from st
     const DevState *st;
-    float *D2;             // FIRST: out; ROUND: in/out
-    int32_t *idx;          // FIRST: out; ROUND: in/out
+    float *D2;             // ROUND: in/out
+    int32_t *idx;          // ROUND: in/out
     int32_t *labels;       // ASSIGN: out (nullable)
     const int32_t *prev;   // ASSIGN: previous labels (nullable)
     int *changed;          // ASSIGN: +number of labels != prev (nullable)
@@ -56,11 +55,91 @@ __device__ __forceinline__ void take_if_better(double v, int j, double &best, in
     if (v < best || (v == best && j < bj)) { best = v; bj = j; }
 }
 
+// The decision for row pt once its lexicographic (value, center) best and runner-up
+// (b1, i1), (b2, i2) are known (INT_MAX: none): writes the row's outputs, returns the
+// stored distance; chg: a label changed.
+template <int MODE>
+__device__ __forceinline__ float nearest_decide(const NearestParams &p, int64_t pt, float b1, int i1, float b2, int i2,
+                                                int &chg) {
+    const int d = p.d;
+    const float *xrow = p.X + pt * (int64_t)d;
+    const float W = fp32_tie_window(d);
+    if (i1 == INT_MAX) i1 = -1;
+    if (i2 == INT_MAX) i2 = -1;
+    float stored = 0.f;
+    if constexpr (MODE == MODE_ASSIGN) {
+        // a row whose distances are all NaN/inf keeps label 0 (labels stay in range)
+        int lab = i1 >= 0 ? i1 : 0;
+        stored = b1;
+        if (i2 >= 0 && b2 <= b1 + W * b1) {
+            // the FP32 order of the two best may differ from the FP64 order
+            double best = dist2_fp64(xrow, p.C + (int64_t)i1 * d, d);
+            int bj = i1;
+            take_if_better(dist2_fp64(xrow, p.C + (int64_t)i2 * d, d), i2, best, bj);
+            if (bj == i2) { lab = i2; stored = b2; }
+            atomicAdd(p.fp64_cnt, 1ull);
+        }
+        if (p.labels) p.labels[pt] = lab;
+        if (p.dmin) p.dmin[pt] = stored;
+        if (p.prev) chg = (p.prev[pt] != lab);
+    } else {
+        const float old = p.D2[pt];
+        const int oi = p.idx[pt];
+        const float m32 = fminf(old, b1);
+        const float lim = m32 + W * m32;
+        const bool in_old = (oi >= 0) && old <= lim;
+        const bool in1 = i1 >= 0 && b1 <= lim;
+        const bool in2 = i2 >= 0 && b2 <= lim;
+        int win = -1;
+        float wv = old;
+        if ((int)in_old + (int)in1 + (int)in2 >= 2) {
+            double best = DBL_MAX;
+            int bj = INT_MAX;
+            if (in_old) take_if_better(dist2_fp64(xrow, p.C + (int64_t)oi * d, d), oi, best, bj);
+            if (in1) take_if_better(dist2_fp64(xrow, p.C + (int64_t)i1 * d, d), i1, best, bj);
+            if (in2) take_if_better(dist2_fp64(xrow, p.C + (int64_t)i2 * d, d), i2, best, bj);
+            atomicAdd(p.fp64_cnt, 1ull);
+            if (in1 && in2) atomicAdd(p.wide_cnt, 1ull);
+            if (bj == i1) { win = i1; wv = b1; }
+            else if (bj == i2) { win = i2; wv = b2; }
+        } else if (i1 >= 0 && b1 < old) {
+            win = i1; wv = b1;
+        }
+        if (win >= 0) {
+            p.D2[pt] = wv;
+            p.idx[pt] = win;
+            stored = wv;
+        } else {
+            stored = old;
+        }
+    }
+    return stored;
+}
+
+// (value, index) order with the lower index first on equal values
+__device__ __forceinline__ bool lex_lt(float v, int i, float w, int j) { return v < w || (v == w && i < j); }
+
+// top-2 of the union of two top-2 lists
+__device__ __forceinline__ void top2_merge(float &b1, int &i1, float &b2, int &i2, float c1, int j1, float c2, int j2) {
+    if (lex_lt(c1, j1, b1, i1)) {
+        // c1 is the new best; second = best of (b1, c2)
+        if (lex_lt(b1, i1, c2, j2)) { b2 = b1; i2 = i1; } else { b2 = c2; i2 = j2; }
+        b1 = c1; i1 = j1;
+    } else if (lex_lt(c1, j1, b2, i2)) {
+        b2 = c1; i2 = j1;
+    }
+}
+
+// The scan for d <= 32: a row a thread, its coordinates in registers, 64 centers at a
+// time in shared memory.  With so few coordinates the tiled scan's handling of its tile's
+// results outweighs the sums (3e6 x 3 against 100: 0.36 ms, tiled 0.8; 1e6 x 32 against
+// 100: 0.59, 0.68; at 50 coordinates 200,000 rows against 300 take 0.62, tiled 0.52).
+constexpr int kNearThreads = 128;
+
 template <int DP, int MODE>
 __global__ void __launch_bounds__(kNearThreads) nearest_kernel(NearestParams p) {
-    constexpr int TC = DP == 0 ? 1 : (DP <= 64 ? 64 : 32);
-    constexpr int TILE = DP == 0 ? 4 : TC * DP;
-    __shared__ __align__(16) float tile[TILE];
+    constexpr int TC = 64;
+    __shared__ __align__(16) float tile[TC * DP];
     __shared__ double red[32];
     __shared__ int redi[32];
 
@@ -76,11 +155,9 @@ __global__ void __launch_bounds__(kNearThreads) nearest_kernel(NearestParams p) 
     const int d = p.d;
     const float *xrow = p.X + (valid ? pt : 0) * (int64_t)d;
 
-    float xr[DP == 0 ? 1 : DP];
-    if constexpr (DP > 0) {
+    float xr[DP];
 #pragma unroll
-        for (int q = 0; q < DP; ++q) xr[q] = (valid && q < d) ? __ldg(xrow + q) : 0.f;
-    }
+    for (int q = 0; q < DP; ++q) xr[q] = (valid && q < d) ? __ldg(xrow + q) : 0.f;
 
     int begin, cnt;
     if constexpr (MODE == MODE_ASSIGN) {
@@ -90,33 +167,27 @@ __global__ void __launch_bounds__(kNearThreads) nearest_kernel(NearestParams p) 
     }
 
     float b1 = FLT_MAX, b2 = FLT_MAX;
-    int i1 = -1, i2 = -1;
+    int i1 = INT_MAX, i2 = INT_MAX;
     for (int t0 = 0; t0 < cnt; t0 += TC) {
         const int nt = min(TC, cnt - t0);
-        if constexpr (DP > 0) {
-            __syncthreads();
-            for (int e = tid; e < TC * DP; e += kNearThreads) {
-                const int r = e / DP, q = e - r * DP;
-                tile[e] = (r < nt && q < d) ? __ldg(p.C + (int64_t)(begin + t0 + r) * d + q) : 0.f;
-            }
-            __syncthreads();
+        __syncthreads();
+        for (int e = tid; e < TC * DP; e += kNearThreads) {
+            const int r = e / DP, q = e - r * DP;
+            tile[e] = (r < nt && q < d) ? __ldg(p.C + (int64_t)(begin + t0 + r) * d + q) : 0.f;
         }
+        __syncthreads();
         if (valid) {
             for (int r = 0; r < nt; ++r) {
                 float acc = 0.f;
-                if constexpr (DP > 0) {
-                    const float4 *c4 = reinterpret_cast<const float4 *>(tile + r * DP);
+                const float4 *c4 = reinterpret_cast<const float4 *>(tile + r * DP);
 #pragma unroll
-                    for (int q4 = 0; q4 < DP / 4; ++q4) {
-                        const float4 c = c4[q4];
-                        float t;
-                        t = __fsub_rn(xr[4 * q4 + 0], c.x); acc = __fmaf_rn(t, t, acc);
-                        t = __fsub_rn(xr[4 * q4 + 1], c.y); acc = __fmaf_rn(t, t, acc);
-                        t = __fsub_rn(xr[4 * q4 + 2], c.z); acc = __fmaf_rn(t, t, acc);
-                        t = __fsub_rn(xr[4 * q4 + 3], c.w); acc = __fmaf_rn(t, t, acc);
-                    }
-                } else {
-                    acc = dist2_fp32(xrow, p.C + (int64_t)(begin + t0 + r) * d, d);
+                for (int q4 = 0; q4 < DP / 4; ++q4) {
+                    const float4 c = c4[q4];
+                    float t;
+                    t = __fsub_rn(xr[4 * q4 + 0], c.x); acc = __fmaf_rn(t, t, acc);
+                    t = __fsub_rn(xr[4 * q4 + 1], c.y); acc = __fmaf_rn(t, t, acc);
+                    t = __fsub_rn(xr[4 * q4 + 2], c.z); acc = __fmaf_rn(t, t, acc);
+                    t = __fsub_rn(xr[4 * q4 + 3], c.w); acc = __fmaf_rn(t, t, acc);
                 }
                 const int j = begin + t0 + r;
                 if (acc < b2) {
@@ -129,60 +200,7 @@ __global__ void __launch_bounds__(kNearThreads) nearest_kernel(NearestParams p) 
 
     float stored = 0.f;
     int chg = 0;
-    if (valid) {
-        const float W = fp32_tie_window(d);
-        if constexpr (MODE == MODE_ASSIGN) {
-            // a row whose distances are all NaN/inf keeps label 0 (labels stay in range)
-            int lab = i1 >= 0 ? i1 : 0;
-            stored = b1;
-            if (i2 >= 0 && b2 <= b1 + W * b1) {
-                // the FP32 order of the two best may differ from the FP64 order
-                double best = dist2_fp64(xrow, p.C + (int64_t)i1 * d, d);
-                int bj = i1;
-                take_if_better(dist2_fp64(xrow, p.C + (int64_t)i2 * d, d), i2, best, bj);
-                if (bj == i2) { lab = i2; stored = b2; }
-                atomicAdd(p.fp64_cnt, 1ull);
-            }
-            if (p.labels) p.labels[pt] = lab;
-            if (p.dmin) p.dmin[pt] = stored;
-            if (p.prev) chg = (p.prev[pt] != lab);
-        } else if constexpr (MODE == MODE_FIRST) {
-            stored = (i1 >= 0) ? b1 : __int_as_float(0x7f800000);
-            p.D2[pt] = stored;
-            p.idx[pt] = 0;
-        } else {
-            const float old = p.D2[pt];
-            const int oi = p.idx[pt];
-            const float m32 = fminf(old, b1);
-            const float lim = m32 + W * m32;
-            const bool in_old = (oi >= 0) && old <= lim;
-            const bool in1 = i1 >= 0 && b1 <= lim;
-            const bool in2 = i2 >= 0 && b2 <= lim;
-            int win = -1;
-            float wv = old;
-            if ((int)in_old + (int)in1 + (int)in2 >= 2) {
-                double best = DBL_MAX;
-                int bj = INT_MAX;
-                if (in_old) take_if_better(dist2_fp64(xrow, p.C + (int64_t)oi * d, d), oi, best, bj);
-                if (in1) take_if_better(dist2_fp64(xrow, p.C + (int64_t)i1 * d, d), i1, best, bj);
-                if (in2) take_if_better(dist2_fp64(xrow, p.C + (int64_t)i2 * d, d), i2, best, bj);
-                atomicAdd(p.fp64_cnt, 1ull);
-                if (in1 && in2) atomicAdd(p.wide_cnt, 1ull);
-                if (bj == i1) { win = i1; wv = b1; }
-                else if (bj == i2) { win = i2; wv = b2; }
-            } else if (i1 >= 0 && b1 < old) {
-                win = i1; wv = b1;
-            }
-            if (win >= 0) {
-                p.D2[pt] = wv;
-                p.idx[pt] = win;
-                stored = wv;
-            } else {
-                stored = old;
-            }
-        }
-    }
-
+    if (valid) stored = nearest_decide<MODE>(p, pt, b1, i1, b2, i2, chg);
     const double s = block_sum_f64(valid ? (double)stored : 0.0, red);
     if (tid == 0 && p.partials) p.partials[blockIdx.x] = s;
     if constexpr (MODE == MODE_ASSIGN) {
@@ -200,31 +218,268 @@ __global__ void __launch_bounds__(kNearThreads) nearest_kernel(NearestParams p) 
     }
 }
 
-template <int MODE>
-static cudaError_t launch_nearest_mode(const NearestParams &p, cudaStream_t s) {
-    const int grid = (int)((p.n + kNearThreads - 1) / kNearThreads);   // p.n = rows capacity for row lists
-    const int d = p.d;
-#define KMP_NEAREST_CASE(DPV)                                              \
-    if (d <= DPV) {                                                         \
-        nearest_kernel<DPV, MODE><<<grid, kNearThreads, 0, s>>>(p);          \
-        count_launches(1);                                                   \
-        return cudaGetLastError();                                           \
+// The exact FP32 nearest-center scan, tiled like a GEMM.  A block of 8 x RT threads takes
+// BM rows and walks the centers 8 TN at a time; a thread holds 4 x TN distances of its
+// tile in registers and adds coordinate after coordinate (t = x - c, acc = fma(t, t, acc),
+// ascending: the chain of dist2_fp32), so the FP32 pipe always has 4 TN independent
+// chains a thread and each shared-memory read feeds several.  Rows (resident while
+// d <= kTileK) and centers lie in shared memory coordinate-major with 16 bytes of padding
+// a coordinate, brought in by 4-byte asynchronous copies (the transposition costs no
+// registers); the next tile of centers is copied while one is summed.  A thread meets its
+// centers in ascending order; the 8 threads of a row merge their top two.  (The FP32 pipe
+// gives packed pairs no more lanes: in a loop of this shape 8 x 4 scalar chains ran at 31 T
+// operations/s of 40.3, packed ones at 30.)  Bound by FP32 issue: the cost of 1e6 x 42
+// against 500 centers 2.23 -> 1.96 ms, a fit of 200k x 50, k = 300 11.9 -> 8.9 ms, against a
+// row per thread with its coordinates in registers.
+constexpr int kTileK = 96;    // coordinates resident: two blocks an SM
+constexpr int kTileChunk = 64;   // coordinates of a step when the rows are not resident
+
+__device__ __forceinline__ void cp_async4_zfill(uint32_t dst, const float *src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+
+// coordinates q0 .. q0 + kn - 1 of rows first .. first + B - 1 (rows given: of the rows
+// rows[first + r]; rows at or past `limit` as zeros) to dst[q * stride + r], consecutive
+// threads along a row and then the next
+template <int THREADS>
+__device__ __forceinline__ void tile_copy(float *dst, int stride, int B, const float *src, int64_t first, int64_t limit,
+                                          const int32_t *rows, int d, int q0, int kn) {
+    int r = threadIdx.x / kn, q = threadIdx.x % kn;
+    const int dr = THREADS / kn, dq = THREADS % kn;
+    uint32_t to = static_cast<uint32_t>(__cvta_generic_to_shared(dst + q * stride + r));
+    const uint32_t step = 4u * (dq * stride + dr), wrap = 4u * (kn * stride - 1);
+    if (!rows) {
+        const float *from = src + (first + r) * d + q0 + q;
+        const int64_t fs = (int64_t)dr * d + dq, fw = d - kn;
+        const int lim = (int)min((int64_t)B, limit - first);
+#pragma unroll 4
+        while (r < B) {
+            const bool ok = r < lim;
+            cp_async4_zfill(to, ok ? from : src, ok);
+            r += dr;
+            q += dq;
+            from += fs;
+            to += step;
+            if (q >= kn) { q -= kn; ++r; from += fw; to -= wrap; }
+        }
+    } else {
+        while (r < B) {
+            const bool ok = first + r < limit;
+            cp_async4_zfill(to, ok ? src + (int64_t)rows[first + r] * d + q0 + q : src, ok);
+            r += dr;
+            q += dq;
+            to += step;
+            if (q >= kn) { q -= kn; ++r; to -= wrap; }
+        }
     }
-    KMP_NEAREST_CASE(4)
-    KMP_NEAREST_CASE(8)
-    KMP_NEAREST_CASE(16)
-    KMP_NEAREST_CASE(32)
-    KMP_NEAREST_CASE(48)
-    KMP_NEAREST_CASE(64)
-    KMP_NEAREST_CASE(96)
-    KMP_NEAREST_CASE(128)
-#undef KMP_NEAREST_CASE
-    nearest_kernel<0, MODE><<<grid, kNearThreads, 0, s>>>(p);
+}
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <int MODE, int BM, int TN>
+__global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 8) nearest_tile_kernel(NearestParams p, int kc) {
+    constexpr int TM = 4, threads = 2 * BM, BN = 8 * TN;
+    constexpr int XS = BM + 4, CS = BN + 4;   // floats per coordinate
+    extern __shared__ __align__(16) float tsm[];
+    __shared__ double red[32];
+    __shared__ int redi[32];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3, d = p.d;
+    const bool resident = d <= kc;
+    float *xb = tsm, *cb = tsm + (resident ? 1 : 2) * kc * XS;   // rows (two buffers in steps), centers (two)
+    const int64_t base = (int64_t)blockIdx.x * BM;
+    const int64_t nrows = p.rows ? (int64_t)*p.rows_cnt : p.n;
+    if (p.rows && base >= nrows) return;   // uniform per block
+    int begin, cnt;
+    if constexpr (MODE == MODE_ASSIGN) {
+        begin = p.c_begin; cnt = p.c_cnt;
+    } else {
+        begin = p.st->batch_begin; cnt = p.st->batch_cnt;
+    }
+    const int chunks = (d + kc - 1) / kc, steps = ((cnt + BN - 1) / BN) * chunks;
+    auto issue = [&](int s) {   // step s: tile s / chunks of the centers, chunk s % chunks of the coordinates
+        const int t = s / chunks, q0 = (s - t * chunks) * kc, kn = min(kc, d - q0);
+        if (!resident || s == 0)
+            tile_copy<threads>(xb + (resident ? 0 : (s & 1) * kc * XS), XS, BM, p.X, base, nrows, p.rows, d, q0, kn);
+        tile_copy<threads>(cb + (s & 1) * kc * CS, CS, BN, p.C, begin + (int64_t)t * BN, begin + (int64_t)cnt, nullptr, d,
+                           q0, kn);
+    };
+    float b1[TM], b2[TM];
+    int i1[TM], i2[TM];
+#pragma unroll
+    for (int i = 0; i < TM; ++i) { b1[i] = b2[i] = FLT_MAX; i1[i] = i2[i] = INT_MAX; }
+    float acc[TM][TN];
+    if (steps > 0) issue(0);
+    cp_async_commit();
+    for (int s = 0; s < steps; ++s) {
+        cp_async_wait<0>();
+        __syncthreads();   // step s is in, and every thread is done with step s - 1
+        if (s + 1 < steps) issue(s + 1);
+        cp_async_commit();
+        const int t = s / chunks, ch = s - t * chunks, kn = min(kc, d - ch * kc);
+        if (ch == 0) {
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+        }
+        const float *xq = xb + (resident ? 0 : (s & 1) * kc * XS) + ty * 4, *cq = cb + (s & 1) * kc * CS + tx * 4;
+#pragma unroll 2
+        for (int q = 0; q < kn; ++q, xq += XS, cq += CS) {
+            float x[TM], c[TN];
+            const float4 xv = *reinterpret_cast<const float4 *>(xq);
+            x[0] = xv.x; x[1] = xv.y; x[2] = xv.z; x[3] = xv.w;
+#pragma unroll
+            for (int j = 0; j < TN; j += 4) {   // columns 4 tx .. + 3 of each 32
+                const float4 v = *reinterpret_cast<const float4 *>(cq + 8 * j);
+                c[j] = v.x; c[j + 1] = v.y; c[j + 2] = v.z; c[j + 3] = v.w;
+            }
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) {
+                    const float u = __fsub_rn(x[i], c[j]);
+                    acc[i][j] = __fmaf_rn(u, u, acc[i][j]);
+                }
+        }
+        if (ch + 1 < chunks) continue;
+        // the thread's centers of this tile, ascending: a row whose smallest value is not
+        // below its runner-up needs no look at the others (after the first tiles, most)
+        const int c0 = t * BN + tx * 4;   // column j: c0 + (j / 4) 32 + j % 4
+        if (t * BN + BN > cnt) {   // pad columns hold the distance to 0
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                if (c0 + (j >> 2) * 32 + (j & 3) >= cnt) {
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) acc[i][j] = FLT_MAX;
+                }
+        }
+#pragma unroll
+        for (int r = 0; r < TM; ++r) {
+            float m = acc[r][0];
+#pragma unroll
+            for (int j = 1; j < TN; ++j) m = fminf(m, acc[r][j]);
+            if (m < b2[r]) {
+#pragma unroll
+                for (int j = 0; j < TN; ++j) {
+                    const float a = acc[r][j];
+                    if (a < b2[r]) {
+                        const int c = begin + c0 + (j >> 2) * 32 + (j & 3);
+                        if (a < b1[r]) { b2[r] = b1[r]; i2[r] = i1[r]; b1[r] = a; i1[r] = c; }
+                        else { b2[r] = a; i2[r] = c; }
+                    }
+                }
+            }
+        }
+    }
+    auto number = [&](int r) -> int64_t {
+        const int64_t at = base + r;
+        return at < nrows ? (p.rows ? (int64_t)p.rows[at] : at) : -1;
+    };
+    // merge the 8 threads of a row, then thread tx = r decides the thread row's row r
+    float m1 = FLT_MAX, m2 = FLT_MAX;
+    int n1 = INT_MAX, n2 = INT_MAX;
+#pragma unroll
+    for (int r = 0; r < TM; ++r) {
+        float v1 = b1[r], v2 = b2[r];
+        int j1 = i1[r], j2 = i2[r];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            const float u1 = __shfl_xor_sync(0xffffffffu, v1, o), u2 = __shfl_xor_sync(0xffffffffu, v2, o);
+            const int k1 = __shfl_xor_sync(0xffffffffu, j1, o), k2 = __shfl_xor_sync(0xffffffffu, j2, o);
+            top2_merge(v1, j1, v2, j2, u1, k1, u2, k2);
+        }
+        if (tx == r) { m1 = v1; m2 = v2; n1 = j1; n2 = j2; }
+    }
+    const int64_t pt = tx < TM ? number(ty * 4 + tx) : -1;
+    float stored = 0.f;
+    int chg = 0;
+    if (pt >= 0) stored = nearest_decide<MODE>(p, pt, m1, n1, m2, n2, chg);
+    const double s = block_sum_f64(pt >= 0 ? (double)stored : 0.0, red);
+    if (tid == 0 && p.partials) p.partials[blockIdx.x] = s;
+    if constexpr (MODE == MODE_ASSIGN) {
+        if (p.changed) {
+            int c = warp_sum_i32(chg);
+            __syncthreads();
+            if ((tid & 31) == 0) redi[tid >> 5] = c;
+            __syncthreads();
+            if (tid == 0) {
+                int tot = 0;
+                for (int i = 0; i < threads / 32; ++i) tot += redi[i];
+                if (tot) atomicAdd(p.changed, tot);
+            }
+        }
+    }
+}
+
+// rows per block of the scan: small sets are cut finer, so that more SMs take part (40,000
+// rows in blocks of 128 are two a SM; from there on the larger tile's reuse counts for more).
+// Up to 32 coordinates a row per thread holds them in registers and needs no tile of rows.
+static int scan_rows(int64_t n, int d) { return d > 32 && n <= 40000 ? 32 : 128; }
+
+int assign_num_partials(int64_t n, int d) { return (int)((n + scan_rows(n, d) - 1) / scan_rows(n, d)); }
+
+template <int MODE>
+static cudaError_t launch_nearest_mode(const NearestParams &p, int cnt_hint, cudaStream_t s) {
+    const int grid = assign_num_partials(p.n, p.d);   // p.n = rows capacity for row lists
+    const int kc = p.d <= kTileK ? p.d : kTileChunk;
+    const bool small = scan_rows(p.n, p.d) == 32, narrow = cnt_hint <= 32;
+    const size_t smem = sizeof(float) * kc * ((p.d <= kTileK ? 1 : 2) * (small ? 36 : 132) + 2 * (narrow ? 36 : 68));
+    auto tiles = [&](auto kern, int threads) -> cudaError_t {
+        if (smem > 40 * 1024) {   // (the static shared memory counts too)
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        kern<<<grid, threads, smem, s>>>(p, kc);
+        return cudaGetLastError();
+    };
     count_launches(1);
+    if (p.d <= 4) nearest_kernel<4, MODE><<<grid, kNearThreads, 0, s>>>(p);
+    else if (p.d <= 8) nearest_kernel<8, MODE><<<grid, kNearThreads, 0, s>>>(p);
+    else if (p.d <= 16) nearest_kernel<16, MODE><<<grid, kNearThreads, 0, s>>>(p);
+    else if (p.d <= 32) nearest_kernel<32, MODE><<<grid, kNearThreads, 0, s>>>(p);
+    else if (small) return narrow ? tiles(nearest_tile_kernel<MODE, 32, 4>, 64) : tiles(nearest_tile_kernel<MODE, 32, 8>, 64);
+    else return narrow ? tiles(nearest_tile_kernel<MODE, 128, 4>, 256) : tiles(nearest_tile_kernel<MODE, 128, 8>, 256);
     return cudaGetLastError();
 }
 
-int assign_num_partials(int64_t n, int) { return (int)((n + kNearThreads - 1) / kNearThreads); }
+// Alg. 2 step 2: D^2 to the first center, idx = 0.  128 rows a block, 32 coordinates at a
+// time through shared memory (coalesced loads, a lane-per-row walk at an odd stride):
+// bound by reading X.
+constexpr int kFirstRows = 128;
+
+__global__ void __launch_bounds__(kFirstRows) first_dist_kernel(const float *__restrict__ X, int64_t n, int d,
+                                                               const float *__restrict__ C, float *__restrict__ D2,
+                                                               int32_t *__restrict__ idx, double *partials) {
+    __shared__ float xs[kFirstRows][33];
+    __shared__ float cq[32];
+    __shared__ double red[32];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int64_t base = (int64_t)blockIdx.x * kFirstRows, R = base + tid;
+    float v = 0.f;
+    for (int q0 = 0; q0 < d; q0 += 32) {
+        const int kn = min(32, d - q0);
+        __syncthreads();   // the walkers of the last piece are done
+#pragma unroll 8
+        for (int r = w; r < kFirstRows; r += kFirstRows / 32)
+            if (lane < kn && base + r < n) xs[r][lane] = __ldg(X + (base + r) * d + q0 + lane);
+        if (tid < kn) cq[tid] = C[q0 + tid];
+        __syncthreads();
+        for (int q = 0; q < kn; ++q) {
+            const float t = __fsub_rn(xs[tid][q], cq[q]);
+            v = __fmaf_rn(t, t, v);
+        }
+    }
+    // (a distance that is not below the largest float counts as infinite)
+    const float stored = v < FLT_MAX ? v : __int_as_float(0x7f800000);
+    if (R < n) {
+        D2[R] = stored;
+        idx[R] = 0;
+    }
+    const double s = block_sum_f64(R < n ? (double)stored : 0.0, red);
+    if (tid == 0) partials[blockIdx.x] = s;
+}
 
 // ------------------------------------------------------------------ init
 __global__ void pick_first_kernel(const float *X, int64_t n, int d, uint64_t seed, DevState *st,
@@ -252,12 +507,11 @@ cudaError_t launch_init_first(Ctx &c) {
     count_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    NearestParams p{};
-    p.X = c.X; p.n = c.n; p.d = c.d; p.C = c.C; p.st = c.st; p.D2 = c.D2; p.idx = c.idx;
-    p.partials = c.partials; p.fp64_cnt = &c.st->argmin_fp64; p.wide_cnt = &c.st->argmin_wide;
-    e = launch_nearest_mode<MODE_FIRST>(p, c.stream);
-    if (e != cudaSuccess) return e;
-    return launch_phi_finalize(c, assign_num_partials(c.n, c.d), &c.st->phi, &c.st->phi_hist[0]);
+    const int grid = (int)((c.n + kFirstRows - 1) / kFirstRows);
+    first_dist_kernel<<<grid, kFirstRows, 0, c.stream>>>(c.X, c.n, c.d, c.C, c.D2, c.idx, c.partials);
+    count_launches(1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_phi_finalize(c, grid, &c.st->phi, &c.st->phi_hist[0]);
 }
 
 // ------------------------------------------------------------------ sampling
@@ -473,7 +727,7 @@ cudaError_t launch_round_distance(Ctx &c, int round) {
     NearestParams p{};
     p.X = c.X; p.n = c.n; p.d = c.d; p.C = c.C; p.st = c.st; p.D2 = c.D2; p.idx = c.idx;
     p.partials = c.partials; p.fp64_cnt = &c.st->argmin_fp64; p.wide_cnt = &c.st->argmin_wide;
-    if ((e = launch_nearest_mode<MODE_ROUND>(p, c.stream)) != cudaSuccess) return e;
+    if ((e = launch_nearest_mode<MODE_ROUND>(p, c.cap_round, c.stream)) != cudaSuccess) return e;
     if ((e = timing_end(c, ev, 0)) != cudaSuccess) return e;
     return launch_phi_finalize(c, assign_num_partials(c.n, c.d), &c.st->phi, &c.st->phi_hist[round]);
 }
@@ -485,7 +739,7 @@ cudaError_t launch_assign(const float *X, int64_t n, int d, const float *C, int 
     p.X = X; p.n = n; p.d = d; p.C = C; p.c_begin = 0; p.c_cnt = k;
     p.labels = labels; p.prev = prev; p.changed = changed; p.partials = partials;
     p.fp64_cnt = fp64_cnt; p.wide_cnt = fp64_cnt;
-    return launch_nearest_mode<MODE_ASSIGN>(p, s);
+    return launch_nearest_mode<MODE_ASSIGN>(p, k, s);
 }
 
 // ------------------------------------------------------------------ generator export
@@ -562,21 +816,8 @@ cudaError_t launch_sum_rows(const float *v, int64_t n, double *partials, int max
     return launch_sum_f64(partials, (int)nb, out, copy, s);
 }
 
-// (value, index) top-2 of the union of two top-2 lists (lowest index on equal values)
-__device__ __forceinline__ bool lex_lt(float v, int i, float w, int j) { return v < w || (v == w && i < j); }
-
-__device__ __forceinline__ void top2_merge(float &b1, int &i1, float &b2, int &i2, float c1, int j1, float c2, int j2) {
-    if (lex_lt(c1, j1, b1, i1)) {
-        // c1 is the new best; second = best of (b1, c2)
-        if (lex_lt(b1, i1, c2, j2)) { b2 = b1; i2 = i1; } else { b2 = c2; i2 = j2; }
-        b1 = c1; i1 = j1;
-    } else if (lex_lt(c1, j1, b2, i2)) {
-        b2 = c1; i2 = j1;
-    }
-}
-
 // The decision for row R once its best and runner-up candidates (b1, i1), (b2, i2)
-// have exact FP32 values (i2 = -1: none), taken exactly as nearest_kernel takes
+// have exact FP32 values (i2 = -1: none), taken exactly as nearest_decide takes
 // it.  Lloyd: the label is the best, re-decided in FP64 against the runner-up
 // when their FP32 values lie within the tie window.  Round: the current center
 // is replaced by the best new candidate when nearer; when two or more of (current,
@@ -684,9 +925,6 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
                  "l"(src)
                  : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 struct ScreenBound {
     const float *xnorm;            // ||x'||^2 per point (x' = x - anchor)
@@ -1178,7 +1416,7 @@ size_t refine_smem_bytes(int d) { return sizeof(float) * refine_warps(d) * 96 * 
 // dist2_fp32): per coordinate pair four broadcast and two conflict-free 8-byte
 // shared loads (row stride 2 mod 4) feed 32 FP32 operations, and every center chunk
 // serves 32 rows.  A lexicographic top-2 per row is merged across the warp, then the
-// same decision as nearest_kernel (decide_top2).  Persistent: the row count is read
+// same decision as nearest_decide (decide_top2).  Persistent: the row count is read
 // on the device.
 constexpr int kFxWarpRows = 4;
 constexpr int kFxRows = 8 * kFxWarpRows;
