@@ -318,6 +318,7 @@ cudaError_t launch_sum_rows(const float *v, int64_t n, double *partials, int max
                             cudaStream_t s);
 cudaError_t launch_uniforms(int64_t count, uint32_t round, uint32_t tag, uint64_t seed, double *out,
                             cudaStream_t s);
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s);   // cudaFreeAsync on s
 cudaError_t launch_sum_f64(const double *parts, int nparts, double *out, double *copy, cudaStream_t s);
 
 }  // namespace kmp
