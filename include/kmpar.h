@@ -118,8 +118,8 @@ typedef struct {
                                      itself kept (the others took the list pass)     */
     int64_t recluster_snapshots;  /* batched reclustering: D^2 snapshots taken       */
     int64_t lloyd_settled;        /* Lloyd assignments (rows x iterations) that the
-                                     bounds between iterations settled without the
-                                     tensor pass (tensor modes; same results)        */
+                                     bounds or the lists of nearby centers settled
+                                     without the tensor pass (same results)          */
 } kmpar_stats;
 
 /*
@@ -277,8 +277,9 @@ KMPAR_API kmpar_status kmpar_fit(const float *X, int64_t n, int32_t d, int32_t k
  * l + 10 sqrt(l) + 64 <= 4096.  results (host, count entries) receive each
  * problem's outcome; a problem whose round overflows its capacity stops there
  * with status KMPAR_ERR_CAPACITY, the others are unaffected.  Work space comes
- * from the library's pool; a problem runs in one thread block, or in a
- * thread-block cluster of 2, 4 or 8 blocks when it has more than 25,000 rows
+ * from the library's pool (beyond 256 MB from the device's); a problem runs in
+ * one thread block, or in a thread-block cluster of 2, 4 or 8 blocks when it has more than 25,000 rows,
+ * or fewer where the call's blocks would not fill the SMs
  * (each block a contiguous range of rows; the cluster combines its sums and its
  * ordered draws in rank order; see kmpar_batch_set_split), largest problems
  * first, one kernel launch per (dimension class, cluster size).  Synchronises.
@@ -309,7 +310,8 @@ typedef struct {
 
 /* Schedule of kmpar_batch_run (process-wide): a problem of more than
  * rows_per_block rows is split over a thread-block cluster of 2, 4 or 8 blocks
- * (default 25,000; 0: never split).  Results do not depend on it beyond the
+ * (default 25,000; 0: never split), finer when the blocks of a call would
+ * not fill the SMs.  Results do not depend on it beyond the
  * association of FP64 sums.  KMPAR_ERR_ARG for a negative value. */
 KMPAR_API kmpar_status kmpar_batch_set_split(int32_t rows_per_block);
 
