@@ -260,6 +260,7 @@ kmpar_status kmpar_init(kmpar_ctx **out, const float *X, int64_t n, int32_t d, i
     c.cap_total = (int)cap_total64;
     c.sort_block = kmp::sort_block_size(n, k);
     c.nsb = (int)((n + c.sort_block - 1) / c.sort_block);
+    c.sum_blocks = (int)((n + 127) / 128);
     c.num_partials = (int)((n + 31) / 32) + 1;   // enough for a scan of up to n rows, and one slot more
 
     auto bail = [&](kmpar_status s) {
@@ -613,7 +614,7 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
                                                                      changed, c.dmin)
                                     : kmp::launch_lloyd_first_pass(c, centers_dev, c.labels[cur], changed, c.dmin),
                          "bounded assign pass");
-                KMP_CUDA(&c, kmp::launch_sum_rows(c.dmin, c.n, c.partials, c.num_partials, c.cost_dev, nullptr,
+                KMP_CUDA(&c, kmp::launch_sum_rows(c.dmin, c.n, c.partials, c.sum_blocks, c.cost_dev, nullptr,
                                                   c.stream),
                          "cost sum");
             } else {
@@ -624,7 +625,7 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
                                                            tt > 0 ? c.labels[cur ^ 1] : nullptr, changed, c.dmin, 1);
                 c.refine_order = nullptr;
                 KMP_CUDA(&c, pe, "tensor assign pass");
-                KMP_CUDA(&c, kmp::launch_sum_rows(c.dmin, c.n, c.partials, c.num_partials, c.cost_dev, nullptr,
+                KMP_CUDA(&c, kmp::launch_sum_rows(c.dmin, c.n, c.partials, c.sum_blocks, c.cost_dev, nullptr,
                                                   c.stream),
                          "cost sum");
             }

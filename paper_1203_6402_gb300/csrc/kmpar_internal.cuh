@@ -80,7 +80,8 @@ struct Ctx {
     int *rc_err = nullptr;        // recluster timeout flag
     int32_t *chosen = nullptr;    // k
     double *partials = nullptr;   // per-block FP64 partial sums
-    int num_partials = 0;
+    int num_partials = 0;        // slots of partials
+    int sum_blocks = 0;          // blocks (and partials) of a sum over the rows
     // Lloyd
     int32_t *labels[2] = {nullptr, nullptr};
     int32_t *perm = nullptr;

@@ -720,7 +720,7 @@ cudaError_t launch_round_distance(Ctx &c, int round) {
             count_launches(1);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-        return launch_sum_rows(c.D2, c.n, c.partials, c.num_partials, &c.st->phi, &c.st->phi_hist[round], c.stream);
+        return launch_sum_rows(c.D2, c.n, c.partials, c.sum_blocks, &c.st->phi, &c.st->phi_hist[round], c.stream);
     }
     cudaEvent_t ev = nullptr;
     if ((e = timing_begin(c, &ev)) != cudaSuccess) return e;
