@@ -140,6 +140,45 @@ cudaError_t alloc(kmp::Ctx &c, T **p, size_t count) {
     return cudaSuccess;
 }
 
+template <typename F>
+void give_back(kmp::Ctx &c, F request) {
+    request([&](auto *&p, size_t count) {
+        if (!p) return;
+        cudaFreeAsync(p, c.stream);
+        c.alloc_bytes -= (sizeof(*p) * (count ? count : 1) + 255) & ~(size_t)255;
+        p = nullptr;
+    });
+}
+
+// the round filter's buffers; given back after the last round
+template <typename T>
+void round_filter_buffers(kmp::Ctx &c, T take) {
+    const size_t cap = (size_t)c.cap_total;
+    take(c.rf_rad2, 2 * cap);
+    take(c.rf_num, 2 * cap);
+    take(c.rf_lst, cap * 4 * kmp::tc::kListSlots);
+    take(c.rf_head, cap);
+    take(c.rf_lcnt, (size_t)kmp::tc::kListLevels);
+    take(c.rf_rows, (size_t)c.n);
+    take(c.rf_cnt, (size_t)1);
+}
+
+// Buffers that only make a pass faster: all of them, or, when the memory is short, none
+// (the context then keeps the passes that do without).  request(take): take(p, count) on each.
+template <typename F>
+cudaError_t alloc_or_none(kmp::Ctx &c, F request) {
+    cudaError_t e = cudaSuccess;
+    request([&](auto *&p, size_t count) {
+        if (e == cudaSuccess && !p) e = alloc(c, &p, count);
+    });
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        give_back(c, request);
+        e = cudaSuccess;
+    }
+    return e;
+}
+
 void free_ctx(kmp::Ctx &c) {
     void *bufs[] = {c.st, c.D2, c.idx, c.drawn, c.cand, c.C, c.w, c.rD2, c.chosen, c.partials,
                     c.labels[0], c.labels[1], c.perm, c.hist, c.base, c.cost_dev, c.tc_img,
@@ -320,15 +359,6 @@ kmpar_status kmpar_init(kmpar_ctx **out, const float *X, int64_t n, int32_t d, i
             KMP_INIT_CUDA(alloc(c, &c.tc_lcnt, (size_t)n * 4), "alloc list counts");
             KMP_INIT_CUDA(alloc(c, &c.fix_rows2, n), "alloc exact-scan rows");
             KMP_INIT_CUDA(alloc(c, &c.fix_cnt2, 1), "alloc exact-scan count");
-            if (kmp::round_filter_sizes(c)) {
-                KMP_INIT_CUDA(alloc(c, &c.rf_rad2, 2 * (size_t)c.cap_total), "alloc candidate radii");
-                KMP_INIT_CUDA(alloc(c, &c.rf_num, 2 * (size_t)c.cap_total), "alloc candidate numbers");
-                KMP_INIT_CUDA(alloc(c, &c.rf_lst, (size_t)c.cap_total * 4 * tc::kListSlots), "alloc candidate lists");
-                KMP_INIT_CUDA(alloc(c, &c.rf_head, c.cap_total), "alloc candidate list heads");
-                KMP_INIT_CUDA(alloc(c, &c.rf_lcnt, tc::kListLevels), "alloc candidate list counts");
-                KMP_INIT_CUDA(alloc(c, &c.rf_rows, n), "alloc open rows");
-                KMP_INIT_CUDA(alloc(c, &c.rf_cnt, 1), "alloc open row count");
-            }
         }
         KMP_INIT_CUDA(alloc(c, &c.tc_anchor, d), "alloc anchor");
         KMP_INIT_CUDA(alloc(c, &c.tc_anchor_part, tc::tc_anchor_scratch_doubles(d)), "alloc anchor sums");
@@ -336,6 +366,10 @@ kmpar_status kmpar_init(kmpar_ctx **out, const float *X, int64_t n, int32_t d, i
         KMP_INIT_CUDA(tc::launch_prep_points(X, n, d, fmt, c.tc_anchor, c.tc_ximg, c.tc_xnorm, c.tc_xscale, c.stream),
                       "points image");
         KMP_INIT_CUDA(alloc(c, &c.fix_cnt, 1), "alloc fix-up count");
+        if (c.tc_list && kmp::round_filter_sizes(c)) {
+            KMP_INIT_CUDA(alloc_or_none(c, [&](auto take) { round_filter_buffers(c, take); }),
+                          "alloc round filter");
+        }
         KMP_INIT_CUDA(cudaMemsetAsync(c.tc_err, 0, sizeof(int), c.stream), "memset error word");
     }
     KMP_INIT_CUDA(cudaMemsetAsync(c.st, 0, sizeof(kmp::DevState), c.stream), "memset state");
@@ -411,6 +445,7 @@ kmpar_status kmpar_weight(kmpar_ctx *ctx, int64_t *m_out, const int32_t **cand_i
     if (ts != KMPAR_OK) return ts;
     c.weighted = true;
     c.m_host = st.m;
+    give_back(c, [&](auto take) { round_filter_buffers(c, take); });
     if (m_out) *m_out = st.m;
     if (cand_idx_dev) *cand_idx_dev = c.cand;
     if (w_dev) *w_dev = reinterpret_cast<const int64_t *>(c.w);
@@ -527,21 +562,24 @@ static kmpar_status ensure_lloyd_buffers(kmp::Ctx &c) {
         KMP_ENSURE(c.ll_cold, (size_t)c.k * c.d, "alloc previous centers");
         KMP_ENSURE(c.ll_drift, (size_t)c.k, "alloc center drifts");
         KMP_ENSURE(c.ll_other, (size_t)c.k, "alloc center drifts");
-        if (kmp::lloyd_lists_usable(c)) {
+        if (kmp::lloyd_lists_sizes(c)) {
             namespace tc = kmp::tc;
             const size_t cap = (size_t)std::max(c.cap_total, c.k), k128 = (size_t)((c.k + 127) / 128) * 128;
-            KMP_ENSURE(c.ll_rad2, 2 * cap, "alloc Lloyd list radii");
-            KMP_ENSURE(c.ll_num, 2 * cap, "alloc Lloyd list numbers");
-            KMP_ENSURE(c.ll_lst, cap * 4 * tc::kListSlots, "alloc Lloyd lists");
-            KMP_ENSURE(c.ll_head, cap, "alloc Lloyd list heads");
-            KMP_ENSURE(c.ll_lcnt, tc::kListLevels + 2, "alloc Lloyd list counts");
-            KMP_ENSURE(c.ll_tau2, cap, "alloc Lloyd list distances");
-            KMP_ENSURE(c.ll_img, tc::tc_points_image_bytes(c.d, c.tc_fmt, c.k), "alloc center image");
-            KMP_ENSURE(c.ll_xnorm, k128, "alloc center norms");
-            KMP_ENSURE(c.ll_xscale, k128, "alloc center scales");
-            KMP_ENSURE(c.ll_pend, (size_t)c.n, "alloc pending rows");
-            KMP_ENSURE(c.ll_flag, (size_t)c.k, "alloc cluster flags");
-            KMP_ENSURE(c.ll_pick, (size_t)kmp::pick_counts(c.n) + 1, "alloc changed row counts");
+            e = alloc_or_none(c, [&](auto take) {
+                take(c.ll_rad2, 2 * cap);
+                take(c.ll_num, 2 * cap);
+                take(c.ll_lst, cap * 4 * tc::kListSlots);
+                take(c.ll_head, cap);
+                take(c.ll_lcnt, (size_t)tc::kListLevels + 2);
+                take(c.ll_tau2, cap);
+                take(c.ll_img, tc::tc_points_image_bytes(c.d, c.tc_fmt, c.k));
+                take(c.ll_xnorm, k128);
+                take(c.ll_xscale, k128);
+                take(c.ll_pend, (size_t)c.n);
+                take(c.ll_flag, (size_t)c.k);
+                take(c.ll_pick, (size_t)kmp::pick_counts(c.n) + 1);
+            });
+            if (e != cudaSuccess) return cuda_fail(&c, e, "alloc Lloyd lists");
         }
     }
 #undef KMP_ENSURE

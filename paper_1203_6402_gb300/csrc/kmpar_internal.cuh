@@ -313,6 +313,7 @@ bool lloyd_bounds_usable(const Ctx &c, const float *C);
 cudaError_t launch_lloyd_bounded_pass(Ctx &c, const float *C, int32_t *labels, const int32_t *prev, int *changed,
                                       float *dmin);
 // the first assignment of a context that can use the bounds, by the candidates' lists
+bool lloyd_lists_sizes(const Ctx &c);
 bool lloyd_lists_usable(const Ctx &c);
 cudaError_t launch_lloyd_first_pass(Ctx &c, const float *C, int32_t *labels, int *changed, float *dmin);
 cudaError_t launch_sum_rows(const float *v, int64_t n, double *partials, int max_parts, double *out, double *copy,

@@ -2499,11 +2499,12 @@ bool lloyd_bounds_usable(const Ctx &c, const float *C) {
 // references have to be few against the rows, and the rows x centers of a dense pass
 // have to outweigh the lists' 18 launches an assignment (10 updates: 300,000 x 128,
 // k = 1,000 4.3 ms without, 4.6 with; 1,000,000 x 96, k = 2,000 8.2 and 6.3).
-bool lloyd_lists_usable(const Ctx &c) {
+bool lloyd_lists_sizes(const Ctx &c) {
     return c.precision != KMPAR_FP32 && c.tc_cimg && tc::tc_norms_in_epilogue(c.tc_fmt) && c.d % 4 == 0 &&
            resident_plan(c.k, c.d).parts == 0 && (int64_t)std::max(c.cap_total, c.k) <= c.n / 8 &&
            (double)c.n * c.k >= 1e9;
 }
+bool lloyd_lists_usable(const Ctx &c) { return lloyd_lists_sizes(c) && c.ll_pick; }
 
 __global__ void set_int_kernel(int *p, int v) { *p = v; }
 
