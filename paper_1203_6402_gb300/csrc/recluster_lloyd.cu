@@ -858,14 +858,16 @@ __global__ void __launch_bounds__(1024) base_scan_kernel(int32_t *tot_base, int 
 }
 
 // one warp per sort block: stable scatter of point numbers into label order
-// (the rows are 0 .. n - 1, or `rows`)
+// (PICKED: *n_dev rows, those of `rows`; else 0 .. n - 1.  A run-time choice inside the loop
+// read 16.8 us against 12.8 without it, over 1.25M rows.)
+template <bool PICKED>
 __global__ void __launch_bounds__(32) scatter_kernel(const int32_t *__restrict__ labels,
                                                      const int32_t *__restrict__ rows, int64_t n, const int *n_dev,
                                                      int k, int sb, const int32_t *__restrict__ hist,
                                                      const int32_t *__restrict__ base, int32_t *perm) {
     extern __shared__ int32_t cur[];
     const int lane = threadIdx.x;
-    if (n_dev) {
+    if (PICKED) {
         n = *n_dev;
         if ((int64_t)blockIdx.x * sb >= n) return;   // uniform per block
     }
@@ -879,7 +881,7 @@ __global__ void __launch_bounds__(32) scatter_kernel(const int32_t *__restrict__
         const int l = valid ? labels[i] : -1;
         const unsigned mask = __match_any_sync(0xffffffffu, l);
         const int rank = __popc(mask & ((1u << lane) - 1u));
-        if (valid) perm[cur[l] + rank] = rows ? rows[i] : (int32_t)i;
+        if (valid) perm[cur[l] + rank] = PICKED ? rows[i] : (int32_t)i;
         __syncwarp();
         if (valid && lane == __ffs(mask) - 1) cur[l] += __popc(mask);
         __syncwarp();
@@ -1138,8 +1140,8 @@ cudaError_t launch_centroids(Ctx &c, const int32_t *labels, const int32_t *befor
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     base_scan_kernel<<<1, 1024, 0, c.stream>>>(c.base, k, c.piece);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    scatter_kernel<<<c.nsb, 32, sizeof(int32_t) * k, c.stream>>>(lab, rows, c.n, n_dev, k, sb, c.hist, c.base,
-                                                                  c.perm);
+    auto scatter = rows ? scatter_kernel<true> : scatter_kernel<false>;
+    scatter<<<c.nsb, 32, sizeof(int32_t) * k, c.stream>>>(lab, rows, c.n, n_dev, k, sb, c.hist, c.base, c.perm);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // coordinate pairs need 8-byte aligned rows: d even and X 8-byte aligned
     const int pairs = (c.d % 2 == 0) && (reinterpret_cast<uintptr_t>(c.X) % 8 == 0);
@@ -1165,7 +1167,10 @@ cudaError_t configure_kernels(int max_sort_pow2, int k) {
         if ((e = cudaFuncSetAttribute(label_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
             cudaSuccess)
             return e;
-        if ((e = cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
+        if ((e = cudaFuncSetAttribute(scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
+            cudaSuccess)
+            return e;
+        if ((e = cudaFuncSetAttribute(scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
             cudaSuccess)
             return e;
     }
