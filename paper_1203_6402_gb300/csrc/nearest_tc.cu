@@ -452,7 +452,9 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restr
 
 // After a list pass over references (position i of the pass = reference rin_num[i], or i):
 // a reference whose lists hold gets head {entries, squared radius} and its entries in
-// one run; one that overflowed goes to the next pass (its image row, scale, number,
+// one run (pad columns of the last center tile, numbers from the center count on, are
+// dropped: their norm is finite, so a large enough reach lists them); one that overflowed
+// goes to the next pass (its image row, scale, number,
 // radius and threshold to the next position there) with half the radius, or, when there
 // is none (cout null), gets a negative radius: no row of it is covered.  One warp per
 // reference.
@@ -461,10 +463,11 @@ __global__ void __launch_bounds__(256) list_level_kernel(
     const int32_t *__restrict__ lst, const int32_t *__restrict__ lcnt, const uint8_t *__restrict__ img,
     const float *__restrict__ scale, int KA, int d, const int32_t *__restrict__ cand,
     const float *__restrict__ xnorm, const float *__restrict__ tau2, const unsigned int *cmax_bits, float ep, float en,
-    float ec, int32_t *glst, int2 *ghead, int *cnt_out, int32_t *cout, unsigned int *rout, uint8_t *img_out, float *scale_out, float *thr_out) {
+    float ec, const DevState *batch, int centers, int32_t *glst, int2 *ghead, int *cnt_out, int32_t *cout, unsigned int *rout, uint8_t *img_out, float *scale_out, float *thr_out) {
     const int lane = threadIdx.x & 31;
     const int nw = (int)((gridDim.x * blockDim.x) >> 5);
     const int total = *cnt;
+    const int ncol = batch ? batch->batch_cnt : centers;   // real columns of the pass
     const float W = fp32_tie_window(d);
     const float cmax = __uint_as_float(*cmax_bits);
     for (int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); i < total; i += nw) {
@@ -477,7 +480,7 @@ __global__ void __launch_bounds__(256) list_level_kernel(
             const int g = lane >> 3, e = lane & 7;
             const int n = g == 0 ? c.x : g == 1 ? c.y : g == 2 ? c.z : c.w;
             const int v = e < n ? lst[(size_t)i * 4 * kListSlots + lane] : -1;
-            const bool keep = v >= 0 && (cand || v != a);
+            const bool keep = v >= 0 && v < ncol && (cand || v != a);
             const unsigned m = __ballot_sync(0xffffffffu, keep);
             if (keep) glst[(size_t)a * 4 * kListSlots + __popc(m & ((1u << lane) - 1u))] = v;
             if (lane == 0) ghead[a] = make_int2(__popc(m), __float_as_int(r2));
@@ -679,7 +682,7 @@ cudaError_t launch_reference_lists(TcParams p, int mode_round, const ListBufs &b
         if ((e = launch_nearest_tc(p, mode_round, EPI_LIST, num_sms, s)) != cudaSuccess) return e;
         list_level_kernel<<<num_sms * 4, 256, 0, s>>>(
             p.nrows_dev, l == 0 ? nullptr : num[h], rad[h], p.lst, p.lcnt, img[h], scale[h], KA, p.d, cand, xnorm, tau2,
-            p.cmax_bits, ep, en, ec, b.glst, b.ghead, last ? nullptr : b.cnt + l + 1, last ? nullptr : num[h ^ 1],
+            p.cmax_bits, ep, en, ec, mode_round ? p.st : nullptr, p.cnt, b.glst, b.ghead, last ? nullptr : b.cnt + l + 1, last ? nullptr : num[h ^ 1],
             rad[h ^ 1], img[h ^ 1], scale[h ^ 1], thr[h ^ 1]);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
