@@ -389,10 +389,11 @@ __global__ void __launch_bounds__(256) anchor_final_kernel(const double *__restr
 // above ub (1 + 2 W) (see the list refine).
 // list threshold of a row whose nearest distance is at most u (exact FP32): every
 // center whose screened value exceeds it is provably farther than the nearest one
-// (twice the screening bound plus the FP32 tie window); +inf without a bound
+// (twice the screening bound plus the FP32 tie window); +inf without a bound; NaN or
+// infinite when a norm is
 __device__ __forceinline__ float list_threshold(float u, float xnorm, float cmax, float ep, float en, float ec,
                                                 float W) {
-    const float xn = fmaxf(xnorm, 0.f);
+    const float xn = xnorm < 0.f ? 0.f : xnorm;   // (a NaN stays one)
     const float X = sqrtf(xn);
     float t = __uint_as_float(0x7F800000u);
     if (u < FLT_MAX) {
@@ -454,16 +455,19 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restr
 // a reference whose lists hold gets head {entries, squared radius} and its entries in
 // one run (pad columns of the last center tile, numbers from the center count on, are
 // dropped: their norm is finite, so a large enough reach lists them); one that overflowed
-// goes to the next pass (its image row, scale, number,
-// radius and threshold to the next position there) with half the radius, or, when there
-// is none (cout null), gets a negative radius: no row of it is covered.  One warp per
-// reference.
+// goes to the next pass (its image row, scale, number, radius and threshold to the next
+// position there) with half the radius, or, when there is none (cout null), gets a negative radius: no row of it is covered.  Nor is one whose
+// threshold is not finite: a norm beyond FP32 makes it NaN or infinite, and what passed
+// it says nothing (NaN passes no value, and an empty list would read as a complete one).
+// A finite threshold implies finite norms of the reference and of every center.  One warp
+// per reference.
 __global__ void __launch_bounds__(256) list_level_kernel(
     const int *cnt, const int32_t *__restrict__ cin, const unsigned int *__restrict__ rin,
     const int32_t *__restrict__ lst, const int32_t *__restrict__ lcnt, const uint8_t *__restrict__ img,
-    const float *__restrict__ scale, int KA, int d, const int32_t *__restrict__ cand,
+    const float *__restrict__ scale, const float *__restrict__ thr, int KA, int d, const int32_t *__restrict__ cand,
     const float *__restrict__ xnorm, const float *__restrict__ tau2, const unsigned int *cmax_bits, float ep, float en,
-    float ec, const DevState *batch, int centers, int32_t *glst, int2 *ghead, int *cnt_out, int32_t *cout, unsigned int *rout, uint8_t *img_out, float *scale_out, float *thr_out) {
+    float ec, const DevState *batch, int centers, int32_t *glst, int2 *ghead, int *cnt_out, int32_t *cout,
+    unsigned int *rout, uint8_t *img_out, float *scale_out, float *thr_out) {
     const int lane = threadIdx.x & 31;
     const int nw = (int)((gridDim.x * blockDim.x) >> 5);
     const int total = *cnt;
@@ -473,8 +477,9 @@ __global__ void __launch_bounds__(256) list_level_kernel(
     for (int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); i < total; i += nw) {
         const int a = cin ? cin[i] : i;
         const float r2 = __uint_as_float(rin[i]);
+        const bool finite = fabsf(thr[i]) <= FLT_MAX;
         const int4 c = __ldg(reinterpret_cast<const int4 *>(lcnt) + i);
-        if (max(max(c.x, c.y), max(c.z, c.w)) <= kListSlots) {
+        if (finite && max(max(c.x, c.y), max(c.z, c.w)) <= kListSlots) {
             // lane l: entry l % 8 of column group l / 8; references that are the centers
             // themselves (cand null) are left off their own lists
             const int g = lane >> 3, e = lane & 7;
@@ -486,7 +491,7 @@ __global__ void __launch_bounds__(256) list_level_kernel(
             if (lane == 0) ghead[a] = make_int2(__popc(m), __float_as_int(r2));
             continue;
         }
-        if (!cout) {
+        if (!cout || !finite) {
             if (lane == 0) ghead[a] = make_int2(0, __float_as_int(-1.f));
             continue;
         }
@@ -681,9 +686,10 @@ cudaError_t launch_reference_lists(TcParams p, int mode_round, const ListBufs &b
         p.nrows_dev = l == 0 ? cnt : b.cnt + l;
         if ((e = launch_nearest_tc(p, mode_round, EPI_LIST, num_sms, s)) != cudaSuccess) return e;
         list_level_kernel<<<num_sms * 4, 256, 0, s>>>(
-            p.nrows_dev, l == 0 ? nullptr : num[h], rad[h], p.lst, p.lcnt, img[h], scale[h], KA, p.d, cand, xnorm, tau2,
-            p.cmax_bits, ep, en, ec, mode_round ? p.st : nullptr, p.cnt, b.glst, b.ghead, last ? nullptr : b.cnt + l + 1, last ? nullptr : num[h ^ 1],
-            rad[h ^ 1], img[h ^ 1], scale[h ^ 1], thr[h ^ 1]);
+            p.nrows_dev, l == 0 ? nullptr : num[h], rad[h], p.lst, p.lcnt, img[h], scale[h], thr[h], KA, p.d, cand,
+            xnorm, tau2, p.cmax_bits, ep, en, ec, mode_round ? p.st : nullptr, p.cnt, b.glst, b.ghead,
+            last ? nullptr : b.cnt + l + 1, last ? nullptr : num[h ^ 1], rad[h ^ 1], img[h ^ 1], scale[h ^ 1],
+            thr[h ^ 1]);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

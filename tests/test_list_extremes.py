@@ -68,3 +68,21 @@ def test_columns_beyond_the_centers_stay_off_the_lists(d, prec):
     C0 = X[torch.randperm(len(X), generator=torch.Generator().manual_seed(3))[:4093].cuda()].contiguous()
     C0[7] = X[0]   # a center at the mean, whatever the draw
     _same_lloyd(X, C0, 5, prec)
+
+
+# rows whose norm, or whose share of the mean, is beyond FP32: no screened value of theirs
+# says anything, and no list may take that for "no center is near"
+@pytest.mark.gpu
+@pytest.mark.parametrize("value", [1e20, 1e30, float("inf"), float("nan")])
+@pytest.mark.parametrize("d,prec", [(64, "bf16"), (128, "bf16"), (20, "fp8"), (96, "fp8")])
+def test_lists_without_finite_thresholds_cover_no_row(d, prec, value):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    X = datagen.gauss_mixture(250_007, d, 4093, 10.0, 4)
+    X[1234] = value
+    Xd = torch.from_numpy(np.ascontiguousarray(X)).cuda()
+    _same_rounds(Xd, 300, 1000.0, 4, prec, "bernoulli")
+    C0 = Xd[torch.randperm(len(X), generator=torch.Generator().manual_seed(5))[:4093].cuda()].contiguous()
+    if np.isfinite(value):
+        C0[11] = Xd[1234]   # the row is a center, as step 8 makes it
+    _same_lloyd(Xd, C0, 5, prec)
