@@ -195,17 +195,10 @@ void free_ctx(kmp::Ctx &c) {
         if (b) cudaFreeAsync(b, c.stream);
 }
 
-int sort_pow2(int cap) {
-    int P = 1;
-    while (P < cap) P <<= 1;
-    return P;
-}
-
 }  // namespace
 
 namespace kmp {
-// kernels configured once per process (dynamic shared memory above 48 KB)
-cudaError_t configure_kernels(int max_sort_pow2, int k);
+cudaError_t configure_kernels();   // limits of dynamic shared memory
 
 std::atomic<long long> g_launches{0};
 
@@ -314,7 +307,7 @@ kmpar_status kmpar_init(kmpar_ctx **out, const float *X, int64_t n, int32_t d, i
     if ((e = (expr)) != cudaSuccess) return bail(cuda_fail(&c, e, where))
     KMP_INIT_CUDA(cudaGetDevice(&c.dev), "cudaGetDevice");
     KMP_INIT_CUDA(cudaDeviceGetAttribute(&c.num_sms, cudaDevAttrMultiProcessorCount, c.dev), "sm count");
-    KMP_INIT_CUDA(kmp::configure_kernels(sort_pow2(cap_round), k), "configure kernels");
+    KMP_INIT_CUDA(kmp::configure_kernels(), "configure kernels");
     KMP_INIT_CUDA(alloc(c, &c.st, 1), "alloc state");
     KMP_INIT_CUDA(alloc(c, &c.D2, n), "alloc D2");
     KMP_INIT_CUDA(alloc(c, &c.idx, n), "alloc idx");
@@ -593,7 +586,7 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
     kmp::Ctx &c = ctx->c;
     if (!centers_dev) return fail(&c, KMPAR_ERR_ARG, "centers_dev is NULL");
     if (max_iter < 0) return fail(&c, KMPAR_ERR_ARG, "max_iter < 0");
-    if (c.k > 49152) return fail(&c, KMPAR_ERR_UNSUPPORTED, "Lloyd supports k <= 49152");
+    if (c.k > kmp::kMaxLloydK) return fail(&c, KMPAR_ERR_UNSUPPORTED, "Lloyd supports k <= 49152");
     kmpar_status s = ensure_lloyd_buffers(c);
     if (s != KMPAR_OK) return s;
     // At a fixed point an iteration changes nothing (the same labels give the same

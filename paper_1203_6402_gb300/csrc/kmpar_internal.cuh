@@ -20,6 +20,7 @@ constexpr uint32_t TAG_RECLUSTER = 3u;
 
 constexpr int kMaxRoundCap = 32768;   // single-CTA sort of one round's draws
 constexpr int kMaxRounds = 64;
+constexpr int kMaxLloydK = 49152;     // label counters of one block in shared memory
 
 // Device-resident state of one context (one allocation, read by kernels).
 struct DevState {

@@ -32,6 +32,9 @@ __host__ __device__ __forceinline__ uint32_t sw128_off(int r, int c) {
     return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4));
 }
 
+// the refine and fix-up kernels size their shared-memory rows for d <= 190
+constexpr int kMaxD = 190;
+
 // ------------------------------------------------------------------ operand encoding
 __device__ __forceinline__ __nv_bfloat16 bf(float v) { return __float2bfloat16_rn(v); }
 __device__ __forceinline__ uint8_t e4m3(float v) {
@@ -252,6 +255,7 @@ __global__ void __launch_bounds__(256) prep_centers_ne_kernel(const float *__res
 // 1e7 x 128 for BF16 (kmpar_init as a whole) takes 7.1 ms; 14.6 ms with a thread a row,
 // whose reads of one bank queued.
 constexpr int kPrepWarps = 8, kPrepRows = 8;
+constexpr size_t prep_smem(int d) { return sizeof(float) * kPrepWarps * kPrepRows * (size_t)(d | 1); }
 
 template <int fmt>
 __global__ void __launch_bounds__(32 * kPrepWarps) prep_points_kernel(const float *__restrict__ X, int64_t n,
@@ -538,8 +542,7 @@ int tc_katoms(int d, int fmt) { return (k_bytes(d, fmt) + 127) / 128; }
 int tc_ksteps(int d, int fmt) { return (k_bytes(d, fmt) + 31) / 32; }
 int tc_block_n(int d, int fmt) { return tc_katoms(d, fmt) <= 2 ? 256 : 128; }
 bool tc_norms_in_epilogue(int fmt) { return fmt == FMT_BF16N || fmt == FMT_FP8; }
-// the refine and fix-up kernels size their shared-memory rows for d <= 190
-bool tc_supported(int d, int fmt) { return fmt >= 0 && d >= 1 && d <= 190 && tc_katoms(d, fmt) <= 3; }
+bool tc_supported(int d, int fmt) { return fmt >= 0 && d >= 1 && d <= kMaxD && tc_katoms(d, fmt) <= 3; }
 
 size_t tc_points_image_bytes(int d, int fmt, int64_t n) {
     const int64_t tiles = (n + BM - 1) / BM;
@@ -560,11 +563,12 @@ cudaError_t launch_prep_points(const float *X, int64_t n, int d, int fmt, const 
     const int64_t n_pad = ((n + BM - 1) / BM) * BM;
     const int64_t blocks = n_pad / (kPrepWarps * kPrepRows);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, 8192));
-    const size_t sm = sizeof(float) * kPrepWarps * kPrepRows * (size_t)(d | 1);
     auto go = [&](auto kern) -> cudaError_t {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        // (the same limit in every call: it belongs to the process)
+        const cudaError_t e =
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prep_smem(kMaxD));
         if (e != cudaSuccess) return e;
-        kern<<<grid, 32 * kPrepWarps, sm, s>>>(X, n, n_pad, d, tc_katoms(d, fmt), anchor, img, xnorm, xscale);
+        kern<<<grid, 32 * kPrepWarps, prep_smem(d), s>>>(X, n, n_pad, d, tc_katoms(d, fmt), anchor, img, xnorm, xscale);
         return cudaGetLastError();
     };
     cudaError_t e = cudaErrorInvalidValue;

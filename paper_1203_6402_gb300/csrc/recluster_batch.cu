@@ -521,11 +521,12 @@ cudaError_t launch_recluster_batch(Ctx &c, float *centers) {
     // in the chunk-mass buffer (2 nchunk + 2048 doubles)
     float2 *gch = reinterpret_cast<float2 *>(c.rc_cmass);
     float2 *gincl = gch + nchunk;
-    const size_t acc_smem = sizeof(float) * ((size_t)P * P + 4 * P) + sizeof(int) * 2 * P;
+    auto accept_smem = [](size_t P) { return sizeof(float) * (P * P + 4 * P) + sizeof(int) * 2 * P; };
+    const size_t acc_smem = accept_smem(P);
     auto upd = c.d % 4 == 0 ? rs_update_kernel<false, true> : rs_update_kernel<false, false>;
-    if (acc_smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(rs_accept_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)acc_smem)) != cudaSuccess)
+    // (the same limit in every call: it belongs to the process)
+    if ((e = cudaFuncSetAttribute(rs_accept_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)accept_smem(kRsMaxProposals))) != cudaSuccess)
         return e;
     if ((e = cudaMemsetAsync(ctl, 0, sizeof(RsCtl), c.stream)) != cudaSuccess) return e;
     const int pgrid = (P + kPropWarps - 1) / kPropWarps;

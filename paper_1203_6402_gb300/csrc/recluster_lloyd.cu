@@ -612,9 +612,9 @@ cudaError_t launch_recluster_grid(Ctx &c, float *centers) {
     int qs = (int)((budget - base_smem) / (sizeof(float) * (size_t)cpc_cap * 32));
     qs = std::max(0, std::min(qs, c.d));
     const size_t smem = base_smem + sizeof(float) * (size_t)qs * cpc_cap * 32;
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(recluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
+    // (the same limit in every call: it belongs to the process)
+    if ((e = cudaFuncSetAttribute(recluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget)) !=
+        cudaSuccess)
         return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, recluster_kernel, kRcThreads, smem)) !=
@@ -1157,23 +1157,20 @@ cudaError_t launch_centroids(Ctx &c, const int32_t *labels, const int32_t *befor
 }  // namespace kmp
 
 namespace kmp {
-cudaError_t configure_round_kernels(int max_sort_pow2);
+cudaError_t configure_round_kernels();
 
-cudaError_t configure_kernels(int max_sort_pow2, int k) {
-    cudaError_t e = configure_round_kernels(max_sort_pow2);
+// Limits of dynamic shared memory belong to the process: each kernel gets its largest size,
+// not this context's, which could be below what another context launches with.
+cudaError_t configure_kernels() {
+    cudaError_t e = configure_round_kernels();
     if (e != cudaSuccess) return e;
-    const int hist_bytes = (int)sizeof(int32_t) * std::min(k, 49152);
-    if (hist_bytes > 48 * 1024) {
-        if ((e = cudaFuncSetAttribute(label_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
-            cudaSuccess)
-            return e;
-        if ((e = cudaFuncSetAttribute(scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
-            cudaSuccess)
-            return e;
-        if ((e = cudaFuncSetAttribute(scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
-            cudaSuccess)
-            return e;
-    }
-    return cudaSuccess;
+    const int hist_bytes = (int)sizeof(int32_t) * kMaxLloydK;
+    if ((e = cudaFuncSetAttribute(label_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
+        cudaSuccess)
+        return e;
+    if ((e = cudaFuncSetAttribute(scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes)) !=
+        cudaSuccess)
+        return e;
+    return cudaFuncSetAttribute(scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hist_bytes);
 }
 }  // namespace kmp

@@ -420,27 +420,38 @@ static int scan_rows(int64_t n, int d) { return d > 32 && n <= 40000 ? 32 : 128;
 
 int assign_num_partials(int64_t n, int d) { return (int)((n + scan_rows(n, d) - 1) / scan_rows(n, d)); }
 
+// dynamic shared memory of a tile kernel at d coordinates: rows (two buffers in steps) and
+// two buffers of centers
+constexpr size_t tile_smem(int d, int BM, int BN) {
+    return sizeof(float) * (d <= kTileK ? d * (BM + 4 + 2 * (BN + 4)) : kTileChunk * 2 * (BM + 4 + BN + 4));
+}
+
+template <int MODE, int BM, int TN>
+static cudaError_t launch_tiles(const NearestParams &p, int grid, cudaStream_t s) {
+    constexpr size_t at_k = tile_smem(kTileK, BM, 8 * TN), steps = tile_smem(kTileK + 1, BM, 8 * TN);
+    constexpr size_t most = at_k > steps ? at_k : steps;
+    // the limit belongs to the process: always the kernel's largest size, whatever this
+    // call takes, so that no call lowers it under another one
+    if (most > 40 * 1024) {   // (the static shared memory counts too)
+        const cudaError_t e = cudaFuncSetAttribute(nearest_tile_kernel<MODE, BM, TN>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+        if (e != cudaSuccess) return e;
+    }
+    nearest_tile_kernel<MODE, BM, TN><<<grid, 2 * BM, tile_smem(p.d, BM, 8 * TN), s>>>(p, p.d <= kTileK ? p.d : kTileChunk);
+    return cudaGetLastError();
+}
+
 template <int MODE>
 static cudaError_t launch_nearest_mode(const NearestParams &p, int cnt_hint, cudaStream_t s) {
     const int grid = assign_num_partials(p.n, p.d);   // p.n = rows capacity for row lists
-    const int kc = p.d <= kTileK ? p.d : kTileChunk;
     const bool small = scan_rows(p.n, p.d) == 32, narrow = cnt_hint <= 32;
-    const size_t smem = sizeof(float) * kc * ((p.d <= kTileK ? 1 : 2) * (small ? 36 : 132) + 2 * (narrow ? 36 : 68));
-    auto tiles = [&](auto kern, int threads) -> cudaError_t {
-        if (smem > 40 * 1024) {   // (the static shared memory counts too)
-            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        kern<<<grid, threads, smem, s>>>(p, kc);
-        return cudaGetLastError();
-    };
     count_launches(1);
     if (p.d <= 4) nearest_kernel<4, MODE><<<grid, kNearThreads, 0, s>>>(p);
     else if (p.d <= 8) nearest_kernel<8, MODE><<<grid, kNearThreads, 0, s>>>(p);
     else if (p.d <= 16) nearest_kernel<16, MODE><<<grid, kNearThreads, 0, s>>>(p);
     else if (p.d <= 32) nearest_kernel<32, MODE><<<grid, kNearThreads, 0, s>>>(p);
-    else if (small) return narrow ? tiles(nearest_tile_kernel<MODE, 32, 4>, 64) : tiles(nearest_tile_kernel<MODE, 32, 8>, 64);
-    else return narrow ? tiles(nearest_tile_kernel<MODE, 128, 4>, 256) : tiles(nearest_tile_kernel<MODE, 128, 8>, 256);
+    else if (small) return narrow ? launch_tiles<MODE, 32, 4>(p, grid, s) : launch_tiles<MODE, 32, 8>(p, grid, s);
+    else return narrow ? launch_tiles<MODE, 128, 4>(p, grid, s) : launch_tiles<MODE, 128, 8>(p, grid, s);
     return cudaGetLastError();
 }
 
@@ -762,9 +773,9 @@ cudaError_t launch_uniforms(int64_t count, uint32_t round, uint32_t tag, uint64_
 namespace kmp {
 cudaError_t configure_refine_kernels();
 
-cudaError_t configure_round_kernels(int max_sort_pow2) {
+cudaError_t configure_round_kernels() {
     cudaError_t e = cudaFuncSetAttribute(sort_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         max_sort_pow2 * (int)sizeof(int32_t));
+                                         kMaxRoundCap * (int)sizeof(int32_t));
     if (e != cudaSuccess) return e;
     return configure_refine_kernels();
 }
@@ -2056,8 +2067,9 @@ __global__ void __launch_bounds__(256) refine_group_kernel(GroupArgs g) {
 }
 
 // warps per CTA: about 100 KB of staged rows a CTA, two CTAs on an SM
+constexpr unsigned kStageSmem = 108u * 1024u;
 int stage_warps(int d) {
-    const int w = (int)((108u * 1024u) / (64u * 16u * (unsigned)stage_stride4(d) + kStageExtra));
+    const int w = (int)(kStageSmem / (64u * 16u * (unsigned)stage_stride4(d) + kStageExtra));
     return w < 1 ? 1 : (w > 8 ? 8 : w);
 }
 size_t stage_smem_bytes(int d) { return (size_t)stage_warps(d) * (64 * 16 * stage_stride4(d) + kStageExtra); }
@@ -2065,8 +2077,9 @@ size_t stage_smem_bytes(int d) { return (size_t)stage_warps(d) * (64 * 16 * stag
 // a kernel of the staged kind over n rows: persistent, two CTAs an SM
 template <typename K, typename A>
 static cudaError_t launch_staged(K kern, const Ctx &c, int64_t n, const A &args) {
-    const size_t smem = stage_smem_bytes(c.d);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = stage_smem_bytes(c.d);   // at most kStageSmem up to d = 424
+    // (the same limit in every call: it belongs to the process)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStageSmem);
     if (e != cudaSuccess) return e;
     const int sw = stage_warps(c.d);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n + 32 * sw - 1) / (32 * sw), 2 * (int64_t)c.num_sms));
