@@ -163,6 +163,25 @@ void round_filter_buffers(kmp::Ctx &c, T take) {
     take(c.rf_cnt, (size_t)1);
 }
 
+// Lloyd's lists; see ensure_lloyd_buffers
+template <typename T>
+void lloyd_list_buffers(kmp::Ctx &c, T take) {
+    namespace tc = kmp::tc;
+    const size_t cap = (size_t)std::max(c.cap_total, c.k), k128 = (size_t)((c.k + 127) / 128) * 128;
+    take(c.ll_rad2, 2 * cap);
+    take(c.ll_num, 2 * cap);
+    take(c.ll_lst, cap * 4 * tc::kListSlots);
+    take(c.ll_head, cap);
+    take(c.ll_lcnt, (size_t)tc::kListLevels + 2);
+    take(c.ll_tau2, cap);
+    take(c.ll_img, tc::tc_points_image_bytes(c.d, c.tc_fmt, c.k));
+    take(c.ll_xnorm, k128);
+    take(c.ll_xscale, k128);
+    take(c.ll_pend, (size_t)c.n);
+    take(c.ll_flag, (size_t)c.k);
+    take(c.ll_pick, (size_t)kmp::pick_counts(c.n) + 1);
+}
+
 // Buffers that only make a pass faster: all of them, or, when the memory is short, none
 // (the context then keeps the passes that do without).  request(take): take(p, count) on each.
 template <typename F>
@@ -177,6 +196,19 @@ cudaError_t alloc_or_none(kmp::Ctx &c, F request) {
         e = cudaSuccess;
     }
     return e;
+}
+
+// A buffer that a call cannot do without, asked for after the context may have taken
+// such optional ones: where it is refused they are given back first, so that what runs
+// without them is not refused for their sake.
+template <typename T>
+cudaError_t alloc_needed(kmp::Ctx &c, T **p, size_t count) {
+    const cudaError_t e = alloc(c, p, count);
+    if (e != cudaErrorMemoryAllocation || !(c.rf_rows || c.ll_pick)) return e;
+    (void)cudaGetLastError();
+    give_back(c, [&](auto take) { round_filter_buffers(c, take); });
+    give_back(c, [&](auto take) { lloyd_list_buffers(c, take); });
+    return alloc(c, p, count);
 }
 
 void free_ctx(kmp::Ctx &c) {
@@ -412,13 +444,13 @@ kmpar_status kmpar_set_sampling(kmpar_ctx *ctx, int32_t mode) {
         return fail(&c, KMPAR_ERR_ARG, "exactly-l rounds need l >= 1");
     if (mode == KMPAR_SAMPLE_EXACT) {
         // each buffer once; after a failed call the next one allocates what is missing
-        if (!c.ex_keys) KMP_CUDA(&c, alloc(c, &c.ex_keys, (size_t)c.n), "alloc clocks");
+        if (!c.ex_keys) KMP_CUDA(&c, alloc_needed(c, &c.ex_keys, (size_t)c.n), "alloc clocks");
         if (!c.ex_ws) {
             unsigned char *ws = nullptr;
-            KMP_CUDA(&c, alloc(c, &ws, kmp::exact_work_bytes()), "alloc select state");
+            KMP_CUDA(&c, alloc_needed(c, &ws, kmp::exact_work_bytes()), "alloc select state");
             c.ex_ws = ws;
         }
-        if (!c.ex_ties) KMP_CUDA(&c, alloc(c, &c.ex_ties, (size_t)kmp::exact_tie_cap()), "alloc tie list");
+        if (!c.ex_ties) KMP_CUDA(&c, alloc_needed(c, &c.ex_ties, (size_t)kmp::exact_tie_cap()), "alloc tie list");
     }
     c.sampling = mode == KMPAR_SAMPLE_EXACT ? 1 : 0;
     return KMPAR_OK;
@@ -469,14 +501,14 @@ kmpar_status kmpar_recluster(kmpar_ctx *ctx, float *centers_dev) {
         if (c.rCT) cudaFreeAsync(c.rCT, c.stream);
         c.alloc_bytes -= (sizeof(float) * c.rCT_floats + 255) & ~(size_t)255;
         c.rCT_floats = 0;
-        const cudaError_t e = alloc(c, &c.rCT, nf);
+        const cudaError_t e = plan.cs > 0 ? alloc(c, &c.rCT, nf) : alloc_needed(c, &c.rCT, nf);
         if (e == cudaSuccess) c.rCT_floats = nf;
         else if (plan.cs == 0) return cuda_fail(&c, e, "alloc transposed candidates");
         else cudaGetLastError();
     }
     if (c.rs_batch > 0 && !c.rs_buf) {
         unsigned char *b = nullptr;
-        KMP_CUDA(&c, alloc(c, &b, kmp::recluster_batch_bytes()), "alloc batched recluster buffer");
+        KMP_CUDA(&c, alloc_needed(c, &b, kmp::recluster_batch_bytes()), "alloc batched recluster buffer");
         c.rs_buf = b;
     }
     KMP_CUDA(&c, cudaMemsetAsync(&c.st->warn, 0, sizeof(int32_t), c.stream), "memset warn");
@@ -504,7 +536,7 @@ kmpar_status kmpar_weighted_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t ma
     if (!c.weighted) return fail(&c, KMPAR_ERR_STATE, "weighted Lloyd before weight");
     if (c.d > 4096) return fail(&c, KMPAR_ERR_UNSUPPORTED, "weighted Lloyd supports d <= 4096");
     for (int b = 0; b < 2; ++b)
-        if (!c.wl_lab[b]) KMP_CUDA(&c, alloc(c, &c.wl_lab[b], (size_t)c.cap_total), "alloc candidate labels");
+        if (!c.wl_lab[b]) KMP_CUDA(&c, alloc_needed(c, &c.wl_lab[b], (size_t)c.cap_total), "alloc candidate labels");
     int32_t m = 0;
     KMP_CUDA(&c, cudaMemcpyAsync(&m, &c.st->m, sizeof(m), cudaMemcpyDeviceToHost, c.stream), "read m");
     KMP_CUDA(&c, cudaStreamSynchronize(c.stream), "sync");
@@ -536,7 +568,7 @@ static kmpar_status ensure_lloyd_buffers(kmp::Ctx &c) {
     if (c.lloyd_ready) return KMPAR_OK;
     cudaError_t e;
 #define KMP_ENSURE(ptr, count, what) \
-    if (!(ptr) && (e = alloc(c, &(ptr), (count))) != cudaSuccess) return cuda_fail(&c, e, what)
+    if (!(ptr) && (e = alloc_needed(c, &(ptr), (count))) != cudaSuccess) return cuda_fail(&c, e, what)
     KMP_ENSURE(c.labels[0], (size_t)c.n, "alloc labels");
     KMP_ENSURE(c.labels[1], (size_t)c.n, "alloc labels");
     KMP_ENSURE(c.perm, (size_t)c.n, "alloc perm");
@@ -556,22 +588,7 @@ static kmpar_status ensure_lloyd_buffers(kmp::Ctx &c) {
         KMP_ENSURE(c.ll_drift, (size_t)c.k, "alloc center drifts");
         KMP_ENSURE(c.ll_other, (size_t)c.k, "alloc center drifts");
         if (kmp::lloyd_lists_sizes(c)) {
-            namespace tc = kmp::tc;
-            const size_t cap = (size_t)std::max(c.cap_total, c.k), k128 = (size_t)((c.k + 127) / 128) * 128;
-            e = alloc_or_none(c, [&](auto take) {
-                take(c.ll_rad2, 2 * cap);
-                take(c.ll_num, 2 * cap);
-                take(c.ll_lst, cap * 4 * tc::kListSlots);
-                take(c.ll_head, cap);
-                take(c.ll_lcnt, (size_t)tc::kListLevels + 2);
-                take(c.ll_tau2, cap);
-                take(c.ll_img, tc::tc_points_image_bytes(c.d, c.tc_fmt, c.k));
-                take(c.ll_xnorm, k128);
-                take(c.ll_xscale, k128);
-                take(c.ll_pend, (size_t)c.n);
-                take(c.ll_flag, (size_t)c.k);
-                take(c.ll_pick, (size_t)kmp::pick_counts(c.n) + 1);
-            });
+            e = alloc_or_none(c, [&](auto take) { lloyd_list_buffers(c, take); });
             if (e != cudaSuccess) return cuda_fail(&c, e, "alloc Lloyd lists");
         }
     }
@@ -600,7 +617,7 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
         c.lloyd_rec = nullptr;
         c.lloyd_rec_cap = 0;
         Rec *r = nullptr;
-        KMP_CUDA(&c, alloc(c, &r, (size_t)(max_iter + 1)), "alloc Lloyd records");
+        KMP_CUDA(&c, alloc_needed(c, &r, (size_t)(max_iter + 1)), "alloc Lloyd records");
         c.lloyd_rec = r;
         c.lloyd_rec_cap = max_iter + 1;
     }
