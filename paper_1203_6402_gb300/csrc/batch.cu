@@ -160,6 +160,9 @@ __device__ __forceinline__ void take_better(double v, int j, double &best, int &
 // a distance known to be at most / at least the real one, from an exact FP32 square
 __device__ __forceinline__ float upper_of(float v, float W) { return sqrtf(v * (1.f + W)) * (1.f + 1e-6f); }
 __device__ __forceinline__ float lower_of(float v, float W) { return sqrtf(v * (1.f - 2.f * W)) * (1.f - 1e-6f); }
+// ... of the runner-up v (center j; j < 0: the squares of all others are beyond FP32, which
+// puts them that far and no farther)
+__device__ __forceinline__ float runner_up(float v, int j, float W) { return lower_of(j >= 0 ? v : FLT_MAX, W); }
 
 // Shared state of one block.
 template <int DP>
@@ -309,7 +312,7 @@ __device__ __forceinline__ void row_decide(const BPass &p, int64_t pt, float m1,
         }
         p.lab[pt] = l;
         p.dm[pt] = stored;
-        p.lb[pt] = n2 >= 0 ? lower_of(l == n1 ? m2 : m1, W) : FLT_MAX;
+        p.lb[pt] = runner_up(l == n1 ? m2 : m1, n2, W);
     } else {
         const float old = p.D2[pt];
         const int oi = p.idx[pt];
@@ -776,7 +779,7 @@ __device__ __noinline__ void lists_rows(BShared<DP> &sh, float *dsm, const float
             lab[pt] = best;
             D2[pt] = stored;
             reinterpret_cast<float *>(idx)[pt] =
-                fmaxf(0.f, fminf(off, i2 >= 0 ? lower_of(best == i1 ? b2 : b1, W) : FLT_MAX));
+                fmaxf(0.f, fminf(off, runner_up(best == i1 ? b2 : b1, i2, W)));
         } else if (n > 0) {
             const float m32 = fminf(dd, b1), lim = m32 + W * m32;
             const bool in_old = dd <= lim, in1 = i1 >= 0 && b1 <= lim, in2 = i2 >= 0 && b2 <= lim;
@@ -907,7 +910,7 @@ __device__ __noinline__ int pending_rows(BShared<DP> &sh, float *dsm, const floa
                 dm[pt] = stored;
             }
             const float off = 2.f * sqrtf(cov) * (1.f - 1e-6f) - upper_of(dd, W);
-            lb[pt] = fmaxf(0.f, fminf(off, i2 >= 0 ? lower_of(best == i1 ? b2 : b1, W) : FLT_MAX));
+            lb[pt] = fmaxf(0.f, fminf(off, runner_up(best == i1 ? b2 : b1, i2, W)));
         }
         __syncthreads();   // the chunk's entries are read before rows are put back over them
         block_append(op, pt, pend, &sh.s_cnt);
