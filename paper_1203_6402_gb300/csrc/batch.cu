@@ -883,7 +883,8 @@ __device__ __noinline__ int pending_rows(BShared<DP> &sh, float *dsm, const floa
             cov = __uint_as_float(rad[a]);
             n = lcnt[a];
         }
-        const bool op = mine && !(dd <= cov);
+        // (a row whose own center's square is beyond FP32 has the dense pass's label and value)
+        const bool op = mine && !(dd <= cov && dd < FLT_MAX);
         if (op || !mine) n = 0;
         const float *xrow = Xp + (int64_t)pt * d;
         float b1 = dd, b2 = FLT_MAX;

@@ -8,6 +8,19 @@ import pytest
 torch = pytest.importorskip("torch")
 
 
+def _steps(seed):
+    """Uneven groups of rows 1.3e19 apart: a center among them comes out of reach of some."""
+    rng = np.random.default_rng(1000 + seed)
+    d = int(rng.integers(1, 3))
+    n = int(rng.integers(4096, 6000))
+    k = int(rng.integers(2, 5))
+    places = rng.integers(k + 1, k + 5)
+    at = np.zeros((places, d))
+    at[:, 0] = 1.3 * rng.permutation(2 * places)[:places]
+    X = at[rng.choice(places, size=n, p=rng.dirichlet(np.full(places, 0.4)))] + rng.normal(0.0, 0.02, size=(n, d))
+    return (X * 1e19).astype(np.float32), k
+
+
 def _line(seed):
     """Clusters along a line of some 1e19 (FP32 squares end at 1.84e19), a few rows wide each."""
     rng = np.random.default_rng(seed)
@@ -22,14 +35,15 @@ def _line(seed):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("rows", [_line, _steps])
 @pytest.mark.parametrize("split", [0, 3000])
-def test_far_rows_follow_the_centers(split):
+def test_far_rows_follow_the_centers(split, rows):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_1203_6402_gb300 import kmpar as km
     Xs, probs, off = [], [], dict(x=0, c=0, l=0)
     for seed in range(160):
-        X, k = _line(seed)
+        X, k = rows(seed)
         n, d = X.shape
         Xs.append(X)
         probs.append(dict(n=n, d=d, k=k, ell=1.0, rounds=seed % 4, max_iter=1 + seed % 7, seed=seed,
@@ -48,7 +62,7 @@ def test_far_rows_follow_the_centers(split):
         res = km.kmpar_batch_run(Xd.data_ptr(), probs, C.data_ptr(), L.data_ptr())[1]
     finally:
         km.kmpar_batch_set_split(25000)
-    bad = []
+    bad, costs = [], []
     for i, (p, r, X) in enumerate(zip(probs, res, Xs)):
         if r["status"] == km.KMPAR_ERR_CAPACITY:
             continue
@@ -58,4 +72,6 @@ def test_far_rows_follow_the_centers(split):
         g.close()
         if not torch.equal(o["labels"], L[p["l_offset"]: p["l_offset"] + n]):
             bad.append((i, int((o["labels"] != L[p["l_offset"]: p["l_offset"] + n]).sum())))
-    assert not bad, bad
+        if not r["final_cost"] == pytest.approx(o["final_cost"], rel=1e-12):   # FP64 sums of the same FP32 distances
+            costs.append((i, r["final_cost"], o["final_cost"]))
+    assert not bad and not costs, (bad, costs)
