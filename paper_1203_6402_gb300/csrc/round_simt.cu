@@ -455,30 +455,34 @@ static cudaError_t launch_nearest_mode(const NearestParams &p, int cnt_hint, cud
     return cudaGetLastError();
 }
 
-// Alg. 2 step 2: D^2 to the first center, idx = 0.  128 rows a block, 32 coordinates at a
-// time through shared memory (coalesced loads, a lane-per-row walk at an odd stride):
-// bound by reading X.
-constexpr int kFirstRows = 128;
+// Alg. 2 step 2: D^2 to the first center, idx = 0.  128 rows a block, up to kFirstPiece
+// coordinates at a time through shared memory, coordinate-major at an odd stride: all of a
+// piece is on its way at once (asynchronous copies along the rows), and a lane then walks
+// its row.  Bound by reading X; with loads of 32 lanes a row, eight rows in flight, most lanes
+// idle in a row of 3 to 24 coordinates: 9e6 x 8 525 us, so 126; 4.8e6 x 42 432, 201; 2e6 x
+// 128 500, 249.
+constexpr int kFirstRows = 128, kFirstPiece = 64, kFirstStride = kFirstRows + 1;
 
 __global__ void __launch_bounds__(kFirstRows) first_dist_kernel(const float *__restrict__ X, int64_t n, int d,
                                                                const float *__restrict__ C, float *__restrict__ D2,
                                                                int32_t *__restrict__ idx, double *partials) {
-    __shared__ float xs[kFirstRows][33];
-    __shared__ float cq[32];
+    extern __shared__ __align__(16) float fsm[];   // min(d, kFirstPiece) x kFirstStride
+    __shared__ float cq[kFirstPiece];
     __shared__ double red[32];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int tid = threadIdx.x;
     const int64_t base = (int64_t)blockIdx.x * kFirstRows, R = base + tid;
     float v = 0.f;
-    for (int q0 = 0; q0 < d; q0 += 32) {
-        const int kn = min(32, d - q0);
+    for (int q0 = 0; q0 < d; q0 += kFirstPiece) {
+        const int kn = min(kFirstPiece, d - q0);
         __syncthreads();   // the walkers of the last piece are done
-#pragma unroll 8
-        for (int r = w; r < kFirstRows; r += kFirstRows / 32)
-            if (lane < kn && base + r < n) xs[r][lane] = __ldg(X + (base + r) * d + q0 + lane);
+        tile_copy<kFirstRows>(fsm, kFirstStride, kFirstRows, X, base, n, nullptr, d, q0, kn);
+        cp_async_commit();
         if (tid < kn) cq[tid] = C[q0 + tid];
+        cp_async_wait<0>();
         __syncthreads();
+#pragma unroll 8
         for (int q = 0; q < kn; ++q) {
-            const float t = __fsub_rn(xs[tid][q], cq[q]);
+            const float t = __fsub_rn(fsm[q * kFirstStride + tid], cq[q]);
             v = __fmaf_rn(t, t, v);
         }
     }
@@ -519,7 +523,8 @@ cudaError_t launch_init_first(Ctx &c) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int grid = (int)((c.n + kFirstRows - 1) / kFirstRows);
-    first_dist_kernel<<<grid, kFirstRows, 0, c.stream>>>(c.X, c.n, c.d, c.C, c.D2, c.idx, c.partials);
+    const size_t smem = sizeof(float) * (size_t)std::min(c.d, kFirstPiece) * kFirstStride;
+    first_dist_kernel<<<grid, kFirstRows, smem, c.stream>>>(c.X, c.n, c.d, c.C, c.D2, c.idx, c.partials);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return launch_phi_finalize(c, grid, &c.st->phi, &c.st->phi_hist[0]);
