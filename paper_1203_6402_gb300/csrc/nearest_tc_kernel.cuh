@@ -141,6 +141,10 @@ __device__ __forceinline__ void tmem_wait_ld_dep(uint32_t (&r)[32]) {
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(dst)), "l"(src) : "memory");
 }
+// ... through L1
+__device__ __forceinline__ void cp_async16_l1(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(su32(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async4(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(su32(dst)), "l"(src) : "memory");
 }
@@ -399,12 +403,15 @@ __global__ void __launch_bounds__(kThreads, 1) nearest_tc_kernel(TcParams p, int
         // one immediate of a single logic op per key
         const uint32_t vmask = p.vmask;
         // norms of center tile tn into buffer slot: one 16-byte copy per lane (a
-        // tile's copies were issued one tile earlier, so their latency is hidden)
+        // tile's copies were issued one tile earlier, so their latency is hidden).  Through
+        // L1: every warp of the GPU reads the same kilobyte, and straight from L2 a pass over
+        // 1,254,978 x 85 rows and 133 centers took 126 or 157 us, depending on where
+        // that kilobyte lay in L2.
         float *nbw = nbuf + (size_t)e * 2 * C::NB;
         auto prefetch_norms = [&](int tn, int slot) {
             if (NE) {
                 float *dst = nbw + slot * C::NB;
-                if (lane < C::GW / 4) cp_async16(dst + lane * 4, p.ncol + (size_t)tn * BN + grp * C::GW + lane * 4);
+                if (lane < C::GW / 4) cp_async16_l1(dst + lane * 4, p.ncol + (size_t)tn * BN + grp * C::GW + lane * 4);
                 if (FMT == FMT_FP8 && lane == C::GW / 4) cp_async4(dst + C::GW, p.tscale + tn);
                 cp_async_commit();
             }
