@@ -34,6 +34,7 @@ __host__ __device__ __forceinline__ uint32_t sw128_off(int r, int c) {
 
 // the refine and fix-up kernels size their shared-memory rows for d <= 190
 constexpr int kMaxD = 190;
+constexpr int kMaxKA = 3;   // K atoms of the screening kernels
 
 // ------------------------------------------------------------------ operand encoding
 __device__ __forceinline__ __nv_bfloat16 bf(float v) { return __float2bfloat16_rn(v); }
@@ -60,22 +61,6 @@ struct Enc {
 // x'_q = fl(x_q - a_q)
 __device__ __forceinline__ float moved(const Enc &e, const float *x, int q) {
     return e.a ? __fsub_rn(x[q], e.a[q]) : x[q];
-}
-
-// element k of a BF16 A (point) row
-__device__ __forceinline__ __nv_bfloat16 a_elem(const Enc &e, const float *x, int k) {
-    const int d = e.d;
-    if (e.fmt == FMT_BF16N) return k < d ? bf(moved(e, x, k)) : bf(0.f);
-    if (e.fmt == FMT_BF16) {
-        if (k < d) return bf(moved(e, x, k));
-        if (k == d || k == d + 1) return bf(1.f);
-        return bf(0.f);
-    }
-    if (k < d) return bf(moved(e, x, k));
-    if (k < 2 * d) { const float v = moved(e, x, k - d); return bf(v - __bfloat162float(bf(v))); }
-    if (k < 3 * d) return bf(moved(e, x, k - 2 * d));
-    if (k == 3 * d || k == 3 * d + 1) return bf(1.f);
-    return bf(0.f);
 }
 
 // element k of a BF16 B (center) row.  Pad rows (no center) get a huge FINITE squared
@@ -253,9 +238,18 @@ __global__ void __launch_bounds__(256) prep_centers_ne_kernel(const float *__res
 // row's atom (position p of row r holds logical chunk p ^ (r & 7)), so loads, stores and
 // shared-memory reads all spread.  Bound by reading X and writing the image: preparing
 // 1e7 x 128 for BF16 (kmpar_init as a whole) takes 7.1 ms; 14.6 ms with a thread a row,
-// whose reads of one bank queued.
+// whose reads of one bank queued.  In the formats with norm columns a coordinate is
+// encoded once, when it is loaded, into an image of the row in shared memory (the split
+// format holds its high half twice); its chunks are then copied.  Their rows are short, and
+// two steps of loads in flight count: 4.8e6 x 42 split 360 us (771 encoded by chunk,
+// one step at a time; 749 with a thread a row), x 24 289 (724, 652), x 60 BF16 297 (655, 659).
 constexpr int kPrepWarps = 8, kPrepRows = 8;
-constexpr size_t prep_smem(int d) { return sizeof(float) * kPrepWarps * kPrepRows * (size_t)(d | 1); }
+__host__ __device__ constexpr bool prep_encoded(int fmt) { return fmt == FMT_BF16 || fmt == FMT_BF16X3; }
+__host__ __device__ constexpr int prep_row_halves(int KA) { return KA * 64 + 8; }   // 16 bytes more: rows start in different banks
+constexpr size_t prep_smem(int d, int KA, int fmt) {
+    return (size_t)kPrepWarps * kPrepRows *
+           (sizeof(float) * (d | 1) + (prep_encoded(fmt) ? sizeof(__nv_bfloat16) * prep_row_halves(KA) : 0));
+}
 
 template <int fmt>
 __global__ void __launch_bounds__(32 * kPrepWarps) prep_points_kernel(const float *__restrict__ X, int64_t n,
@@ -268,20 +262,52 @@ __global__ void __launch_bounds__(32 * kPrepWarps) prep_points_kernel(const floa
     __shared__ float inv_s[kPrepWarps][kPrepRows];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ds = d | 1;
     float *xw = xsm + (size_t)w * kPrepRows * ds;
+    // per warp kPrepRows encoded rows; the columns past the coordinates stay as set here
+    const int es = prep_row_halves(KA), base = fmt == FMT_BF16X3 ? 3 * d : d;
+    __nv_bfloat16 *ew = reinterpret_cast<__nv_bfloat16 *>(xsm + (size_t)kPrepWarps * kPrepRows * ds) +
+                        (size_t)w * kPrepRows * es;
+    if (prep_encoded(fmt))
+        for (int r = 0; r < kPrepRows; ++r)
+            for (int q = base + lane; q < KA * 64; q += 32) ew[r * es + q] = bf(q < base + 2 ? 1.f : 0.f);
     const int64_t nblk = n_pad / kPrepRows, stride = (int64_t)gridDim.x * kPrepWarps;
-    const Enc em{d, fmt, nullptr};   // the staged rows are already moved
     for (int64_t b = (int64_t)blockIdx.x * kPrepWarps + w; b < nblk; b += stride) {   // uniform per warp
         const int64_t r0 = b * kPrepRows;
         const int nr = (int)max((int64_t)0, min((int64_t)kPrepRows, n - r0));
         __syncwarp();   // the previous rows' readers are done
-        for (int q = lane; q < d; q += 32) {
-            const float a = __ldg(anchor + q);
-            float v[kPrepRows];
+        // (with few coordinates two steps' loads are in flight at once: the warp waits for them)
+        constexpr int U = prep_encoded(fmt) ? 2 : 1;
+        for (int q0 = lane; q0 < d; q0 += 32 * U) {
+            float v[U][kPrepRows], a[U];
 #pragma unroll
-            for (int r = 0; r < kPrepRows; ++r) v[r] = r < nr ? __ldg(X + (r0 + r) * d + q) : a;
+            for (int u = 0; u < U; ++u) {
+                const int q = q0 + 32 * u;
+                a[u] = q < d ? __ldg(anchor + q) : 0.f;
 #pragma unroll
-            for (int r = 0; r < kPrepRows; ++r) xw[r * ds + q] = __fsub_rn(v[r], a);
+                for (int r = 0; r < kPrepRows; ++r) v[u][r] = r < nr && q < d ? __ldg(X + (r0 + r) * d + q) : a[u];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int q = q0 + 32 * u;
+                if (q >= d) break;
+#pragma unroll
+                for (int r = 0; r < kPrepRows; ++r) {
+                    const float x = __fsub_rn(v[u][r], a[u]);
+                    xw[r * ds + q] = x;
+                    if (prep_encoded(fmt)) {
+                        __nv_bfloat16 *e = ew + r * es + q;
+                        const __nv_bfloat16 h = bf(x);
+                        e[0] = h;
+                        if (fmt == FMT_BF16X3) {
+                            e[d] = bf(x - __bfloat162float(h));
+                            e[2 * d] = h;
+                        }
+                    }
+                }
+            }
         }
+        // rows past the last (only a warp's last block has any): all zeros
+        if (prep_encoded(fmt) && lane < 2)
+            for (int r = nr; r < kPrepRows; ++r) ew[r * es + base + lane] = bf(0.f);
         __syncwarp();
         {
             const int r = lane >> 2;
@@ -312,12 +338,17 @@ __global__ void __launch_bounds__(32 * kPrepWarps) prep_points_kernel(const floa
                 const int r = f >> 3, pos = f & 7, ch = pos ^ ((rb + r) & 7);
                 const float *x = xw + r * ds;
                 uint4 u;
-                if (fmt == FMT_FP8) {
+                if (prep_encoded(fmt)) {
+                    u = *reinterpret_cast<const uint4 *>(ew + r * es + a * 64 + ch * 8);
+                } else if (fmt == FMT_FP8) {
                     u = pack16_e4m3(x, d, a * 128 + ch * 16, inv_s[w][r], r >= nr);
                 } else {
                     __nv_bfloat16 v[8];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) v[q] = r < nr ? a_elem(em, x, a * 64 + ch * 8 + q) : bf(0.f);
+                    for (int q = 0; q < 8; ++q) {
+                        const int k = a * 64 + ch * 8 + q;
+                        v[q] = bf(r < nr && k < d ? x[k] : 0.f);
+                    }
                     u = pack8(v);
                 }
                 *reinterpret_cast<uint4 *>(tile + (size_t)a * BM * 128 + (rb + r) * 128 + pos * 16) = u;
@@ -542,7 +573,7 @@ int tc_katoms(int d, int fmt) { return (k_bytes(d, fmt) + 127) / 128; }
 int tc_ksteps(int d, int fmt) { return (k_bytes(d, fmt) + 31) / 32; }
 int tc_block_n(int d, int fmt) { return tc_katoms(d, fmt) <= 2 ? 256 : 128; }
 bool tc_norms_in_epilogue(int fmt) { return fmt == FMT_BF16N || fmt == FMT_FP8; }
-bool tc_supported(int d, int fmt) { return fmt >= 0 && d >= 1 && d <= kMaxD && tc_katoms(d, fmt) <= 3; }
+bool tc_supported(int d, int fmt) { return fmt >= 0 && d >= 1 && d <= kMaxD && tc_katoms(d, fmt) <= kMaxKA; }
 
 size_t tc_points_image_bytes(int d, int fmt, int64_t n) {
     const int64_t tiles = (n + BM - 1) / BM;
@@ -563,12 +594,13 @@ cudaError_t launch_prep_points(const float *X, int64_t n, int d, int fmt, const 
     const int64_t n_pad = ((n + BM - 1) / BM) * BM;
     const int64_t blocks = n_pad / (kPrepWarps * kPrepRows);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(blocks, 8192));
+    const int KA = tc_katoms(d, fmt);
     auto go = [&](auto kern) -> cudaError_t {
         // (the same limit in every call: it belongs to the process)
-        const cudaError_t e =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prep_smem(kMaxD));
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)prep_smem(kMaxD, kMaxKA, FMT_BF16));
         if (e != cudaSuccess) return e;
-        kern<<<grid, 32 * kPrepWarps, prep_smem(d), s>>>(X, n, n_pad, d, tc_katoms(d, fmt), anchor, img, xnorm, xscale);
+        kern<<<grid, 32 * kPrepWarps, prep_smem(d, KA, fmt), s>>>(X, n, n_pad, d, KA, anchor, img, xnorm, xscale);
         return cudaGetLastError();
     };
     cudaError_t e = cudaErrorInvalidValue;
