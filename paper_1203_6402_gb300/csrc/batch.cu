@@ -54,7 +54,8 @@ namespace {
 constexpr int kBT = 256;          // threads per problem block
 constexpr int kBW = kBT / 32;     // warps per block
 constexpr int kBMaxCluster = 8;   // blocks per problem
-constexpr int kBMinRows = 400;    // a finer cut for few problems ends here
+constexpr int kBMinRows = 400;    // a finer cut for few problems ends here, where a row has some work (kBMinWork)
+constexpr int kBMinWork = 2048;   // centers x padded coordinates
 constexpr int kBRows = 128;       // rows of a tile
 constexpr int kBCols = 64;        // centers of a tile
 constexpr int kBXS = kBRows + 4, kBCS = kBCols + 4;   // floats per coordinate in shared memory
@@ -93,6 +94,7 @@ struct BArgs {
     long long *w_out;        // nullable
     BRes *res;
     bool lists;              // the lists have their memory
+    bool tiles;              // the launch has the shared memory of tiles and lists
     // work space
     float *D2;
     int32_t *idx, *lab, *perm;
@@ -108,16 +110,29 @@ struct BArgs {
 };
 
 constexpr int kBList = 16;   // entries of a reference's list
-// Centers x padded coordinates from which a pass goes by tiles of rows.  Below, a tile is
+// Centers x padded coordinates from which a dense pass goes by tiles of rows.  Below, a tile is
 // mostly its copies and its merge: 11 assignments of 2,975 x 15 to 6 centers take 0.23 ms a
-// row per thread and 1.2 ms by tiles; above, the tiles' reuse counts: 64 problems of 500 -
-// 3,000 rows, up to 60 centers, 3.8 ms with the rule and 4.6 ms with a row per thread alone.
-constexpr int kBTileWork = 4096;
+// row per thread and 1.2 ms by tiles; 64 problems of 30,000 - 60,000 x 101, k = 30 - 60, 67 ms
+// with the line at 64 centers and 72 at 32.  Above, the tiles' reuse counts: 64 problems of
+// 500 - 3,000 rows, up to 60 centers, 3.8 ms with the rule and 4.6 ms with a row per thread
+// alone; of 30,000 - 60,000 x 128, k = 200 - 256, 235 ms by tiles and 276 without.
+template <int DP>
+constexpr int kBTileWork = DP == 128 ? 8192 : 4096;
 // Fewer rows go through the dense passes alone (lists, radii and their barriers cost more
 // there than the few tiles they save).  With lists 512 problems of up to 200,000 rows,
 // d = 32 - 128, take 305 ms instead of 577, 273 with the tiles below and step 8 over the
 // whole cluster (22 -> 2.4 ms of the largest problem's time).
 constexpr int kBListRows = 4096;
+// Centers x coordinates of a dense pass from which lists pay: a row against its list costs some
+// 15 to 30 ns of its block whatever the dimension (16 rows a warp), and its pairs' rows and
+// centers are staged, by 16-byte copies where their rows allow it, else by 4-byte ones.
+// 64 problems of 30,000 - 60,000 rows, k = 30 - 60, mixtures with R = 10, without lists / with:
+// d = 128 75 ms / 42, d = 64 47 / 30; d = 101 55 / 65, d = 42 34 / 39.
+constexpr int kBListWork = 8192, kBListWorkVec = 1024;
+// After a list pass that left over 7/8 of the references without a list, or most rows open (the
+// data do not separate), the problem goes on densely until its references are this many times
+// as many.
+constexpr int kBListRetry = 6;
 
 enum { BM_FIRST = 0, BM_ROUND = 1, BM_ASSIGN = 2 };
 
@@ -182,6 +197,8 @@ struct BShared {
     float s_m1, s_m2;
     int s_mi;
     int s_cnt;                 // rows listed by the block
+    bool tiles;                // the launch's shared memory holds tiles
+    int s_dead;                // list_pass: references of the block whose lists cover no row
     double s_dslot;
     int s_islot;
     unsigned long long s_uslot;
@@ -197,6 +214,10 @@ __host__ __device__ constexpr size_t batch_smem(int dp) {
     const size_t stage = sizeof(float) * kBW * (2 * kBStage * stage_stride(dp) + 2 * kBStage);
     return tiles > stage ? tiles : stage;
 }
+
+// ... and of a launch whose problems have no use for tiles or lists (see uses_tiles): the rows
+// a thread reads then find an L1 to stay in
+constexpr size_t kBLeanSmem = 16 * 1024;
 
 __device__ __forceinline__ void copy4(uint32_t dst, const float *src, bool valid) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
@@ -410,12 +431,15 @@ __device__ __noinline__ int rows_by_tile(const BPass p, float *dsm, int64_t r0, 
 }
 
 // a row per thread, its coordinates in registers (padded to DP with zeros: they add exact
-// zeros to the sums); 8 chains, one per center, over centers 32 at a time
+// zeros to the sums); 8 chains, one per center, over centers 32 at a time.  Inlined: as a
+// function of its own the compiler serialised the chains (11% fewer instructions an issue slot;
+// 400 problems of 300 - 2,000 x 42, k = 30 - 60: 4.6 ms, inlined 3.8).
 template <int DP, int MODE>
-__device__ __noinline__ int rows_by_thread(const BPass p, float *dsm, int64_t r0, int64_t r1,
+__device__ __forceinline__ int rows_by_thread(const BPass p, float *dsm, int64_t r0, int64_t r1,
                                            unsigned long long *fp64_cnt) {
-    constexpr int B = 32, NCH = 8;
-    const int tid = threadIdx.x;
+    constexpr int B = 32, NCH = 8, P = DP / 2;
+    const int tid = threadIdx.x, lane = tid & 31;
+    float *stage = dsm + B * DP + (tid >> 5) * 32 * (P + 1);
     int chg = 0;
     unsigned long long nfp64 = 0;
     for (int64_t base = r0; base < r1; base += kBT) {
@@ -485,6 +509,13 @@ __device__ __noinline__ int rows_by_thread(const BPass p, float *dsm, int64_t r0
     return chg;
 }
 
+// ... as a function of its own above 64 coordinates, where a block has the SM's registers
+template <int DP, int MODE>
+__device__ __noinline__ int rows_by_thread_wide(const BPass p, float *dsm, int64_t r0, int64_t r1,
+                                                unsigned long long *fp64_cnt) {
+    return rows_by_thread<DP, MODE>(p, dsm, r0, r1, fp64_cnt);
+}
+
 // One pass over the rows [r0, r1) of a problem (with `list`: the rows list[r0 .. r1))
 // against `cnt` centers: the rows of C_rows (a center matrix, stride d) or, when cand is
 // given, X rows cand[begin + r].  Each row's lexicographic (value, center number) top-2
@@ -497,8 +528,7 @@ __device__ __noinline__ int rows_by_thread(const BPass p, float *dsm, int64_t r0
 //   ASSIGN  the best, re-decided in FP64 against the runner-up inside the window; takes
 //           the distance to it and a lower bound of the distance to every other center
 //           (dm, lb), and marks the centers that a row left or joined (flag; nullable)
-// Sets *changed to the block's number of changed labels.  Few centers go a row per thread
-// (with less than kBTileWork coordinates of them a tile is mostly its copies and its merge).
+// Sets *changed to the block's number of changed labels.
 template <int DP, int MODE>
 __device__ __forceinline__ void dist_pass(BShared<DP> &sh, float *dsm, const float *__restrict__ Xp, int64_t r0, int64_t r1,
                                           int d, const float *C_rows, const int32_t *__restrict__ cand, int begin, int cnt,
@@ -508,12 +538,9 @@ __device__ __forceinline__ void dist_pass(BShared<DP> &sh, float *dsm, const flo
     const BPass p{Xp, C_rows, cand, list, D2, idx, lab, dm, lb, flag, d, begin, cnt, changed != nullptr};
     __syncthreads();
     int chg = 0;
-    if constexpr (DP <= 64) {
-        chg = cnt * DP < kBTileWork ? rows_by_thread<DP, MODE>(p, dsm, r0, r1, fp64_cnt)
-                                    : rows_by_tile<DP, MODE>(p, dsm, r0, r1, fp64_cnt);
-    } else {
-        chg = rows_by_tile<DP, MODE>(p, dsm, r0, r1, fp64_cnt);
-    }
+    if (sh.tiles && cnt * DP >= kBTileWork<DP>) chg = rows_by_tile<DP, MODE>(p, dsm, r0, r1, fp64_cnt);
+    else if constexpr (DP <= 64) chg = rows_by_thread<DP, MODE>(p, dsm, r0, r1, fp64_cnt);
+    else chg = rows_by_thread_wide<DP, MODE>(p, dsm, r0, r1, fp64_cnt);
     if (MODE == BM_ASSIGN && changed) *changed = bsum_i32(chg, sh.redi);   // every thread
     __syncthreads();
 }
@@ -617,7 +644,7 @@ __device__ void radius_pass(int64_t r0, int64_t r1, const float *D2, const int32
 // X rows ccand[begin + j]) within 2 r + tau, r^2 = rad[i], tau the distance to the nearest
 // of them (want_tau; else 0).  A list that overflows is taken again at half the radius,
 // three times at most.  On return rad[i] holds the bits of the squared radius covered
-// (-1: none), lcnt and lst the list (numbers from begin, in no order).
+// (-1: none; sh.s_dead of the block's), lcnt and lst the list (numbers from begin, in no order).
 template <int DP>
 __device__ __noinline__ void list_pass(BShared<DP> &sh, float *dsm, const float *__restrict__ Xp, int f0, int f1, int d,
                                        const int32_t *__restrict__ cand, const float *C_rows,
@@ -629,6 +656,9 @@ __device__ __noinline__ void list_pass(BShared<DP> &sh, float *dsm, const float 
     auto center = [&](int j) -> const float * {
         return ccand ? Xp + (int64_t)ccand[begin + j] * d : C_rows + (int64_t)(begin + j) * d;
     };
+    __syncthreads();
+    if (tid == 0) sh.s_dead = 0;
+    __syncthreads();
     for (int base = f0; base < f1; base += kBRows) {   // uniform per block
         auto row = [&](int r) -> const float * {
             const int i = base + r;
@@ -706,6 +736,7 @@ __device__ __noinline__ void list_pass(BShared<DP> &sh, float *dsm, const float 
             if (active[i]) {
                 rad[f] = __float_as_uint(-1.f);
                 lcnt[f] = 0;
+                atomicAdd(&sh.s_dead, 1);
             }
             if (want_tau) tau2[f] = tau[i];
         }
@@ -1056,6 +1087,7 @@ __global__ void __launch_bounds__(kBT, DP == 128 ? 1 : 2) batch_kernel(BArgs a, 
     // rows of 16-byte pieces
     const bool vec = (d & 3) == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(C)) & 15u) == 0;
     if (tid == 0) {
+        sh.tiles = a.tiles;
         sh.s_near = 0; sh.s_fp64 = 0; sh.s_rnear = 0;
         if (rank == 0) {
             // Alg. 2 step 1: the first center, uniform over the problem's points
@@ -1070,6 +1102,7 @@ __global__ void __launch_bounds__(kBT, DP == 128 ? 1 : 2) batch_kernel(BArgs a, 
     dist_pass<DP, BM_FIRST>(sh, dsm, X, r0, r1, d, nullptr, cand, 0, 1, D2, idx, nullptr, nullptr, &sh.s_fp64);
     double phi = csum<CS>(sum_rows_of(sh, D2, r0, r1), &sh.s_dslot);
     int m = 1, status = KMPAR_OK;
+    int fail = 0;   // references of the last list pass if it left most rows open
     for (int r = 1; r <= P.rounds; ++r) {
         // step 4: independent draws of the block's rows; p and the near-draw rule as
         // in the single-problem path
@@ -1128,12 +1161,17 @@ __global__ void __launch_bounds__(kBT, DP == 128 ? 1 : 2) batch_kernel(BArgs a, 
         // step 5: D^2 and idx against the batch, then phi.  While the references (the
         // candidates before a part of the batch) are few against the rows, their lists
         // settle most rows; a first round starts with a dense part.
-        const bool lists = a.lists && n >= kBListRows && n >= 8 * (int64_t)(m + appended_all);
-        const int parts = lists ? max(1, min(4, appended_all / 64)) : 1;
-        for (int part = 0; part < parts; ++part) {
-            const int b0 = m + (int)((int64_t)appended_all * part / parts);
-            const int b1 = m + (int)((int64_t)appended_all * (part + 1) / parts);
-            if (!lists || b0 == 1) {
+        const bool lists = a.lists && a.tiles && n >= kBListRows && n >= 8 * (int64_t)(m + appended_all) &&
+                           appended_all * d >= (vec ? kBListWorkVec : kBListWork);
+        const int parts = max(1, min(4, appended_all / 64));
+        for (int part = 0, from = 0; part == 0 || from < appended_all; ++part) {
+            const int b0 = m + from;
+            const bool by_list = lists && b0 > 1 && b0 >= kBListRetry * fail;
+            // (the first part of a first round is dense, what lists have failed for all at once)
+            if (by_list || (lists && b0 == 1)) from = min(appended_all, (int)((int64_t)appended_all * (part + 1) / parts));
+            else from = appended_all;
+            const int b1 = m + from;
+            if (!by_list) {
                 dist_pass<DP, BM_ROUND>(sh, dsm, X, r0, r1, d, nullptr, cand, b0, b1 - b0, D2, idx, nullptr, nullptr,
                                         &sh.s_fp64);
                 csync<CS>();
@@ -1147,9 +1185,18 @@ __global__ void __launch_bounds__(kBT, DP == 128 ? 1 : 2) batch_kernel(BArgs a, 
             list_pass<DP>(sh, dsm, X, min(b0, rank * per_f), min(b0, (rank + 1) * per_f), d, cand, nullptr, cand, b0, b1 - b0,
                           false, rad, lcnt, lst, nullptr);
             csync<CS>();
+            if (8 * csum<CS>(sh.s_dead, &sh.s_islot) > 7 * b0) {   // (nor are there rows to look at)
+                fail = b0;
+                dist_pass<DP, BM_ROUND>(sh, dsm, X, r0, r1, d, nullptr, cand, b0, b1 - b0, D2, idx, nullptr, nullptr,
+                                        &sh.s_fp64);
+                csync<CS>();
+                continue;
+            }
             lists_rows<BM_ROUND, DP>(sh, dsm, X, r0, r1, d, vec, nullptr, cand, rad, lcnt, lst, nullptr, D2, idx, nullptr,
                                      perm + r0, &sh.s_fp64);
             const int no = sh.s_cnt;
+            const int64_t open = csum<CS>(no, &sh.s_islot);
+            fail = 8 * open > (r == 1 ? 7 : 6) * n ? b0 : 0;   // (round 1 still has clusters without a candidate)
             __syncthreads();
             dist_pass<DP, BM_ROUND>(sh, dsm, X, 0, no, d, nullptr, cand, b0, b1 - b0, D2, idx, nullptr, nullptr, &sh.s_fp64,
                                     perm + r0);
@@ -1175,7 +1222,7 @@ __global__ void __launch_bounds__(kBT, DP == 128 ? 1 : 2) batch_kernel(BArgs a, 
         {
             const int per_m = (m + CS - 1) / CS;
             const int j0 = min(m, rank * per_m), ml = min(m, j0 + per_m) - j0;
-            const int cap = (int)(batch_smem(DP) / sizeof(float));
+            const int cap = (int)((a.tiles ? batch_smem(DP) : kBLeanSmem) / sizeof(float));
             const int mls = per_m | 1;   // odd: the transposing stores below meet no bank twice
             const bool in_smem = 2 * per_m <= cap;
             const int Q = in_smem ? min((cap - 2 * per_m) / mls & ~7, (d + 7) & ~7) : 0;
@@ -1317,8 +1364,9 @@ __global__ void __launch_bounds__(kBT, DP == 128 ? 1 : 2) batch_kernel(BArgs a, 
         // Lloyd's iteration from the seed centers: dm (in place of D2) the exact distance to a
         // row's center, lb (in place of idx) a lower bound of those to the others
         float *dm = D2, *lb = reinterpret_cast<float *>(idx);
-        const bool first_lists = a.lists && n >= kBListRows && n >= 8 * (int64_t)m;
-        const bool center_lists = a.lists && n >= kBListRows && n >= 8 * (int64_t)k;
+        bool center_lists = a.lists && a.tiles && n >= kBListRows && n >= 8 * (int64_t)k && k * d >= (vec ? kBListWorkVec : kBListWork) &&
+                            m >= kBListRetry * fail;
+        const bool first_lists = center_lists && n >= 8 * (int64_t)m;
         int it = 0;
         double cost = 0.0;
         for (;; ++it) {
@@ -1335,6 +1383,7 @@ __global__ void __launch_bounds__(kBT, DP == 128 ? 1 : 2) batch_kernel(BArgs a, 
                 lists_rows<BM_ASSIGN, DP>(sh, dsm, X, r0, r1, d, vec, C, nullptr, rad, lcnt, lst, tau2, D2, idx, lab,
                                           perm + r0, &sh.s_fp64);
                 const int no = sh.s_cnt;
+                if (8 * (int64_t)csum<CS>(no, &sh.s_islot) > 7 * n) center_lists = false;
                 __syncthreads();
                 dist_pass<DP, BM_ASSIGN>(sh, dsm, X, 0, no, d, C, nullptr, 0, k, nullptr, nullptr, lab, nullptr, &sh.s_fp64,
                                          perm + r0, dm, lb);
@@ -1371,6 +1420,7 @@ __global__ void __launch_bounds__(kBT, DP == 128 ? 1 : 2) batch_kernel(BArgs a, 
                 const int tc = pending_rows<DP>(sh, dsm, X, np, d, vec, C, rad, lcnt, lst, lab, dm, lb, perm + r0, flag,
                                                 &sh.s_fp64);
                 const int no = sh.s_cnt;
+                if (2 * (int64_t)csum<CS>(no, &sh.s_islot) > n) center_lists = false;   // (the dense pass settles most rows)
                 __syncthreads();
                 dist_pass<DP, BM_ASSIGN>(sh, dsm, X, 0, no, d, C, nullptr, 0, k, nullptr, nullptr, lab, &chg, &sh.s_fp64,
                                          perm + r0, dm, lb, flag);
@@ -1540,25 +1590,43 @@ kmpar_status batch_fail(kmpar_status s, const std::string &m) {
 // (kmpar_batch_set_split; 0: never split)
 std::atomic<int64_t> g_rows_per_block{25000};
 
-int cluster_size(int64_t n, int64_t rpb) {
+int padded_dim(int d) { return d <= 32 ? 32 : (d <= 64 ? 64 : 128); }
+
+// blocks of a problem at rpb rows a block; below the set size (full) blocks of little work
+// a row stay larger, or their barriers outweigh it (one problem of some 10,000 x 3, k = 5,
+// box: 0.96 ms in one block, 1.30 in eight)
+int cluster_size(const kmpar_problem &p, int64_t rpb, int64_t full) {
+    const int64_t work = (int64_t)p.k * padded_dim(p.d);
+    if (rpb < full && work < kBMinWork) rpb = std::max(rpb, std::min(full, (int64_t)kBMinRows * kBMinWork / work));
     int cs = 1;
-    while (rpb > 0 && cs < 8 && (n + cs - 1) / cs > rpb) cs *= 2;
+    while (rpb > 0 && cs < 8 && (p.n + cs - 1) / cs > rpb) cs *= 2;
     return cs;
+}
+
+// whether a problem's passes may go by tiles or lists; a launch of which none may takes
+// little shared memory (400 problems of 300 - 2,000 x 15 and 42, k = 30 - 60: 4.9 ms with
+// the tiles' 92 KB a block, 3.9 without)
+bool uses_tiles(const kmpar_problem &p) {
+    const double most = std::max((double)p.k, p.ell);   // centers of a pass
+    const int dp = padded_dim(p.d);
+    return most * dp >= 2.0 * (dp == 128 ? kBTileWork<128> : kBTileWork<64>) ||
+           (p.n >= kBListRows && most * p.d >= (p.d % 4 == 0 ? kBListWorkVec : kBListWork));
 }
 
 template <int DP, int CS>
 cudaError_t launch_cs(const kmp::BArgs &a, int first, int count, cudaStream_t s) {
     if (count == 0) return cudaSuccess;
+    const size_t smem = a.tiles ? kmp::batch_smem(DP) : kmp::kBLeanSmem;
     const cudaError_t ea = cudaFuncSetAttribute(kmp::batch_kernel<DP, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)kmp::batch_smem(DP));
     if (ea != cudaSuccess) return ea;
     if (CS == 1) {
-        kmp::batch_kernel<DP, 1><<<count, kmp::kBT, kmp::batch_smem(DP), s>>>(a, first);
+        kmp::batch_kernel<DP, 1><<<count, kmp::kBT, smem, s>>>(a, first);
     } else {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(count * CS));
         cfg.blockDim = dim3(kmp::kBT);
-        cfg.dynamicSmemBytes = kmp::batch_smem(DP);
+        cfg.dynamicSmemBytes = smem;
         cfg.stream = s;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1639,20 +1707,20 @@ kmpar_status kmpar_batch_run(const float *X, const kmpar_problem *problems, int3
         k_tot += q.k;
         s_tot += (int64_t)q.k * q.d;
         // distance evaluations of the rounds and of Lloyd, times the padded dimension
-        const int dp = q.d <= 32 ? 32 : (q.d <= 64 ? 64 : 128);
-        work[(size_t)i] = (double)q.n * dp * (1.0 + q.rounds * q.ell + (double)(q.max_iter + 1) * q.k);
+        work[(size_t)i] = (double)q.n * padded_dim(q.d) * (1.0 + q.rounds * q.ell + (double)(q.max_iter + 1) * q.k);
     }
     // a call whose blocks would leave SMs idle cuts its problems finer, down to blocks of
     // kBMinRows rows (64 problems of 500 - 3,000 rows, d = 15 and 42: 3.8 ms a block each,
     // 1.8 ms at 780 rows a block)
-    int64_t rpb = g_rows_per_block.load(std::memory_order_relaxed);
+    const int64_t full = g_rows_per_block.load(std::memory_order_relaxed);
+    int64_t rpb = full;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 0;
     while (rpb >= 2 * kBMinRows) {
         int64_t blocks = 0;
-        for (int i = 0; i < count && blocks < sms; ++i) blocks += cluster_size(problems[i].n, rpb);
+        for (int i = 0; i < count && blocks < sms; ++i) blocks += cluster_size(problems[i], rpb, full);
         if (blocks >= sms) break;
         rpb /= 2;
     }
@@ -1666,7 +1734,7 @@ kmpar_status kmpar_batch_run(const float *X, const kmpar_problem *problems, int3
         for (int cs = 8; cs >= 1; cs /= 2) {
             std::vector<int32_t> ids;
             for (int i = 0; i < count; ++i)
-                if (problems[i].d >= lo && problems[i].d <= hi && cluster_size(problems[i].n, rpb) == cs) ids.push_back(i);
+                if (problems[i].d >= lo && problems[i].d <= hi && cluster_size(problems[i], rpb, full) == cs) ids.push_back(i);
             if (ids.empty()) continue;
             std::stable_sort(ids.begin(), ids.end(), [&](int32_t x, int32_t y) { return work[x] > work[y]; });
             classes.push_back({c == 0 ? 32 : (c == 1 ? 64 : 128), cs, (int)order.size(), (int)ids.size()});
@@ -1746,6 +1814,8 @@ kmpar_status kmpar_batch_run(const float *X, const kmpar_problem *problems, int3
     for (int i = 0; i < nside && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(side[(size_t)i], ev_fork, 0);
     for (size_t c = 0; c < classes.size() && e == cudaSuccess; ++c) {
         const Cls &q = classes[c];
+        a.tiles = false;
+        for (int i = 0; i < q.count; ++i) a.tiles |= uses_tiles(problems[order[(size_t)(q.first + i)]]);
         cudaStream_t cs = c == 0 ? s : side[c - 1];
         if (q.dp == 32) e = launch_class<32>(a, q.cs, q.first, q.count, cs);
         else if (q.dp == 64) e = launch_class<64>(a, q.cs, q.first, q.count, cs);
