@@ -462,7 +462,10 @@ kmpar_status kmpar_weight(kmpar_ctx *ctx, int64_t *m_out, const int32_t **cand_i
     if (c.rounds_done != c.rounds) return fail(&c, KMPAR_ERR_STATE, "weight before the last round");
     KMP_CUDA(&c, kmp::launch_weights(c), "weights kernel");
     kmp::DevState st;
+    int open = 0;   // rows the last round's lists left
     KMP_CUDA(&c, cudaMemcpyAsync(&st, c.st, sizeof(st), cudaMemcpyDeviceToHost, c.stream), "read state");
+    if (c.rf_cnt && c.rounds > 1)
+        KMP_CUDA(&c, cudaMemcpyAsync(&open, c.rf_cnt, sizeof(int), cudaMemcpyDeviceToHost, c.stream), "read open rows");
     KMP_CUDA(&c, cudaStreamSynchronize(c.stream), "sync");
     KMP_CUDA(&c, kmp::timing_drain(c), "timing");
     if (st.overflow) return fail(&c, KMPAR_ERR_CAPACITY, "a round drew more points than its capacity");
@@ -470,6 +473,10 @@ kmpar_status kmpar_weight(kmpar_ctx *ctx, int64_t *m_out, const int32_t **cand_i
     if (ts != KMPAR_OK) return ts;
     c.weighted = true;
     c.m_host = st.m;
+    if (c.rf_cnt && c.rounds > 1 && st.round_added[c.rounds - 1] > 0) {
+        c.lists_known = true;
+        c.lists_failed = 4 * (int64_t)open > 3 * c.n;
+    }
     give_back(c, [&](auto take) { round_filter_buffers(c, take); });
     if (m_out) *m_out = st.m;
     if (cand_idx_dev) *cand_idx_dev = c.cand;
@@ -628,19 +635,22 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
     // after the first assignment, rows whose bounds prove their center unchanged are
     // settled without the tensor pass (the results are the same)
     const bool bounded = kmp::lloyd_bounds_usable(c, centers_dev);
-    const bool listed = bounded && kmp::lloyd_lists_usable(c);
+    // (the lists are given up once they do not pay: unless those of the last round held, the
+    // first two assignments make up a batch of their own, so that the host learns it early)
+    bool listed = bounded && kmp::lloyd_lists_usable(c);
+    bool by_change = listed;   // only clusters whose members changed are sorted and summed
     auto keep_centers = [&]() -> cudaError_t {
         return bounded ? cudaMemcpyAsync(c.ll_cold, centers_dev, sizeof(float) * (size_t)c.k * c.d,
                                          cudaMemcpyDeviceToDevice, c.stream)
                        : cudaSuccess;
     };
     while (done < 0) {
-        const int batch = t < 8 ? 4 : 8;
+        const int batch = listed && t == 0 && !c.lists_known ? 2 : t < 8 ? 4 : 8;
         const int t_end = std::min(max_iter, t + batch - 1);
         for (int tt = t; tt <= t_end; ++tt) {
             if (tt > t) {
                 KMP_CUDA(&c, keep_centers(), "keep centers");
-                KMP_CUDA(&c, kmp::launch_centroids(c, c.labels[cur], listed && tt > 1 ? c.labels[cur ^ 1] : nullptr,
+                KMP_CUDA(&c, kmp::launch_centroids(c, c.labels[cur], by_change && tt > 1 ? c.labels[cur ^ 1] : nullptr,
                                                    centers_dev),
                          "centroid kernels");
                 cur ^= 1;
@@ -659,7 +669,7 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
                          "cost sum");
             } else if (bounded && (tt > 0 || listed)) {
                 KMP_CUDA(&c, tt > 0 ? kmp::launch_lloyd_bounded_pass(c, centers_dev, c.labels[cur], c.labels[cur ^ 1],
-                                                                     changed, c.dmin)
+                                                                     changed, c.dmin, listed)
                                     : kmp::launch_lloyd_first_pass(c, centers_dev, c.labels[cur], changed, c.dmin),
                          "bounded assign pass");
                 KMP_CUDA(&c, kmp::launch_sum_rows(c.dmin, c.n, c.partials, c.sum_blocks, c.cost_dev, nullptr,
@@ -683,6 +693,13 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
         KMP_CUDA(&c, cudaMemcpyAsync(hrec.data() + t, rec + t, sizeof(Rec) * (size_t)(t_end - t + 1),
                                      cudaMemcpyDeviceToHost, c.stream),
                  "read records");
+        int pending = 0, open = 0;   // of the last assignment
+        if (listed && t_end > 0) {
+            KMP_CUDA(&c, cudaMemcpyAsync(&pending, kmp::lloyd_pending(c), sizeof(int), cudaMemcpyDeviceToHost, c.stream),
+                     "read pending rows");
+            KMP_CUDA(&c, cudaMemcpyAsync(&open, c.ll_cnt, sizeof(int), cudaMemcpyDeviceToHost, c.stream),
+                     "read open rows");
+        }
         KMP_CUDA(&c, cudaStreamSynchronize(c.stream), "sync");
         KMP_CUDA(&c, kmp::timing_drain(c), "timing");
         if (c.tc_err) {
@@ -695,11 +712,15 @@ kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter, i
         if (done < 0) {
             // the last iteration of the batch still needs its centroid update
             KMP_CUDA(&c, keep_centers(), "keep centers");
-            KMP_CUDA(&c, kmp::launch_centroids(c, c.labels[cur], listed && t_end > 0 ? c.labels[cur ^ 1] : nullptr,
+            KMP_CUDA(&c, kmp::launch_centroids(c, c.labels[cur], by_change && t_end > 0 ? c.labels[cur ^ 1] : nullptr,
                                                centers_dev),
                      "centroid kernels");
             cur ^= 1;
             t = t_end + 1;
+            if (listed && !kmp::lloyd_lists_paid(c, pending, open)) {
+                listed = false;
+                by_change = 2 * (int64_t)pending < c.n;   // else most clusters change
+            }
         }
     }
     t = done;

@@ -41,7 +41,10 @@ struct DevState {
     unsigned long long screen_listed;                  // undecided round rows refined from the pass's own lists
     unsigned long long recluster_snapshots;            // batched reclustering: D^2 snapshots taken
     int32_t part_begin, part_total, part_next;         // the round's batch while its parts are passed over
-    int32_t part_open;                                 // rows the filter left open in the last pass (-1: none yet)
+    int32_t part_open;                                 // rows the filter left open in its last pass (-1: none yet)
+    int32_t list_refs;                                 // references listed in this pass (0: none)
+    int32_t list_fail;                                 // references of the last list pass if it left most rows open
+    int32_t list_skip;                                 // this pass goes without lists, over all rows
     unsigned long long lloyd_settled;                  // Lloyd rows whose assignment the bounds settled
 };
 
@@ -154,6 +157,8 @@ struct Ctx {
     int32_t *rf_rows = nullptr;
     int *rf_cnt = nullptr;
     int round_part = 0;           // part of the round's batch that the pass covers
+    bool lists_known = false;     // the last round used lists, and
+    bool lists_failed = false;    // they left most rows open
     // exactly-l rounds (Sec. 5.3): 0 = independent draws, 1 = floor(l) per round
     int sampling = 0;
     uint32_t *ex_keys = nullptr;  // per point: FP32 clock bits
@@ -276,7 +281,7 @@ cudaError_t launch_weights(Ctx &c);
 // step 8 one draw at a time: the cluster form (recluster_cluster.cu) by a plan of
 // its own, cs = 0 when it does not apply, and the cooperative grid form
 struct ReclusterPlan {
-    int cs = 0, cpw = 0, qs4 = 0, slots = 0;
+    int cs = 0, cpw = 0, aw = 0, qs4 = 0, slots = 0;
 };
 ReclusterPlan recluster_plan(int m, int d, int max_cs);
 cudaError_t recluster_max_cluster(int dev, int *max_cs);
@@ -312,7 +317,11 @@ bool round_filter_sizes(const Ctx &c);
 // and one assignment after a centroid update that uses them
 bool lloyd_bounds_usable(const Ctx &c, const float *C);
 cudaError_t launch_lloyd_bounded_pass(Ctx &c, const float *C, int32_t *labels, const int32_t *prev, int *changed,
-                                      float *dmin);
+                                      float *dmin, bool lists);
+// after one with lists: the rows that were pending (c.ll_cnt: those the lists left open), and
+// whether the lists paid
+const int *lloyd_pending(const Ctx &c);
+bool lloyd_lists_paid(const Ctx &c, int pending, int open);
 // the first assignment of a context that can use the bounds, by the candidates' lists
 bool lloyd_lists_sizes(const Ctx &c);
 bool lloyd_lists_usable(const Ctx &c);

@@ -465,11 +465,18 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint8_t *__restr
                                                           uint8_t *__restrict__ cimg, float *__restrict__ cscale,
                                                           float *__restrict__ thr,
                                                           const unsigned int *__restrict__ rad2,
-                                                          const float *__restrict__ tau2) {
+                                                          const float *__restrict__ tau2, const int *all) {
     const int64_t nf = *cnt;
     const int per_row = KA * 8;
     const float W = fp32_tie_window(d);
     const float cmax = __uint_as_float(*cmax_bits);
+    if (all && *all) {
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nf; i += (int64_t)gridDim.x * blockDim.x) {
+            cscale[i] = xscale ? xscale[i] : 1.f;
+            thr[i] = list_threshold(ub[i], xnorm[i], cmax, ep, en, ec, W);
+        }
+        return;
+    }
     for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < nf * per_row;
          f += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = f / per_row;
@@ -689,9 +696,9 @@ void tc_bound(int d, int fmt, float *ep, float *en, float *ec) {
 cudaError_t launch_gather_rows(const uint8_t *img, const float *xscale, int d, int fmt, const int32_t *rows,
                                const int *cnt, const float *ub, const float *xnorm, const unsigned int *cmax_bits,
                                float ep, float en, float ec, uint8_t *cimg, float *cscale, float *thr, int grid,
-                               cudaStream_t s, const unsigned int *rad2, const float *tau2) {
+                               cudaStream_t s, const unsigned int *rad2, const float *tau2, const int *all) {
     gather_rows_kernel<<<grid, 256, 0, s>>>(img, fmt == FMT_FP8 ? xscale : nullptr, d, tc_katoms(d, fmt), rows, cnt,
-                                            ub, xnorm, cmax_bits, ep, en, ec, cimg, cscale, thr, rad2, tau2);
+                                            ub, xnorm, cmax_bits, ep, en, ec, cimg, cscale, thr, rad2, tau2, all);
     count_launches(1);
     return cudaGetLastError();
 }

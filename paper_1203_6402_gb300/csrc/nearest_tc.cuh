@@ -33,6 +33,8 @@ struct TcParams {
     int d;
     int fmt;
     const uint8_t *ximg;     // swizzled image of X (or of the listed rows), one block per 128-row tile
+    const uint8_t *ximg_all; // a compact pass: the image of all rows, used where *all_dev is set (all_dev null: never)
+    const int *all_dev;
     const float *xnorm;      // ||x'||^2 per point (FP32, x' = x - anchor)
     const float *xscale;     // FP8: per-row scale s_x of the A image
     const float *Cf;         // FP32 center rows (ROUND: candidate matrix; ASSIGN: k centers)
@@ -84,7 +86,9 @@ cudaError_t launch_nearest_tc(TcParams p, int mode_round, int epi, int num_sms, 
 cudaError_t launch_gather_rows(const uint8_t *img, const float *xscale, int d, int fmt, const int32_t *rows,
                                const int *cnt, const float *ub, const float *xnorm, const unsigned int *cmax_bits,
                                float ep, float en, float ec, uint8_t *cimg, float *cscale, float *thr, int grid,
-                               cudaStream_t s, const unsigned int *rad2 = nullptr, const float *tau2 = nullptr);
+                               cudaStream_t s, const unsigned int *rad2 = nullptr, const float *tau2 = nullptr,
+                               const int *all = nullptr);
+// (all: where it is set, the rows are all rows in order, and the image is not copied)
 // (rows null: row i.  rad2: instead of by ub, row i is a reference whose list holds every
 // center within 2 r + tau of it, r^2 given by its bits rad2[i], tau^2 = tau2[i] or 0)
 // Lists of the centers around references (points that rows are known to be near): a row

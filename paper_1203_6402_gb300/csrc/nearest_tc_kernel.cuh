@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(kThreads, 1) nearest_tc_kernel(TcParams p, int
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int begin = mode_round ? p.st->batch_begin : 0;
     const int cnt = mode_round ? p.st->batch_cnt : p.cnt;
+    const uint8_t *ximg = p.all_dev && *p.all_dev ? p.ximg_all : p.ximg;
     const int T = (cnt + BN - 1) / BN;
     const bool resident = T <= S;
     const int ksteps = p.ksteps;
@@ -322,15 +323,15 @@ __global__ void __launch_bounds__(kThreads, 1) nearest_tc_kernel(TcParams p, int
             // the A tiles of the next row tiles are pulled into L2 ahead of their copies
             for (int q = 1; q <= kPrefetch; ++q) {
                 const int64_t rq = blockIdx.x + (int64_t)q * gridDim.x;
-                if (rq < nrt) prefetch_l2(p.ximg + (size_t)rq * C::A16_BYTES, C::A16_BYTES);
+                if (rq < nrt) prefetch_l2(ximg + (size_t)rq * C::A16_BYTES, C::A16_BYTES);
             }
             for (int rt = blockIdx.x; rt < nrt; rt += gridDim.x, ++lt) {
                 const int ab = lt % A16B;
                 const int64_t rq = rt + (int64_t)(kPrefetch + 1) * gridDim.x;
-                if (rq < nrt) prefetch_l2(p.ximg + (size_t)rq * C::A16_BYTES, C::A16_BYTES);
+                if (rq < nrt) prefetch_l2(ximg + (size_t)rq * C::A16_BYTES, C::A16_BYTES);
                 if (lt >= A16B && !wait_bar(&sm.a_free[ab], ((lt - A16B) / A16B) & 1, abort, p.err, 11)) break;
                 mbar_expect_tx(&sm.a_full[ab], C::A16_BYTES);
-                bulk_g2s(a16 + ab * C::A16_BYTES, p.ximg + (size_t)rt * C::A16_BYTES, C::A16_BYTES, &sm.a_full[ab]);
+                bulk_g2s(a16 + ab * C::A16_BYTES, ximg + (size_t)rt * C::A16_BYTES, C::A16_BYTES, &sm.a_full[ab]);
                 if (!resident) {
                     bool ok = true;
                     for (int t = 0; t < T; ++t, ++bt) {

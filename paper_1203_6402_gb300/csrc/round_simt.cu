@@ -683,9 +683,18 @@ static bool round_filter_usable(const Ctx &c) {
 // The part of the round's batch that the next distance pass covers: part s of S equal
 // ones, or all that is left when the filter left most rows open in the pass before (the
 // data does not separate, and every part would go over all rows again) or hardly any
-// (nothing is left to save); s = S: the whole batch again.
-__global__ void round_part_kernel(DevState *st, int s, int S, const int *open_cnt, int64_t n) {
-    if (s > 0 && open_cnt && st->batch_cnt > 0) st->part_open = *open_cnt;   // of the pass before
+// (nothing is left to save); s = S: the whole batch again.  filter: the pass may use lists;
+// where they left most rows open, the next try waits until there are kListRetry times as many
+// references (a round's list pass over data that do not separate costs a fifth of it).
+constexpr int kListRetry = 6;
+
+__global__ void round_part_kernel(DevState *st, int s, int S, int filter, const int *open_cnt, int64_t n) {
+    if (st->list_refs > 0) {   // the outcome of the last list pass
+        const int64_t open = *open_cnt;
+        st->part_open = (int32_t)open;
+        st->list_fail = open * 4 > 3 * n ? st->list_refs : 0;
+        st->list_refs = 0;
+    }
     if (s == 0) {
         st->part_begin = st->batch_begin;
         st->part_total = st->batch_cnt;
@@ -698,11 +707,14 @@ __global__ void round_part_kernel(DevState *st, int s, int S, const int *open_cn
         return;
     }
     const int64_t open = st->part_open;
-    const bool rest = s == S - 1 || (open >= 0 && (open * 4 > 3 * n || open * 50 < n));
+    const bool skip = filter && st->list_fail > 0 && st->part_begin + from < kListRetry * (int64_t)st->list_fail;
+    const bool rest = skip || s == S - 1 || (open >= 0 && (open * 4 > 3 * n || open * 50 < n));
     const int to = rest ? total : max(from, (int)((int64_t)total * (s + 1) / S));
     st->batch_begin = st->part_begin + from;
     st->batch_cnt = to - from;
     st->part_next = to;
+    st->list_skip = skip && to > from;
+    st->list_refs = filter && !skip && to > from ? st->batch_begin : 0;
 }
 
 // Parts of a round's batch.  A part's candidates filter the parts after it, so the dense
@@ -719,11 +731,12 @@ cudaError_t launch_round_distance(Ctx &c, int round) {
     cudaError_t e;
     if (c.precision != KMPAR_FP32) {
         const int S = round_parts(c);
+        const bool planned = round_filter_usable(c);   // (S > 1 only then)
         for (int s = 0; s < S; ++s) {
             c.round_part = s;
-            if (S > 1) {
+            if (planned) {
                 // (the first pass of the first round has no filter)
-                round_part_kernel<<<1, 1, 0, c.stream>>>(c.st, s, S, s + c.rounds_done > 1 ? c.rf_cnt : nullptr, c.n);
+                round_part_kernel<<<1, 1, 0, c.stream>>>(c.st, s, S, s + c.rounds_done > 0, c.rf_cnt, c.n);
                 count_launches(1);
             }
             if ((e = launch_tc_pass(c, 1, c.C, 0, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr)) !=
@@ -732,7 +745,7 @@ cudaError_t launch_round_distance(Ctx &c, int round) {
         }
         c.round_part = 0;
         if (S > 1) {
-            round_part_kernel<<<1, 1, 0, c.stream>>>(c.st, S, S, c.rf_cnt, c.n);
+            round_part_kernel<<<1, 1, 0, c.stream>>>(c.st, S, S, 0, c.rf_cnt, c.n);
             count_launches(1);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
@@ -1838,9 +1851,11 @@ __global__ void __launch_bounds__(256) refine_list_kernel(
 
 // per candidate, the bits of the largest D^2 among its rows (a read first: most rows
 // are below the maximum already stored)
+// (refs: nothing to do where it is 0; null: always)
 __global__ void __launch_bounds__(256) candidate_radius_kernel(const float *__restrict__ D2,
                                                               const int32_t *__restrict__ idx, int64_t n,
-                                                              unsigned int *rad2) {
+                                                              unsigned int *rad2, const int32_t *refs) {
+    if (refs && *refs == 0) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const unsigned int v = __float_as_uint(D2[i]);
         unsigned int *r = rad2 + idx[i];
@@ -1960,6 +1975,12 @@ __global__ void __launch_bounds__(256) refine_group_kernel(GroupArgs g) {
     const int begin = MODE == MODE_ROUND ? g.st->batch_begin : 0;
     const bool any = MODE != MODE_ROUND || g.st->batch_cnt > 0;   // (an empty batch has no lists, changes nothing)
     const int64_t n = g.rows ? (int64_t)*g.rows_cnt : g.n, nb = (n + 31) / 32;
+    if (MODE == MODE_ROUND && g.st->list_skip) {   // no lists: all rows, in order, to the dense pass
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+            g.open_rows[i] = (int32_t)i;
+        if (blockIdx.x == 0 && threadIdx.x == 0) *g.open_cnt = (int)n;
+        return;
+    }
     unsigned int settled = 0, listed = 0, chg = 0;
     int64_t b = (int64_t)blockIdx.x * nwarps + wid;
     // this lane's row of block b: its number, reference, distance and list head
@@ -2147,14 +2168,14 @@ cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_
     if (plist && !rows && round_filter_usable(c)) {
         if ((e = cudaMemsetAsync(c.rf_rad2, 0, sizeof(unsigned int) * (size_t)old, c.stream)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(c.rf_cnt, 0, sizeof(int), c.stream)) != cudaSuccess) return e;
-        candidate_radius_kernel<<<c.num_sms * 8, 256, 0, c.stream>>>(c.D2, c.idx, c.n, c.rf_rad2);
+        candidate_radius_kernel<<<c.num_sms * 8, 256, 0, c.stream>>>(c.D2, c.idx, c.n, c.rf_rad2, &c.st->list_refs);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         tc::TcParams pf = p;
         pf.lst = c.tc_lst; pf.lcnt = c.tc_lcnt;
         const tc::ListBufs lb{c.cap_total, c.tc_cimg, c.tc_cscale, c.tc_thr, c.rf_rad2, c.rf_num, c.rf_lst, c.rf_head,
                               c.rf_lcnt};
-        if ((e = tc::launch_reference_lists(pf, 1, lb, c.cand, &c.st->batch_begin, nullptr, sb.ep, sb.en, sb.ec, c.num_sms,
+        if ((e = tc::launch_reference_lists(pf, 1, lb, c.cand, &c.st->list_refs, nullptr, sb.ep, sb.en, sb.ec, c.num_sms,
                                             c.stream)) != cudaSuccess)
             return e;
         GroupArgs ga{};
@@ -2177,12 +2198,15 @@ cudaError_t launch_tc_pass(Ctx &c, int mode_round, const float *C, int k, int32_
         if (!direct || p.group != 4 || !c.tc_cimg) return cudaErrorInvalidValue;
         if ((e = tc::launch_gather_rows(c.tc_ximg, c.tc_xscale, c.d, fmt, rows, rows_cnt,
                                         mode_round ? c.D2 : c.tc_ub, c.tc_xnorm, c.tc_cmax, sb.ep, sb.en, sb.ec,
-                                        c.tc_cimg, c.tc_cscale, c.tc_thr, c.num_sms * 8, c.stream)) != cudaSuccess)
+                                        c.tc_cimg, c.tc_cscale, c.tc_thr, c.num_sms * 8, c.stream, nullptr, nullptr,
+                                        mode_round ? &c.st->list_skip : nullptr)) != cudaSuccess)
             return e;
+        if (mode_round) { p.all_dev = &c.st->list_skip; p.ximg_all = p.ximg; }
         p.ximg = c.tc_cimg; p.xscale = c.tc_cscale; p.nrows_dev = rows_cnt;
         if ((e = tc::launch_nearest_tc(p, mode_round, plist ? tc::EPI_PAIRLIST : tc::EPI_PAIR, c.num_sms, c.stream)) !=
             cudaSuccess)
             return e;
+        p.all_dev = nullptr;   // (the passes over undecided rows gather theirs)
         const int grid = (int)((c.n + 255) / 256);
         if (mode_round)
             refine_direct_kernel<MODE_ROUND, 4><<<grid, 256, 0, c.stream>>>(
@@ -2382,7 +2406,9 @@ __global__ void __launch_bounds__(1024) lloyd_drift_other_kernel(const float *__
 // the exact FP32 d^2 to the moved center (the chain of the refine, rows and centers staged
 // by whole warps) and with it a tight upper bound for the test (lloyd_moved_kernel).
 // Settled rows get their label, distance and bounds; a pending one has l = 0 until a pass
-// certifies it again, and its distance goes into its center's radius for the lists.
+// certifies it again, and its distance goes into its center's radius for the lists.  Without
+// lists nothing wants the distance of a row that will be pending: rows of moved centers whose
+// old upper bound and its center's drift already fail the test are listed as pending at once.
 // 1e7 x 128, k = 10,000, 4% of the centers moving: 1.9 ms an assignment as one kernel with
 // a row a thread, 0.8 staged over all rows, 0.13 + 0.1 so.
 struct BoundsArgs {
@@ -2422,7 +2448,12 @@ __global__ void __launch_bounds__(256) lloyd_still_kernel(BoundsArgs g) {
             const int a = g.prev[R];
             mv = g.drift[a] != 0.f;
             g.labels[R] = a;
-            if (!mv) {
+            if (mv && !g.rad2) {
+                const float lo = g.lb[R] - g.other[a];
+                pd = !(lo > 0.f && g.ub[R] + g.drift[a] < lo);
+                if (pd) g.lb[R] = 0.f;
+                mv = !pd;
+            } else if (!mv) {
                 const float lo = g.lb[R] - g.other[a];
                 pd = !(lo > 0.f && g.ub[R] < lo);
                 g.lb[R] = pd ? 0.f : lo;
@@ -2522,7 +2553,16 @@ bool lloyd_lists_sizes(const Ctx &c) {
            resident_plan(c.k, c.d).parts == 0 && (int64_t)std::max(c.cap_total, c.k) <= c.n / 8 &&
            (double)c.n * c.k >= 1e9;
 }
-bool lloyd_lists_usable(const Ctx &c) { return lloyd_lists_sizes(c) && c.ll_pick; }
+bool lloyd_lists_usable(const Ctx &c) { return lloyd_lists_sizes(c) && c.ll_pick && !c.lists_failed; }
+const int *lloyd_pending(const Ctx &c) { return c.ll_lcnt + tc::kListLevels + 1; }
+
+// Whether an assignment by the lists paid.  Those that found their center in a list, pending
+// less open, were settled at the price of listing k centers around each other (some 2 k rows of
+// a dense pass, four times that where the lists overflow) and of 18 launches, some 120 us.
+bool lloyd_lists_paid(const Ctx &c, int pending, int open) {
+    const double levels = 1.0 + 3.0 * open / std::max(1, pending);
+    return (double)pending - open > 2.0 * c.k * levels + 8e9 / ((double)c.k * c.d);
+}
 
 __global__ void set_int_kernel(int *p, int v) { *p = v; }
 
@@ -2580,7 +2620,7 @@ cudaError_t launch_lloyd_first_pass(Ctx &c, const float *C, int32_t *labels, int
     const tc::ListBufs lb = lloyd_list_bufs(c);
     if ((e = cudaMemsetAsync(c.ll_rad2, 0, sizeof(unsigned int) * (size_t)lb.cap, c.stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(c.ll_cnt, 0, sizeof(int), c.stream)) != cudaSuccess) return e;
-    candidate_radius_kernel<<<c.num_sms * 8, 256, 0, c.stream>>>(c.D2, c.idx, c.n, c.ll_rad2);
+    candidate_radius_kernel<<<c.num_sms * 8, 256, 0, c.stream>>>(c.D2, c.idx, c.n, c.ll_rad2, nullptr);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // tau: the candidates' best screened groups
@@ -2612,10 +2652,9 @@ cudaError_t launch_lloyd_first_pass(Ctx &c, const float *C, int32_t *labels, int
 // (an open row of a mixture has one or two), and a dense compact pass over the rows
 // beyond the lists.
 cudaError_t launch_lloyd_bounded_pass(Ctx &c, const float *C, int32_t *labels, const int32_t *prev, int *changed,
-                                      float *dmin) {
+                                      float *dmin, bool lists) {
     cudaError_t e;
     const int k = c.k;
-    const bool lists = lloyd_lists_usable(c);
     lloyd_drift_kernel<<<(k + 7) / 8, 256, 0, c.stream>>>(C, c.ll_cold, k, c.d, c.ll_drift);
     lloyd_drift_other_kernel<<<1, 1024, 0, c.stream>>>(c.ll_drift, k, c.ll_other);
     count_launches(2);
