@@ -22,8 +22,8 @@
 // masses, 1,600 totals there, 600 the owner, 400 the candidate and row out, 1,550 row
 // there, 1,600 D^2); 5.9 us with cluster barriers and FP64 scans.
 //
-// Draw t (exchange x): warp gw = 16 rank + wid owns the 32 cpw consecutive
-// candidates from 32 cpw gw, lane l the cpw from there + l cpw, so the order of the
+// Draw t (exchange x): warp gw = aw rank + wid (wid < aw, 16 where there are candidates for as
+// many warps) owns the 32 cpw consecutive candidates from 32 cpw gw, lane l the cpw from there + l cpw, so the order of the
 // prefix is lane by lane.  Warp 0 of every CTA scans its CTA's 16 warp totals, sends
 // their sum to every CTA, waits for all CS sums and finds the CTA whose prefix passes
 // the target u_t * total (exact integers: u_t is a multiple of 2^-53); the owner's
@@ -196,6 +196,7 @@ struct RdArgs {
     int m, d, k;
     uint64_t seed;
     int cs, cpw;             // CTAs, candidates per lane
+    int aw;                  // warps of a CTA that hold candidates
     int qs4;                 // coordinate groups kept in shared memory
     int32_t *chosen;
     float *centers;
@@ -231,8 +232,8 @@ __device__ __forceinline__ void rd_acc(float &s, float4 x, float4 c) {
     t = __fsub_rn(x.w, c.w); s = __fmaf_rn(t, t, s);
 }
 
-__host__ __device__ __forceinline__ size_t rd_smem_bytes(int d4, int cpw, int qs4) {
-    const size_t nc = (size_t)cpw * kRdThreads;
+__host__ __device__ __forceinline__ size_t rd_smem_bytes(int d4, int cpw, int aw, int qs4) {
+    const size_t nc = (size_t)cpw * 32 * aw;
     return 16 * (size_t)(2 * kRdMaxCl + 2 * kRdWarps + 2 * (d4 + 1)) + 16 * nc * qs4 + 8 * nc;
 }
 
@@ -294,7 +295,7 @@ template <int SRC>
 __global__ void __launch_bounds__(kRdThreads, 1) recluster_draws_kernel(RdArgs a) {
     extern __shared__ __align__(16) unsigned char rd_sm[];
     __shared__ uint64_t bar_tot[2], bar_row[2], bar_loc;
-    const int d = a.d, d4 = (d + 3) >> 2, cpw = a.cpw, NC = cpw * kRdThreads, m = a.m, CS = a.cs;
+    const int d = a.d, d4 = (d + 3) >> 2, cpw = a.cpw, NC = cpw * 32 * a.aw, m = a.m, CS = a.cs;
     uint4 *tot = reinterpret_cast<uint4 *>(rd_sm);               // [2][CS]
     uint4 *wtot = tot + 2 * kRdMaxCl;                             // [2][16 warps]
     uint4 *row = wtot + 2 * kRdWarps;                             // [2][header, d4 groups]
@@ -302,6 +303,7 @@ __global__ void __launch_bounds__(kRdThreads, 1) recluster_draws_kernel(RdArgs a
     float *dl = reinterpret_cast<float *>(rows + (size_t)a.qs4 * NC);
     uint32_t *wl = reinterpret_cast<uint32_t *>(dl + NC);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int mine = wid < a.aw ? cpw : 0;   // candidates of a lane of this warp
     uint32_t rank_u;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank_u));
     const int rank = (int)rank_u;
@@ -350,7 +352,7 @@ __global__ void __launch_bounds__(kRdThreads, 1) recluster_draws_kernel(RdArgs a
         if (dirty) {
             U96 s = {0u, 0u, 0u};
             uint32_t E = 0;
-            for (int i = 0; i < cpw; ++i) {
+            for (int i = 0; i < mine; ++i) {
                 const int ls = (wid * cpw + i) * 32 + lane;
                 uint32_t Ei;
                 s = s + rd_mass(wl[ls], t == 0 ? 1.f : dl[ls], eb, Ei);
@@ -489,7 +491,7 @@ __global__ void __launch_bounds__(kRdThreads, 1) recluster_draws_kernel(RdArgs a
         // ---- D^2 against the new center.  Partial sums of non-negative terms never
         // decrease: once every lane's has reached its D^2 the rest is skipped
         bool fell = false;
-        for (int i = 0; i < cpw; ++i)
+        for (int i = 0; i < mine; ++i)
             fell |= rd_update<SRC>(a, rows, dl, wl, cn, (wid * cpw + i) * 32 + lane, s0, NC, d4, first);
         dirty = __any_sync(0xffffffffu, fell) || dirty;
         if (first) {
@@ -526,25 +528,33 @@ __global__ void __launch_bounds__(256) transpose4_kernel(const float *__restrict
 }  // namespace
 
 // How the draws kernel covers m candidates of d coordinates: the fewest CTAs with one
-// candidate per lane, max_cs beyond max_cs x 512 candidates, and as many leading groups
-// of coordinates in shared memory as fit.  The cooperative grid form takes over (cs = 0)
-// when a draw would read more than 512 KB a CTA from L2: measured, us a draw, this
-// form / the grid: 4,933 x 42 2.9 / 8.6, 9,925 x 42 3.8 / 8.7 (nothing from L2);
-// 9,876 x 128 (320 KB) 7.7 / 9.3, 19,960 x 96 (384 KB) 8.2 / 9.5, 39,809 x 128
-// (1.1 MB) 15.9 / 10.3.
+// candidate per lane, max_cs beyond max_cs x 512 candidates, more where that brings all
+// coordinates into shared memory, and else as many leading groups of coordinates there as
+// fit.  The cooperative grid form takes over (cs = 0) when a draw would read more than
+// 512 KB a CTA from L2: measured, us a draw, this form / the grid: 4,933 x 42 2.9 / 8.6,
+// 9,925 x 42 3.8 / 8.7 (nothing from L2); 9,876 x 128 (320 KB) 7.7 / 9.3, 19,960 x 96 (384 KB)
+// 8.2 / 9.5, 39,809 x 128 (1.1 MB) 15.9 / 10.3.
 ReclusterPlan recluster_plan(int m, int d, int max_cs) {
-    ReclusterPlan p{};
     const int d4 = (d + 3) >> 2;
-    p.cs = 1;
-    while (p.cs < max_cs && m > p.cs * kRdThreads) p.cs *= 2;
-    p.cpw = std::max(1, (m + p.cs * kRdThreads - 1) / (p.cs * kRdThreads));
-    const size_t budget = kRdSmemBudget, base = rd_smem_bytes(d4, p.cpw, 0);
-    if (base > budget) return ReclusterPlan{};
-    const int fit = (int)((budget - base) / (16 * (size_t)p.cpw * kRdThreads));
-    p.qs4 = fit >= d4 ? d4 : fit & ~3;
-    if ((size_t)(d4 - p.qs4) * p.cpw * kRdThreads * 16 > 512u * 1024u) return ReclusterPlan{};
-    p.slots = p.cs * p.cpw * kRdThreads;
-    return p;
+    const size_t budget = kRdSmemBudget;
+    int cs = 1;
+    while (cs < max_cs && m > cs * kRdThreads) cs *= 2;
+    ReclusterPlan first{};
+    for (int c = cs; c <= max_cs; c *= 2) {
+        ReclusterPlan p{};
+        p.cs = c;
+        p.cpw = std::max(1, (m + c * kRdThreads - 1) / (c * kRdThreads));
+        p.aw = std::min(kRdWarps, (m + c * 32 * p.cpw - 1) / (c * 32 * p.cpw));
+        p.slots = c * p.cpw * 32 * p.aw;
+        const size_t base = rd_smem_bytes(d4, p.cpw, p.aw, 0);
+        if (base > budget) return ReclusterPlan{};
+        const int fit = (int)((budget - base) / (16 * (size_t)p.cpw * 32 * p.aw));
+        p.qs4 = fit >= d4 ? d4 : fit & ~3;
+        if (p.qs4 == d4) return p;
+        if (c == cs) first = p;
+    }
+    if ((size_t)(d4 - first.qs4) * first.cpw * 32 * first.aw * 16 > 512u * 1024u) return ReclusterPlan{};
+    return first;
 }
 
 static const void *rd_kernels[3] = {(const void *)recluster_draws_kernel<RD_SMEM>,
@@ -597,12 +607,12 @@ cudaError_t launch_recluster_draws(Ctx &c, float *centers, const ReclusterPlan &
     }
     RdArgs a{};
     a.C = c.C; a.CT4 = ct; a.w = c.w; a.st = c.st; a.m = c.m_host; a.d = c.d; a.k = c.k; a.seed = c.seed;
-    a.cs = p.cs; a.cpw = p.cpw; a.qs4 = p.qs4; a.chosen = c.chosen; a.centers = centers; a.err = c.rc_err;
+    a.cs = p.cs; a.cpw = p.cpw; a.aw = p.aw; a.qs4 = p.qs4; a.chosen = c.chosen; a.centers = centers; a.err = c.rc_err;
     a.wait = kRdWait;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)p.cs);
     cfg.blockDim = dim3(kRdThreads);
-    cfg.dynamicSmemBytes = rd_smem_bytes(d4, p.cpw, p.qs4);
+    cfg.dynamicSmemBytes = rd_smem_bytes(d4, p.cpw, p.aw, p.qs4);
     cfg.stream = c.stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
