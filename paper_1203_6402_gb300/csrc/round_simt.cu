@@ -130,15 +130,16 @@ __device__ __forceinline__ void top2_merge(float &b1, int &i1, float &b2, int &i
     }
 }
 
-// The scan for d <= 32: a row a thread, its coordinates in registers, 64 centers at a
+// The scan for d <= 32, and for few centers up to d = 128: a row a thread, its coordinates in registers, 64 centers at a
 // time in shared memory.  With so few coordinates the tiled scan's handling of its tile's
 // results outweighs the sums (3e6 x 3 against 100: 0.36 ms, tiled 0.8; 1e6 x 32 against
-// 100: 0.59, 0.68; at 50 coordinates 200,000 rows against 300 take 0.62, tiled 0.52).
+// 100: 0.59, 0.68; at 50 coordinates 200,000 rows against 300 take 0.62, tiled 0.52), as
+// does a tile's padding to 32 or 64 centers where there are few (see few_centers).
 constexpr int kNearThreads = 128;
 
 template <int DP, int MODE>
 __global__ void __launch_bounds__(kNearThreads) nearest_kernel(NearestParams p) {
-    constexpr int TC = 64;
+    constexpr int TC = DP <= 64 ? 64 : 32;
     __shared__ __align__(16) float tile[TC * DP];
     __shared__ double red[32];
     __shared__ int redi[32];
@@ -441,6 +442,14 @@ static cudaError_t launch_tiles(const NearestParams &p, int grid, cudaStream_t s
     return cudaGetLastError();
 }
 
+// Few centers against many rows (more than the 40,000 cut into small blocks), by the number of
+// centers (an assignment's) or the capacity for them (a round's; that of l = 12 is 110).
+// 2e6 x 33 against 1 center: 0.30 ms a row a thread, 0.41 tiled; x 97 0.52, 0.78;
+// against 30: 1.0 and 0.7.
+static bool few_centers(int mode, int64_t n, int d, int cnt_hint) {
+    return d <= 128 && scan_rows(n, d) == 128 && cnt_hint <= (mode == MODE_ASSIGN ? 8 : 110);
+}
+
 template <int MODE>
 static cudaError_t launch_nearest_mode(const NearestParams &p, int cnt_hint, cudaStream_t s) {
     const int grid = assign_num_partials(p.n, p.d);   // p.n = rows capacity for row lists
@@ -450,7 +459,12 @@ static cudaError_t launch_nearest_mode(const NearestParams &p, int cnt_hint, cud
     else if (p.d <= 8) nearest_kernel<8, MODE><<<grid, kNearThreads, 0, s>>>(p);
     else if (p.d <= 16) nearest_kernel<16, MODE><<<grid, kNearThreads, 0, s>>>(p);
     else if (p.d <= 32) nearest_kernel<32, MODE><<<grid, kNearThreads, 0, s>>>(p);
-    else if (small) return narrow ? launch_tiles<MODE, 32, 4>(p, grid, s) : launch_tiles<MODE, 32, 8>(p, grid, s);
+    else if (few_centers(MODE, p.n, p.d, cnt_hint)) {
+        if (p.d <= 48) nearest_kernel<48, MODE><<<grid, kNearThreads, 0, s>>>(p);
+        else if (p.d <= 64) nearest_kernel<64, MODE><<<grid, kNearThreads, 0, s>>>(p);
+        else if (p.d <= 96) nearest_kernel<96, MODE><<<grid, kNearThreads, 0, s>>>(p);
+        else nearest_kernel<128, MODE><<<grid, kNearThreads, 0, s>>>(p);
+    } else if (small) return narrow ? launch_tiles<MODE, 32, 4>(p, grid, s) : launch_tiles<MODE, 32, 8>(p, grid, s);
     else return narrow ? launch_tiles<MODE, 128, 4>(p, grid, s) : launch_tiles<MODE, 128, 8>(p, grid, s);
     return cudaGetLastError();
 }
