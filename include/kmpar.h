@@ -203,7 +203,8 @@ KMPAR_API kmpar_status kmpar_weighted_lloyd(kmpar_ctx *ctx, float *centers_dev, 
  * multiple of 4, the assignments after the first skip the rows whose distance
  * bounds prove their center unchanged (counted in kmpar_stats.lloyd_settled);
  * every label, distance and center is the one the full assignment gives.
- * Synchronises once per batch of iterations (4, then 8).
+ * Synchronises once per batch of iterations (4, then 8; 2 at first where it is not known yet
+ * whether lists of nearby centers hold).
  */
 KMPAR_API kmpar_status kmpar_lloyd(kmpar_ctx *ctx, float *centers_dev, int32_t max_iter,
                          int32_t *labels_dev, int32_t *iters, double *final_cost,
@@ -279,7 +280,7 @@ KMPAR_API kmpar_status kmpar_fit(const float *X, int64_t n, int32_t d, int32_t k
  * with status KMPAR_ERR_CAPACITY, the others are unaffected.  Work space comes
  * from the library's pool (beyond 256 MB from the device's); a problem runs in
  * one thread block, or in a thread-block cluster of 2, 4 or 8 blocks when it has more than 25,000 rows,
- * or fewer where the call's blocks would not fill the SMs
+ * or fewer where the call's blocks would not fill the SMs and its rows have work enough
  * (each block a contiguous range of rows; the cluster combines its sums and its
  * ordered draws in rank order; see kmpar_batch_set_split), largest problems
  * first, one kernel launch per (dimension class, cluster size).  Synchronises.
