@@ -45,9 +45,6 @@ struct NearestParams {
     int *changed;          // ASSIGN: +number of labels != prev (nullable)
     double *partials;      // per-block FP64 sum of the stored distances (nullable)
     unsigned long long *fp64_cnt, *wide_cnt;
-    const int32_t *rows;   // nullable: process only these rows (the tensor pass's fix-up list)
-    const int *rows_cnt;   // number of entries in rows
-    float *dmin;           // ASSIGN: per-row exact d^2 of the chosen center (nullable)
 };
 
 // lexicographic (value, index) improvement
@@ -80,7 +77,6 @@ __device__ __forceinline__ float nearest_decide(const NearestParams &p, int64_t 
             atomicAdd(p.fp64_cnt, 1ull);
         }
         if (p.labels) p.labels[pt] = lab;
-        if (p.dmin) p.dmin[pt] = stored;
         if (p.prev) chg = (p.prev[pt] != lab);
     } else {
         const float old = p.D2[pt];
@@ -145,14 +141,8 @@ __global__ void __launch_bounds__(kNearThreads) nearest_kernel(NearestParams p) 
     __shared__ int redi[32];
 
     const int tid = threadIdx.x;
-    int64_t pt = (int64_t)blockIdx.x * kNearThreads + tid;
-    bool valid = pt < p.n;
-    if (p.rows) {
-        const int nrows = *p.rows_cnt;
-        if ((int64_t)blockIdx.x * kNearThreads >= nrows) return;   // uniform per block
-        valid = pt < nrows;
-        pt = valid ? p.rows[pt] : 0;
-    }
+    const int64_t pt = (int64_t)blockIdx.x * kNearThreads + tid;
+    const bool valid = pt < p.n;
     const int d = p.d;
     const float *xrow = p.X + (valid ? pt : 0) * (int64_t)d;
 
@@ -239,39 +229,27 @@ __device__ __forceinline__ void cp_async4_zfill(uint32_t dst, const float *src, 
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
 }
 
-// coordinates q0 .. q0 + kn - 1 of rows first .. first + B - 1 (rows given: of the rows
-// rows[first + r]; rows at or past `limit` as zeros) to dst[q * stride + r], consecutive
-// threads along a row and then the next
+// coordinates q0 .. q0 + kn - 1 of rows first .. first + B - 1 (rows at or past `limit` as
+// zeros) to dst[q * stride + r], consecutive threads along a row and then the next
 template <int THREADS>
 __device__ __forceinline__ void tile_copy(float *dst, int stride, int B, const float *src, int64_t first, int64_t limit,
-                                          const int32_t *rows, int d, int q0, int kn) {
+                                          int d, int q0, int kn) {
     int r = threadIdx.x / kn, q = threadIdx.x % kn;
     const int dr = THREADS / kn, dq = THREADS % kn;
     uint32_t to = static_cast<uint32_t>(__cvta_generic_to_shared(dst + q * stride + r));
     const uint32_t step = 4u * (dq * stride + dr), wrap = 4u * (kn * stride - 1);
-    if (!rows) {
-        const float *from = src + (first + r) * d + q0 + q;
-        const int64_t fs = (int64_t)dr * d + dq, fw = d - kn;
-        const int lim = (int)min((int64_t)B, limit - first);
+    const float *from = src + (first + r) * d + q0 + q;
+    const int64_t fs = (int64_t)dr * d + dq, fw = d - kn;
+    const int lim = (int)min((int64_t)B, limit - first);
 #pragma unroll 4
-        while (r < B) {
-            const bool ok = r < lim;
-            cp_async4_zfill(to, ok ? from : src, ok);
-            r += dr;
-            q += dq;
-            from += fs;
-            to += step;
-            if (q >= kn) { q -= kn; ++r; from += fw; to -= wrap; }
-        }
-    } else {
-        while (r < B) {
-            const bool ok = first + r < limit;
-            cp_async4_zfill(to, ok ? src + (int64_t)rows[first + r] * d + q0 + q : src, ok);
-            r += dr;
-            q += dq;
-            to += step;
-            if (q >= kn) { q -= kn; ++r; to -= wrap; }
-        }
+    while (r < B) {
+        const bool ok = r < lim;
+        cp_async4_zfill(to, ok ? from : src, ok);
+        r += dr;
+        q += dq;
+        from += fs;
+        to += step;
+        if (q >= kn) { q -= kn; ++r; from += fw; to -= wrap; }
     }
 }
 
@@ -290,8 +268,6 @@ __global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 8) nearest_tile_kernel
     const bool resident = d <= kc;
     float *xb = tsm, *cb = tsm + (resident ? 1 : 2) * kc * XS;   // rows (two buffers in steps), centers (two)
     const int64_t base = (int64_t)blockIdx.x * BM;
-    const int64_t nrows = p.rows ? (int64_t)*p.rows_cnt : p.n;
-    if (p.rows && base >= nrows) return;   // uniform per block
     int begin, cnt;
     if constexpr (MODE == MODE_ASSIGN) {
         begin = p.c_begin; cnt = p.c_cnt;
@@ -302,9 +278,8 @@ __global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 8) nearest_tile_kernel
     auto issue = [&](int s) {   // step s: tile s / chunks of the centers, chunk s % chunks of the coordinates
         const int t = s / chunks, q0 = (s - t * chunks) * kc, kn = min(kc, d - q0);
         if (!resident || s == 0)
-            tile_copy<threads>(xb + (resident ? 0 : (s & 1) * kc * XS), XS, BM, p.X, base, nrows, p.rows, d, q0, kn);
-        tile_copy<threads>(cb + (s & 1) * kc * CS, CS, BN, p.C, begin + (int64_t)t * BN, begin + (int64_t)cnt, nullptr, d,
-                           q0, kn);
+            tile_copy<threads>(xb + (resident ? 0 : (s & 1) * kc * XS), XS, BM, p.X, base, p.n, d, q0, kn);
+        tile_copy<threads>(cb + (s & 1) * kc * CS, CS, BN, p.C, begin + (int64_t)t * BN, begin + (int64_t)cnt, d, q0, kn);
     };
     float b1[TM], b2[TM];
     int i1[TM], i2[TM];
@@ -376,7 +351,7 @@ __global__ void __launch_bounds__(2 * BM, BM == 128 ? 2 : 8) nearest_tile_kernel
     }
     auto number = [&](int r) -> int64_t {
         const int64_t at = base + r;
-        return at < nrows ? (p.rows ? (int64_t)p.rows[at] : at) : -1;
+        return at < p.n ? at : -1;
     };
     // merge the 8 threads of a row, then thread tx = r decides the thread row's row r
     float m1 = FLT_MAX, m2 = FLT_MAX;
@@ -452,7 +427,7 @@ static bool few_centers(int mode, int64_t n, int d, int cnt_hint) {
 
 template <int MODE>
 static cudaError_t launch_nearest_mode(const NearestParams &p, int cnt_hint, cudaStream_t s) {
-    const int grid = assign_num_partials(p.n, p.d);   // p.n = rows capacity for row lists
+    const int grid = assign_num_partials(p.n, p.d);
     const bool small = scan_rows(p.n, p.d) == 32, narrow = cnt_hint <= 32;
     count_launches(1);
     if (p.d <= 4) nearest_kernel<4, MODE><<<grid, kNearThreads, 0, s>>>(p);
@@ -489,7 +464,7 @@ __global__ void __launch_bounds__(kFirstRows) first_dist_kernel(const float *__r
     for (int q0 = 0; q0 < d; q0 += kFirstPiece) {
         const int kn = min(kFirstPiece, d - q0);
         __syncthreads();   // the walkers of the last piece are done
-        tile_copy<kFirstRows>(fsm, kFirstStride, kFirstRows, X, base, n, nullptr, d, q0, kn);
+        tile_copy<kFirstRows>(fsm, kFirstStride, kFirstRows, X, base, n, d, q0, kn);
         cp_async_commit();
         if (tid < kn) cq[tid] = C[q0 + tid];
         cp_async_wait<0>();
